@@ -147,11 +147,10 @@ int attn_decode(attn_ctx* ctx, const uint16_t* q, const uint16_t* k, const uint1
  * range; the groups of one range read the same cache tiles at about the same time, so the
  * repeats come from L2 while the history fits there.  A sequence whose hist_len[b] + n_new
  * exceeds max_len is skipped and flagged as in attn_decode.
- * head_dim 64: 1 <= n_new <= max_len; the tokens run as n_new attn_decode steps in order
- * (token t at hist_len[b] + t, the same result), each step's rows copied in and out of the
- * context's buffers, so the history is streamed n_new times; a token whose position passes
- * max_len - 1 is flagged and skipped as one attn_decode step would (the tokens before it in
- * that sequence are computed).  n_new = 1 is attn_decode.
+ * head_dim 64: 1 <= n_new <= max_len; up to 16 tokens run in one pass over the history
+ * (more take a pass per 16, in order); a token whose position is outside [0, max_len - 1] is
+ * flagged and skipped as one attn_decode step would (the other tokens of that sequence are
+ * computed).  n_new = 1 is attn_decode.
  */
 int attn_decode_multi(attn_ctx* ctx, const uint16_t* q, const uint16_t* k, const uint16_t* v,
                       const int32_t* d_hist_len, int n_new, uint16_t* k_cache, uint16_t* v_cache, uint16_t* out,

@@ -5,8 +5,9 @@
 // the kernels of each stage on the caller's stream:
 //   prefill / prefill_kv : K1 rope_append (new k rotated + k, v appended in place)
 //                          -> K2 flash_fwd (q rotated in-kernel, causal attention)
-//   decode               : K3 decode_split (new k rotated + k, v appended at slot
-//                          hist_len[b], read on the device) -> K4 decode_combine
+//   decode               : K3 (new k rotated + k, v appended at slot hist_len[b], read on
+//                          the device): decode_tc for head_dim 128, decode_split -> K4
+//                          decode_combine for head_dim 64
 // No call allocates, frees or synchronises except attn_create/attn_destroy and
 // attn_device_error.
 #include <cuda.h>
@@ -328,9 +329,10 @@ namespace {
 // producer_early: the previous launch wrote q, k and v and nothing the decode streams (the
 // fused QKV GEMV of attn_decode_layer); the head_dim 128 decode then starts its K/V stream as
 // a dependent launch before that kernel has finished.
+// seq_tok (head_dim 64): q, k, v and out point into arrays of seq_tok tokens per sequence (0: ntok).
 int run_decode(attn_ctx* c, const uint16_t* q, const uint16_t* k, const uint16_t* v, const int32_t* d_hist_len,
                int hist_add, bool after_decode, uint16_t* k_cache, uint16_t* v_cache, uint16_t* out, cudaStream_t st,
-               int ntok = 1, bool producer_early = false) {
+               int ntok = 1, bool producer_early = false, int seq_tok = 0) {
     if (c == nullptr || q == nullptr || k == nullptr || v == nullptr || d_hist_len == nullptr ||
         k_cache == nullptr || v_cache == nullptr || out == nullptr)
         return ATTN_EINVAL;
@@ -349,28 +351,32 @@ int run_decode(attn_ctx* c, const uint16_t* q, const uint16_t* k, const uint16_t
         c->dec_k = k_cache;
         c->dec_v = v_cache;
     }
-    if (ntok < 1 || ntok > kMaxDraftTokens || (ntok > 1 && !tc)) return ATTN_EINVAL;
+    if (ntok < 1 || ntok > kMaxDraftTokens) return ATTN_EINVAL;
     // the partials hold batch * Hq * nsplit_max rows: ntok tokens share them
     const int ncg = attn::decode_tc_column_groups(c->cfg.n_q_heads / c->cfg.n_kv_heads, ntok);
     // grid y and z (kv heads; sequences x column groups, or kv heads x head passes) stay
     // within the 65535 limit of those grid dimensions
     const int G = c->cfg.n_q_heads / c->cfg.n_kv_heads;
-    if (tc ? static_cast<long>(c->cfg.batch) * ncg > 65535 : static_cast<long>(c->cfg.n_kv_heads) * ((G + 7) / 8) > 65535)
+    if (tc ? static_cast<long>(c->cfg.batch) * ncg > 65535
+           : static_cast<long>(c->cfg.n_kv_heads) * attn::decode_passes(c->shape, ntok) > 65535)
         return ATTN_EINVAL;
+    if (seq_tok == 0) seq_tok = ntok;
     const int nsplit = tc ? std::min(attn::decode_tc_num_splits(c->shape, c->num_sms, ncg, ntok), c->nsplit_max / ntok)
-                          : attn::decode_num_splits(c->shape, c->num_sms, c->nsplit_max);
+                          : attn::decode_num_splits(c->shape, c->num_sms, c->nsplit_max / ntok, ntok);
     cudaError_t e = timed(c, ATTN_KERNEL_DECODE_SPLIT, st, [&](int*) {
         if (tc)
             return attn::launch_decode_tc(c->shape, c->dec_maps, q, k, v, d_hist_len, hist_add, k_cache, v_cache, c->d_cos,
                                           c->d_sin, c->d_part_o, c->d_part_ml, c->d_counters, nsplit, out,
                                           c->d_err, after_decode, ntok, st, producer_early, c->wait_ns, c->num_sms);
-        return attn::launch_decode_split(c->shape, c->dec_maps, q, k, v, d_hist_len, hist_add, k_cache, v_cache, c->d_cos,
-                                         c->d_sin, c->d_part_o, c->d_part_ml, nsplit, c->d_err, st, c->wait_ns);
+        return attn::launch_decode_split(c->shape, c->dec_maps, q, k, v, d_hist_len, hist_add, ntok, seq_tok, k_cache,
+                                         v_cache, c->d_cos, c->d_sin, c->d_part_o, c->d_part_ml, nsplit, c->d_err, st,
+                                         c->wait_ns);
     });
     if (e != cudaSuccess) return cuda_fail(e, "decode_split launch");
     if (tc) return ATTN_OK;  // the tensor-core decode merges its splits itself
     e = timed(c, ATTN_KERNEL_DECODE_COMBINE, st, [&](int*) {
-        return attn::launch_decode_combine(c->shape, d_hist_len, hist_add, c->d_part_o, c->d_part_ml, nsplit, out, st);
+        return attn::launch_decode_combine(c->shape, d_hist_len, hist_add, ntok, seq_tok, c->d_part_o, c->d_part_ml,
+                                           nsplit, out, st);
     });
     if (e != cudaSuccess) return cuda_fail(e, "decode_combine launch");
     return ATTN_OK;
@@ -391,28 +397,19 @@ int attn_decode_multi(attn_ctx* c, const uint16_t* q, const uint16_t* k, const u
     const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (c == nullptr || c->cfg.head_dim == 128 || n_new == 1)
         return run_decode(c, q, k, v, d_hist_len, 0, false, k_cache, v_cache, out, st, n_new);
-    // head_dim 64: the n_new tokens as n_new decode steps in order (token t at hist_len[b] + t
-    // sees the tokens before it in the cache, which is the same computation); each step's
-    // rows are gathered into the context's decode-block buffers and its output scattered back.
+    // head_dim 64: up to 16 tokens per launch, read and written where they lie (n_new may be as
+    // large as max_len); launch t0 continues at positions hist_len[b] + t0.  Fewer per launch
+    // only where the column passes of more would leave the grid's limits.
     if (q == nullptr || k == nullptr || v == nullptr || out == nullptr || n_new < 1 || n_new > c->cfg.max_len)
         return ATTN_EINVAL;
-    const size_t D = static_cast<size_t>(c->cfg.head_dim), B = static_cast<size_t>(c->cfg.batch);
-    const size_t qrow = c->cfg.n_q_heads * D * 2, krow = c->cfg.n_kv_heads * D * 2;  // bytes of one token's rows
-    for (int t = 0; t < n_new; ++t) {
-        cudaError_t e = cudaMemcpy2DAsync(c->d_lq, qrow, reinterpret_cast<const uint8_t*>(q) + t * qrow, n_new * qrow,
-                                          qrow, B, cudaMemcpyDeviceToDevice, st);
-        if (e == cudaSuccess)
-            e = cudaMemcpy2DAsync(c->d_lk, krow, reinterpret_cast<const uint8_t*>(k) + t * krow, n_new * krow, krow, B,
-                                  cudaMemcpyDeviceToDevice, st);
-        if (e == cudaSuccess)
-            e = cudaMemcpy2DAsync(c->d_lv, krow, reinterpret_cast<const uint8_t*>(v) + t * krow, n_new * krow, krow, B,
-                                  cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return cuda_fail(e, "decode_multi gather");
-        const int rc = run_decode(c, c->d_lq, c->d_lk, c->d_lv, d_hist_len, t, false, k_cache, v_cache, c->d_lo, st);
+    int per = std::min(n_new, kMaxDraftTokens);
+    while (per > 1 && static_cast<long>(c->cfg.n_kv_heads) * attn::decode_passes(c->shape, per) > 65535) --per;
+    const size_t qtok = static_cast<size_t>(c->cfg.n_q_heads) * c->cfg.head_dim;  // elements of one token's rows
+    const size_t ktok = static_cast<size_t>(c->cfg.n_kv_heads) * c->cfg.head_dim;
+    for (int t0 = 0; t0 < n_new; t0 += per) {
+        const int rc = run_decode(c, q + t0 * qtok, k + t0 * ktok, v + t0 * ktok, d_hist_len, t0, false, k_cache,
+                                  v_cache, out + t0 * qtok, st, std::min(per, n_new - t0), false, n_new);
         if (rc != ATTN_OK) return rc;
-        e = cudaMemcpy2DAsync(reinterpret_cast<uint8_t*>(out) + t * qrow, n_new * qrow, c->d_lo, qrow, qrow, B,
-                              cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return cuda_fail(e, "decode_multi scatter");
     }
     return ATTN_OK;
 }

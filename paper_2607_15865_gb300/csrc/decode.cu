@@ -1,28 +1,37 @@
-// decode.cu -- K3 split-KV decode attention (with the new token's RoPE + append fused
-// in) and K4 log-sum-exp combine.
+// decode.cu -- K3 split-KV decode attention for head_dim 64 (with the new tokens' RoPE +
+// append fused in) and K4 log-sum-exp combine.
 //
 // Decode (Section 4.4): one new query per sequence b at position p = hist_len[b]
 // attends to cache slots [0, p] of its kv head; its own k/v go to slot p (the
 // in-place "Concat" of Listing 2, Section 4.6.3).  The length mask of the paper is
-// given as hist_len on the device; slots past p are never used.
+// given as hist_len on the device; slots past p are never used.  The same kernel takes
+// ntok new tokens per sequence (verifying a draft): token i at position p + i attends to
+// slots [0, p + i], and the columns of the contraction are (token, query head) pairs.
 //
-// K3: CTA (split s, kv head g [x head pass], sequence b) owns keys
-// [s*per, min((s+1)*per, p+1)), per = max(ceil((p+1)/nsplit), 64) computed on the
-// device.  It streams them once for all query heads of the group:
+// K3: CTA (split s, kv head g x column pass, sequence b) owns keys
+// [s*per, min((s+1)*per, p+ntok)), per = max(ceil((p+ntok)/nsplit), 64) computed on the
+// device.  It streams them once for up to 8 columns (the passes of a kv head read the same
+// keys at about the same time, so the repeats come from L2):
 //   * thread 0 issues TMA tensor loads of 64-key K and V tiles (128-byte swizzle)
 //     into a 3-stage shared-memory ring (two CTAs per SM keep ~200 KB in flight);
 //   * QK: one key per thread over a quarter of D, the rotated queries (scale *
 //     log2(e) folded in) read from shared memory, partial sums to shared memory;
-//   * softmax: one warp per query head merges the partials, keeps the running
-//     (max, sum) in the log2 domain and writes the tile's P;
+//   * softmax: one warp per column merges the partials, masks the keys past the column's
+//     token, keeps the running (max, sum) in the log2 domain and writes the tile's P;
 //   * PV: one 16-byte V chunk per thread over a quarter of the tile's keys,
 //     accumulators rescaled by 2^(m_old - m_new);
-//   * the split whose range holds slot p rotates the new k (RoPE from the table,
-//     the same float arithmetic and bf16 rounding as K1), writes k and v to slot p
+//   * the split whose range holds a new slot rotates that token's k (RoPE from the table,
+//     the same float arithmetic and bf16 rounding as K1), writes k and v to the slot
 //     and substitutes them for that row of the loaded tile.
-// Each split writes its unnormalised partial (m, l, acc[D]) per head.
-// K4: per (query head, sequence): m* = max m_s, l = sum l_s 2^(m_s-m*),
+// Each split writes its unnormalised partial (m, l, acc[D]) per column.
+// K4: per (query head, token, sequence): m* = max m_s, l = sum l_s 2^(m_s-m*),
 // out = sum acc_s 2^(m_s-m*) / l -> bf16; a programmatic dependent launch of K3.
+//
+// What bounds it: for one token the stream of the keys; for several the CUDA cores (float
+// products and weights, 4 * 64 FLOP per key and column).  Several tokens as one launch
+// instead of one decode step each: the history is streamed once and the launches, gathers
+// and scatters of the steps go (5 tokens, 3 sequences of 700-4001 keys, 32 / 8 heads:
+// 30.8 us a call, host included; 153.4 as steps).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -38,6 +47,8 @@ constexpr int KT = 64;        // keys per tile
 constexpr int NSTAGE = 3;     // TMA ring depth
 constexpr int NTHREADS = 256;
 constexpr int NSLICE = 4;     // D slices of the QK phase
+constexpr int kD = 64;        // head_dim (128 runs on the tensor cores, decode_tc.cu)
+constexpr int kMaxTok = 16;   // new tokens per sequence in one launch
 
 template <int D, int GM>
 struct DecLayout {
@@ -50,8 +61,8 @@ struct DecLayout {
     static constexpr int OFF_P = OFF_PART + NSLICE * GM * KT * 4;   // float P[KT][8]
     static constexpr int OFF_ALPHA = OFF_P + KT * 8 * 4;            // float alpha[8]
     static constexpr int OFF_ML = OFF_ALPHA + 8 * 4;                // float m[8], l[8]
-    static constexpr int OFF_KNEW = OFF_ML + 16 * 4;                // bf16 k_new[D], v_new[D]
-    static constexpr int OFF_BAR = OFF_KNEW + 2 * D * 2;
+    static constexpr int OFF_KNEW = OFF_ML + 16 * 4;                // bf16 k_new[tokens][D], v_new[tokens][D]
+    static constexpr int OFF_BAR = OFF_KNEW + kMaxTok * 2 * D * 2;
     static constexpr int BYTES = OFF_BAR + NSTAGE * 8;
     static constexpr int ALLOC = BYTES + 1024;
     static constexpr int NKG = NTHREADS / (D / 8);     // key groups of the PV phase
@@ -91,11 +102,24 @@ __device__ __forceinline__ void fma8(float (&acc)[8], float p, const uint4& w) {
     x = ffma2(p2, make_float2(bf_lo(w.w), bf_hi(w.w)), make_float2(acc[6], acc[7])); acc[6] = x.x; acc[7] = x.y;
 }
 
+// The new tokens of sequence b that have a slot: token i takes position hist + i, and tokens
+// [lo, hi) are those whose position is in [0, max_len) (the others are skipped).
+struct TokRange {
+    int hist, lo, hi;
+};
+__device__ __forceinline__ TokRange decode_tokens(const int32_t* d_hist, int b, int hist_add, int ntok, int max_len) {
+    const long long h = static_cast<long long>(d_hist[b]) + hist_add;
+    const long long lo = h < 0 ? -h : 0, hi = min(static_cast<long long>(ntok), max_len - h);
+    if (lo >= hi) return {0, ntok, 0};
+    return {static_cast<int>(h), static_cast<int>(lo), static_cast<int>(hi)};
+}
+
 template <int D, int GM>
 __global__ void __launch_bounds__(NTHREADS, 2) decode_split_kernel(
     const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
     const uint16_t* __restrict__ q, const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
-    const int32_t* __restrict__ d_hist, int hist_add, uint16_t* __restrict__ k_cache, uint16_t* __restrict__ v_cache,
+    const int32_t* __restrict__ d_hist, int hist_add, int ntok, int seq_tok, uint16_t* __restrict__ k_cache,
+    uint16_t* __restrict__ v_cache,
     const float* __restrict__ cos_tab, const float* __restrict__ sin_tab, int Hq, int Hkv, int G, int passes,
     int max_len, int nsplit, float scale_log2, float* __restrict__ part_o, float* __restrict__ part_ml,
     int* __restrict__ err, uint64_t wait_ns) {
@@ -111,32 +135,36 @@ __global__ void __launch_bounds__(NTHREADS, 2) decode_split_kernel(
     float* alpha_s = reinterpret_cast<float*>(gb + L::OFF_ALPHA);
     float* ml_s = reinterpret_cast<float*>(gb + L::OFF_ML);
     uint16_t* knew_s = reinterpret_cast<uint16_t*>(gb + L::OFF_KNEW);
-    uint16_t* vnew_s = knew_s + D;
+    uint16_t* vnew_s = knew_s + kMaxTok * D;
 
+    // Columns c = token c / G, head c % G of the group; this pass takes c0 .. c0 + gcount - 1.
     const int s = blockIdx.x;
     const int g = blockIdx.y / passes;
     const int pass = blockIdx.y % passes;
     const int b = blockIdx.z;
-    const int h0 = g * G + pass * GM;
-    const int gcount = min(GM, G - pass * GM);
+    const int c0 = pass * GM;
+    const int gcount = min(GM, G * ntok - c0);
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
     const int lane = tid & 31;
 
-    const int hist = decode_hist(d_hist, b, hist_add);
-    if (hist < 0 || hist >= max_len) {
-        if (s == 0 && blockIdx.y == 0 && tid == 0) atomicOr(err, kDevErrHistRange);
-        return;  // sequence skipped: nothing written
-    }
-    const int nkeys = hist + 1;
+    const TokRange tr = decode_tokens(d_hist, b, hist_add, ntok, max_len);
+    if ((tr.lo > 0 || tr.hi < ntok) && s == 0 && blockIdx.y == 0 && tid == 0) atomicOr(err, kDevErrHistRange);
+    if (tr.lo >= tr.hi) return;  // sequence skipped: nothing written
+    const int hist = tr.hist;  // slot of token 0 (negative only where the tokens before tr.lo are skipped)
+    const int nkeys = hist + tr.hi;
     const int per = max((nkeys + nsplit - 1) / nsplit, KT);
     const int start = s * per;
     const int end = min(start + per, nkeys);
-    const size_t row0 = (static_cast<size_t>(b) * Hq + h0) * nsplit + s;  // head h adds h*nsplit
+    // partial row of column c: ((b * ntok + token) * Hq + head) * nsplit + s
+    auto part_row = [&](int c) -> size_t {
+        return ((static_cast<size_t>(b) * ntok + c / G) * Hq + g * G + c % G) * nsplit + s;
+    };
     if (start >= end) {  // an empty split: weight 0 in the combine
         if (tid < gcount) {
-            part_ml[(row0 + static_cast<size_t>(tid) * nsplit) * 2 + 0] = -INFINITY;
-            part_ml[(row0 + static_cast<size_t>(tid) * nsplit) * 2 + 1] = 0.f;
+            const size_t row = part_row(c0 + tid);
+            part_ml[row * 2 + 0] = -INFINITY;
+            part_ml[row * 2 + 1] = 0.f;
         }
         return;
     }
@@ -168,33 +196,44 @@ __global__ void __launch_bounds__(NTHREADS, 2) decode_split_kernel(
         for (int j = 0; j < min(NSTAGE, ntiles); ++j) issue(j);
     }
 
-    // Prologue: rotated queries (scaled into the log2 domain) and, for the split that
-    // owns slot `hist`, the new token's rotated k and its v, appended to the cache.
-    const float* cos_row = cos_tab + static_cast<size_t>(hist) * HALF;
-    const float* sin_row = sin_tab + static_cast<size_t>(hist) * HALF;
+    // Prologue: rotated queries (scaled into the log2 domain) and, for the split that owns
+    // any of the new slots, the new tokens' rotated k and their v, appended to the cache.
     for (int idx = tid; idx < GM * D; idx += NTHREADS) {
         const int h = idx / D, d = idx % D;
+        const int i = (c0 + h) / G;
         float v = 0.f;
-        if (h < gcount) {
-            const uint16_t* qrow = q + (static_cast<size_t>(b) * Hq + h0 + h) * D;
-            v = __bfloat162float(__float2bfloat16_rn(rope_elem<D>(qrow, d, cos_row, sin_row))) * scale_log2;
+        if (h < gcount && i >= tr.lo && i < tr.hi) {
+            const uint16_t* qrow =
+                q + ((static_cast<size_t>(b) * seq_tok + i) * Hq + g * G + (c0 + h) % G) * D;
+            const size_t pos = static_cast<size_t>(hist + i) * HALF;
+            v = __bfloat162float(__float2bfloat16_rn(rope_elem<D>(qrow, d, cos_tab + pos, sin_tab + pos))) * scale_log2;
         }
         qs[idx] = v;
     }
-    const bool own_new = hist >= start && hist < end;
-    if (own_new && tid < D) {
-        const uint16_t* krow = k_new + static_cast<size_t>(kv_row) * D;
-        const uint16_t kr = to_bf16(rope_elem<D>(krow, tid, cos_row, sin_row));
-        const uint16_t vv = v_new[static_cast<size_t>(kv_row) * D + tid];
-        knew_s[tid] = kr;
-        vnew_s[tid] = vv;
-        if (pass == 0) {
-            const size_t dst = (static_cast<size_t>(kv_row) * max_len + hist) * D + tid;
-            k_cache[dst] = kr;
-            v_cache[dst] = vv;
+    const int new0 = hist + tr.lo;  // first new slot
+    const bool own_new = new0 < end && nkeys > start;
+    if (own_new) {
+        for (int idx = tid; idx < ntok * D; idx += NTHREADS) {
+            const int i = idx / D, d = idx % D;
+            const int slot = hist + i;
+            if (i < tr.lo || slot < start || slot >= end) continue;
+            const size_t src = ((static_cast<size_t>(b) * seq_tok + i) * Hkv + g) * D;
+            const size_t pos = static_cast<size_t>(slot) * HALF;
+            const uint16_t kr = to_bf16(rope_elem<D>(k_new + src, d, cos_tab + pos, sin_tab + pos));
+            const uint16_t vv = v_new[src + d];
+            knew_s[idx] = kr;
+            vnew_s[idx] = vv;
+            if (pass == 0) {
+                const size_t dst = (static_cast<size_t>(kv_row) * max_len + slot) * D + d;
+                k_cache[dst] = kr;
+                v_cache[dst] = vv;
+            }
         }
     }
-    float m_run = -INFINITY, l_run = 0.f;  // warp h < gcount: running state of head h
+    // keys column `warp` may see in this split: slots below lim (none for a skipped token)
+    const int my_tok = (c0 + warp) / G;
+    const int my_lim = my_tok >= tr.lo && my_tok < tr.hi ? min(end, hist + my_tok + 1) : 0;
+    float m_run = -INFINITY, l_run = 0.f;  // warp h < gcount: running state of column h
     float acc[GM][8];
 #pragma unroll
     for (int h = 0; h < GM; ++h)
@@ -218,11 +257,14 @@ __global__ void __launch_bounds__(NTHREADS, 2) decode_split_kernel(
         uint8_t* ks = gb + st * L::STAGE;
         uint8_t* vs = ks + L::TILE;
         const int kt0 = start + j * KT;
-        if (own_new && hist >= kt0 && hist < kt0 + KT) {  // CTA-uniform
-            const int r = hist - kt0;
-            if (tid < D / 8) {
-                *reinterpret_cast<uint4*>(ks + swz(r, tid)) = reinterpret_cast<const uint4*>(knew_s)[tid];
-                *reinterpret_cast<uint4*>(vs + swz(r, tid)) = reinterpret_cast<const uint4*>(vnew_s)[tid];
+        const bool has_new = new0 < min(kt0 + KT, end);  // CTA-uniform
+        if (has_new) {
+            for (int idx = tid; idx < ntok * (D / 8); idx += NTHREADS) {
+                const int i = idx / (D / 8), c = idx % (D / 8);
+                const int slot = hist + i;
+                if (i < tr.lo || slot < kt0 || slot >= kt0 + KT || slot >= end) continue;
+                *reinterpret_cast<uint4*>(ks + swz(slot - kt0, c)) = reinterpret_cast<const uint4*>(knew_s)[idx];
+                *reinterpret_cast<uint4*>(vs + swz(slot - kt0, c)) = reinterpret_cast<const uint4*>(vnew_s)[idx];
             }
             __syncthreads();
         }
@@ -255,7 +297,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) decode_split_kernel(
         __syncthreads();
         // every thread is past the PV of tile j-1: refill its ring stage
         if (tid == 0 && j >= 1 && j - 1 + NSTAGE < ntiles) issue(j - 1 + NSTAGE);
-        // ---- softmax: warp h owns head h
+        // ---- softmax: warp h owns column h
         if (warp < gcount) {
             const int h = warp;
             float sc[2];
@@ -265,15 +307,17 @@ __global__ void __launch_bounds__(NTHREADS, 2) decode_split_kernel(
                 float v = 0.f;
 #pragma unroll
                 for (int sl = 0; sl < NSLICE; ++sl) v += part[(sl * GM + h) * KT + r];
-                sc[u] = (kt0 + r < end) ? v : -INFINITY;
+                sc[u] = (kt0 + r < my_lim) ? v : -INFINITY;
             }
             float mx = fmaxf(sc[0], sc[1]);
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
-            const float m_new = fmaxf(m_run, mx);          // finite: the tile has a valid key
-            const float alpha = fast_exp2(m_run - m_new);  // 0 on the first tile
-            const float p0 = fast_exp2(sc[0] - m_new);
-            const float p1 = fast_exp2(sc[1] - m_new);
+            // (the running max stays -inf, and the weights 0, while the column has seen no key)
+            const float m_new = fmaxf(m_run, mx);
+            const float m_ref = m_new == -INFINITY ? 0.f : m_new;
+            const float alpha = fast_exp2(m_run - m_ref);  // 0 on the first tile
+            const float p0 = fast_exp2(sc[0] - m_ref);
+            const float p1 = fast_exp2(sc[1] - m_ref);
             float sum = p0 + p1;
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, off);
@@ -299,8 +343,14 @@ __global__ void __launch_bounds__(NTHREADS, 2) decode_split_kernel(
                 const float4 pa = *reinterpret_cast<const float4*>(P + r * 8);
                 const float4 pb = *reinterpret_cast<const float4*>(P + r * 8 + 4);
                 const float pr[8] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
+                if (kt0 + r <= new0) {  // visible to every token
 #pragma unroll
-                for (int h = 0; h < GM; ++h) fma8(acc[h], pr[h], vw);
+                    for (int h = 0; h < GM; ++h) fma8(acc[h], pr[h], vw);
+                } else {  // a later new token's v, which may be anything, is never multiplied
+#pragma unroll
+                    for (int h = 0; h < GM; ++h)
+                        if (kt0 + r <= hist + (c0 + h) / G) fma8(acc[h], pr[h], vw);
+                }
             }
         }
     }
@@ -342,7 +392,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) decode_split_kernel(
         float a = 0.f;
 #pragma unroll
         for (int w = 0; w < NTHREADS / 32; ++w) a += red[(w * GM + h) * D + d];
-        const size_t row = row0 + static_cast<size_t>(h) * nsplit;
+        const size_t row = part_row(c0 + h);
         part_o[row * D + d] = a;
         if (d == 0) {
             part_ml[row * 2 + 0] = ml_s[h];
@@ -354,19 +404,19 @@ __global__ void __launch_bounds__(NTHREADS, 2) decode_split_kernel(
 template <int D>
 __global__ void __launch_bounds__(256) decode_combine_kernel(const float* __restrict__ part_o,
                                                              const float* __restrict__ part_ml,
-                                                             const int32_t* __restrict__ d_hist, int hist_add, int Hq,
-                                                             int nsplit,
-                                                             int max_len, uint16_t* __restrict__ out) {
+                                                             const int32_t* __restrict__ d_hist, int hist_add,
+                                                             int ntok, int seq_tok, int Hq, int nsplit, int max_len,
+                                                             uint16_t* __restrict__ out) {
     constexpr int PER_LANE = D / 32;
     __shared__ float sm_w[256];
     __shared__ float sm_red[8][D];
     __shared__ float sm_inv_l;
     asm volatile("griddepcontrol.wait;" ::: "memory");  // K3's partials are complete and visible
-    const int h = blockIdx.x;
+    const int tok = blockIdx.x / Hq, h = blockIdx.x % Hq;
     const int b = blockIdx.y;
-    const int hist = decode_hist(d_hist, b, hist_add);
-    if (hist < 0 || hist >= max_len) return;
-    const size_t row0 = (static_cast<size_t>(b) * Hq + h) * nsplit;
+    const TokRange tr = decode_tokens(d_hist, b, hist_add, ntok, max_len);
+    if (tok < tr.lo || tok >= tr.hi) return;
+    const size_t row0 = ((static_cast<size_t>(b) * ntok + tok) * Hq + h) * nsplit;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0) {
         float mm = -INFINITY;
@@ -404,70 +454,44 @@ __global__ void __launch_bounds__(256) decode_combine_kernel(const float* __rest
         float t = 0.f;
 #pragma unroll
         for (int w = 0; w < 8; ++w) t += sm_red[w][d];
-        out[(static_cast<size_t>(b) * Hq + h) * D + d] = to_bf16(t * sm_inv_l);
+        out[((static_cast<size_t>(b) * seq_tok + tok) * Hq + h) * D + d] = to_bf16(t * sm_inv_l);
     }
 }
 
-template <int D, int GM>
+template <int GM>
 cudaError_t launch_split_t(const Shape& s, const DecodeMaps& maps, dim3 grid, const uint16_t* q,
-                           const uint16_t* k_new, const uint16_t* v_new, const int32_t* d_hist, int hist_add,
-                           uint16_t* kc, uint16_t* vc, const float* cos_tab, const float* sin_tab, int G, int passes,
-                           int nsplit,
-                           float scale_log2, float* part_o, float* part_ml, int* err, cudaStream_t st, uint64_t wait_ns) {
-    decode_split_kernel<D, GM><<<grid, NTHREADS, DecLayout<D, GM>::ALLOC, st>>>(
-        maps.k, maps.v, q, k_new, v_new, d_hist, hist_add, kc, vc, cos_tab, sin_tab, s.n_q_heads, s.n_kv_heads, G,
-        passes,
-        s.max_len, nsplit, scale_log2, part_o, part_ml, err, wait_ns);
+                           const uint16_t* k_new, const uint16_t* v_new, const int32_t* d_hist, int hist_add, int ntok,
+                           int seq_tok, uint16_t* kc, uint16_t* vc, const float* cos_tab, const float* sin_tab, int G,
+                           int passes, int nsplit, float* part_o, float* part_ml, int* err, cudaStream_t st,
+                           uint64_t wait_ns) {
+    const float scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(kD)));
+    decode_split_kernel<kD, GM><<<grid, NTHREADS, DecLayout<kD, GM>::ALLOC, st>>>(
+        maps.k, maps.v, q, k_new, v_new, d_hist, hist_add, ntok, seq_tok, kc, vc, cos_tab, sin_tab, s.n_q_heads,
+        s.n_kv_heads, G, passes, s.max_len, nsplit, scale_log2, part_o, part_ml, err, wait_ns);
     return cudaGetLastError();
 }
 
-template <int D>
-cudaError_t launch_split_d(const Shape& s, const DecodeMaps& maps, const uint16_t* q, const uint16_t* k_new,
-                           const uint16_t* v_new, const int32_t* d_hist, int hist_add, uint16_t* kc, uint16_t* vc,
-                           const float* cos_tab, const float* sin_tab, int nsplit, float* part_o, float* part_ml,
-                           int* err, cudaStream_t st, uint64_t wait_ns) {
-    const float scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(D)));
-    const int G = s.n_q_heads / s.n_kv_heads;
-    const int passes = (G + 7) / 8;
-    const int gm = (G + passes - 1) / passes;
-    const dim3 grid(static_cast<unsigned>(nsplit), static_cast<unsigned>(s.n_kv_heads * passes),
-                    static_cast<unsigned>(s.batch));
-    switch (gm) {
-#define ATTN_SPLIT_CASE(N)                                                                                     \
-    case N:                                                                                                    \
-        return launch_split_t<D, N>(s, maps, grid, q, k_new, v_new, d_hist, hist_add, kc, vc, cos_tab, sin_tab, G, \
-                                    passes, nsplit, scale_log2, part_o, part_ml, err, st, wait_ns);
-        ATTN_SPLIT_CASE(1) ATTN_SPLIT_CASE(2) ATTN_SPLIT_CASE(3) ATTN_SPLIT_CASE(4)
-        ATTN_SPLIT_CASE(5) ATTN_SPLIT_CASE(6) ATTN_SPLIT_CASE(7) ATTN_SPLIT_CASE(8)
-#undef ATTN_SPLIT_CASE
-        default:
-            return cudaErrorInvalidValue;
-    }
-}
-
-template <int D, int GM>
+template <int GM>
 cudaError_t set_smem_attr() {
-    return cudaFuncSetAttribute(decode_split_kernel<D, GM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                DecLayout<D, GM>::ALLOC);
+    return cudaFuncSetAttribute(decode_split_kernel<kD, GM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                DecLayout<kD, GM>::ALLOC);
 }
 
 }  // namespace
 
 cudaError_t configure_decode() {
     cudaError_t e = cudaSuccess;
-#define ATTN_CFG(D, N) \
-    if (e == cudaSuccess) e = set_smem_attr<D, N>();
-    ATTN_CFG(128, 1) ATTN_CFG(128, 2) ATTN_CFG(128, 3) ATTN_CFG(128, 4)
-    ATTN_CFG(128, 5) ATTN_CFG(128, 6) ATTN_CFG(128, 7) ATTN_CFG(128, 8)
-    ATTN_CFG(64, 1) ATTN_CFG(64, 2) ATTN_CFG(64, 3) ATTN_CFG(64, 4)
-    ATTN_CFG(64, 5) ATTN_CFG(64, 6) ATTN_CFG(64, 7) ATTN_CFG(64, 8)
+#define ATTN_CFG(N) \
+    if (e == cudaSuccess) e = set_smem_attr<N>();
+    ATTN_CFG(1) ATTN_CFG(2) ATTN_CFG(3) ATTN_CFG(4) ATTN_CFG(5) ATTN_CFG(6) ATTN_CFG(7) ATTN_CFG(8)
 #undef ATTN_CFG
     return e;
 }
 
-int decode_num_splits(const Shape& s, int num_sms, int max_splits) {
-    const int G = s.n_q_heads / s.n_kv_heads;
-    const long items = static_cast<long>(s.batch) * s.n_kv_heads * ((G + 7) / 8);
+int decode_passes(const Shape& s, int ntok) { return (s.n_q_heads / s.n_kv_heads * ntok + 7) / 8; }
+
+int decode_num_splits(const Shape& s, int num_sms, int max_splits, int ntok) {
+    const long items = static_cast<long>(s.batch) * s.n_kv_heads * decode_passes(s, ntok);
     const long slots = 2L * num_sms;  // two CTAs per SM
     const long cap = std::max(1L, std::min<long>(max_splits, (s.max_len + KT - 1) / KT));
     // the smallest split count whose CTAs fill whole waves to >= 90%, else the best seen
@@ -505,20 +529,34 @@ cudaError_t make_decode_maps(PFN_encodeTiled encode, const Shape& s, const uint1
 }
 
 cudaError_t launch_decode_split(const Shape& s, const DecodeMaps& maps, const uint16_t* q, const uint16_t* k_new,
-                                const uint16_t* v_new, const int32_t* d_hist, int hist_add, uint16_t* k_cache,
-                                uint16_t* v_cache, const float* cos_tab, const float* sin_tab, float* part_o,
-                                float* part_ml, int nsplit, int* err, cudaStream_t st, uint64_t wait_ns) {
-    if (s.head_dim == 128)
-        return launch_split_d<128>(s, maps, q, k_new, v_new, d_hist, hist_add, k_cache, v_cache, cos_tab, sin_tab,
-                                   nsplit, part_o, part_ml, err, st, wait_ns);
-    return launch_split_d<64>(s, maps, q, k_new, v_new, d_hist, hist_add, k_cache, v_cache, cos_tab, sin_tab, nsplit,
-                              part_o, part_ml, err, st, wait_ns);
+                                const uint16_t* v_new, const int32_t* d_hist, int hist_add, int ntok, int seq_tok,
+                                uint16_t* k_cache, uint16_t* v_cache, const float* cos_tab, const float* sin_tab,
+                                float* part_o, float* part_ml, int nsplit, int* err, cudaStream_t st,
+                                uint64_t wait_ns) {
+    if (s.head_dim != kD || ntok < 1 || ntok > kMaxTok) return cudaErrorInvalidValue;
+    const int G = s.n_q_heads / s.n_kv_heads;
+    const int passes = decode_passes(s, ntok);
+    const int gm = (G * ntok + passes - 1) / passes;
+    const dim3 grid(static_cast<unsigned>(nsplit), static_cast<unsigned>(s.n_kv_heads * passes),
+                    static_cast<unsigned>(s.batch));
+    switch (gm) {
+#define ATTN_SPLIT_CASE(N)                                                                                             \
+    case N:                                                                                                            \
+        return launch_split_t<N>(s, maps, grid, q, k_new, v_new, d_hist, hist_add, ntok, seq_tok, k_cache, v_cache,    \
+                                 cos_tab, sin_tab, G, passes, nsplit, part_o, part_ml, err, st, wait_ns);
+        ATTN_SPLIT_CASE(1) ATTN_SPLIT_CASE(2) ATTN_SPLIT_CASE(3) ATTN_SPLIT_CASE(4)
+        ATTN_SPLIT_CASE(5) ATTN_SPLIT_CASE(6) ATTN_SPLIT_CASE(7) ATTN_SPLIT_CASE(8)
+#undef ATTN_SPLIT_CASE
+        default:
+            return cudaErrorInvalidValue;
+    }
 }
 
-cudaError_t launch_decode_combine(const Shape& s, const int32_t* d_hist, int hist_add, const float* part_o,
-                                  const float* part_ml, int nsplit, uint16_t* out, cudaStream_t st) {
+cudaError_t launch_decode_combine(const Shape& s, const int32_t* d_hist, int hist_add, int ntok, int seq_tok,
+                                  const float* part_o, const float* part_ml, int nsplit, uint16_t* out,
+                                  cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(s.n_q_heads), static_cast<unsigned>(s.batch));
+    cfg.gridDim = dim3(static_cast<unsigned>(s.n_q_heads) * static_cast<unsigned>(ntok), static_cast<unsigned>(s.batch));
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
@@ -527,11 +565,8 @@ cudaError_t launch_decode_combine(const Shape& s, const int32_t* d_hist, int his
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (s.head_dim == 128)
-        return cudaLaunchKernelEx(&cfg, decode_combine_kernel<128>, part_o, part_ml, d_hist, hist_add, s.n_q_heads, nsplit,
-                                  s.max_len, out);
-    return cudaLaunchKernelEx(&cfg, decode_combine_kernel<64>, part_o, part_ml, d_hist, hist_add, s.n_q_heads, nsplit,
-                              s.max_len, out);
+    return cudaLaunchKernelEx(&cfg, decode_combine_kernel<kD>, part_o, part_ml, d_hist, hist_add, ntok, seq_tok,
+                              s.n_q_heads, nsplit, s.max_len, out);
 }
 
 }  // namespace attn

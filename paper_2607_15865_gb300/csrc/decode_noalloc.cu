@@ -146,8 +146,8 @@ extern "C" int attn_decode_noalloc(const attn_cfg* cfg, const float* d_cos, cons
     cudaError_t e = tc ? attn::launch_decode_tc(s, maps, q, k, v, d_hist_len, 0, k_cache, v_cache, d_cos, d_sin, part_o,
                                                 part_ml, counters, nsplit, out, d_err, false, 1, st, false,
                                                 attn::kWaitLimitNs, num_sms)
-                       : attn::launch_decode_split(s, maps, q, k, v, d_hist_len, 0, k_cache, v_cache, d_cos, d_sin,
+                       : attn::launch_decode_split(s, maps, q, k, v, d_hist_len, 0, 1, 1, k_cache, v_cache, d_cos, d_sin,
                                                    part_o, part_ml, nsplit, d_err, st);
-    if (e == cudaSuccess && !tc) e = attn::launch_decode_combine(s, d_hist_len, 0, part_o, part_ml, nsplit, out, st);
+    if (e == cudaSuccess && !tc) e = attn::launch_decode_combine(s, d_hist_len, 0, 1, 1, part_o, part_ml, nsplit, out, st);
     return e == cudaSuccess ? ATTN_OK : attn::record_cuda_error(e, "attn_decode_noalloc: launch");
 }

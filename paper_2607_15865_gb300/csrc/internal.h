@@ -81,23 +81,28 @@ cudaError_t launch_flash_fwd(const Shape& s, const FlashMaps& maps, int hist, in
                              const float* cos_t, const float* sin_t, uint16_t* out, float* ws_o, float* ws_ml, int* err,
                              int num_sms, cudaStream_t st, int* n_launched, uint64_t wait_ns = kWaitLimitNs);
 
-// K3 + K4: decode.  The maps cover the whole caches as 3-D {D, max_len, B*Hkv}
-// with 64-key boxes (built once per cache pair).  K3 also rotates the new key and
-// appends k and v at slot hist[b]; K4 merges the splits (programmatic dependent launch).
+// K3 + K4: decode, head_dim 64.  The maps cover the whole caches as 3-D {D, max_len, B*Hkv}
+// with 64-key boxes (built once per cache pair).  K3 also rotates the new keys and
+// appends k and v from slot hist[b] on; K4 merges the splits (programmatic dependent launch).
 using PFN_encodeTiled = PFN_cuTensorMapEncodeTiled_v12000;
 struct DecodeMaps {
     CUtensorMap k;
     CUtensorMap v;
 };
 cudaError_t configure_decode();  // dynamic shared-memory limits of K3 (once per device)
-int decode_num_splits(const Shape& s, int num_sms, int max_splits);
+// Passes of up to 8 (token, head) columns that a kv head's ntok new tokens take.
+int decode_passes(const Shape& s, int ntok);
+int decode_num_splits(const Shape& s, int num_sms, int max_splits, int ntok = 1);
 cudaError_t make_decode_maps(PFN_encodeTiled encode, const Shape& s, const uint16_t* k_cache,
                              const uint16_t* v_cache, DecodeMaps* maps);
 // Decode lengths: sequence b's new token takes position d_hist[b] + hist_add (hist_add >= 0
-// lets a run of decode steps share one length array); see decode_hist().
+// lets a run of decode steps share one length array); see decode_hist().  1 <= ntok <= 16 new
+// tokens per sequence at positions d_hist[b] + hist_add + i; q, k_new, v_new and out point at
+// the first of them in arrays of seq_tok tokens per sequence.  A token whose position is
+// outside [0, max_len) is flagged and skipped.  The partials need B * ntok * Hq * nsplit rows.
 cudaError_t launch_decode_split(const Shape& s, const DecodeMaps& maps, const uint16_t* q, const uint16_t* k_new,
-                                const uint16_t* v_new, const int32_t* d_hist, int hist_add, uint16_t* k_cache,
-                                uint16_t* v_cache,
+                                const uint16_t* v_new, const int32_t* d_hist, int hist_add, int ntok, int seq_tok,
+                                uint16_t* k_cache, uint16_t* v_cache,
                                 const float* cos_tab, const float* sin_tab, float* part_o, float* part_ml,
                                 int nsplit, int* err, cudaStream_t st, uint64_t wait_ns = kWaitLimitNs);
 // K3 for head_dim 128 on the tensor cores (decode_tc.cu): maps with 128-key boxes; same
@@ -133,8 +138,9 @@ cudaError_t launch_decode_tc(const Shape& s, const DecodeMaps& maps, const uint1
                              const float* cos_tab, const float* sin_tab, float* part_o, float* part_ml,
                              int* counters, int nsplit, uint16_t* out, int* err, bool after_decode, int ntok,
                              cudaStream_t st, bool producer_early, uint64_t wait_ns, int num_sms);
-cudaError_t launch_decode_combine(const Shape& s, const int32_t* d_hist, int hist_add, const float* part_o,
-                                  const float* part_ml, int nsplit, uint16_t* out, cudaStream_t st);
+cudaError_t launch_decode_combine(const Shape& s, const int32_t* d_hist, int hist_add, int ntok, int seq_tok,
+                                  const float* part_o, const float* part_ml, int nsplit, uint16_t* out,
+                                  cudaStream_t st);
 
 // W4BF16 GEMV (w4_gemv.cu): y[m, n] = sum_k x[m, k] (q[n, k] - z[n, k/128]) s[n, k/128] for
 // the 1 <= M <= w4_gemv_max_rows(K) activation rows of one launch.  tiles: the tile
