@@ -85,3 +85,17 @@ def test_w4_gemm_rejects_bad_arguments(torch):
                  (p, p, 1, 128, 192, p, None), (p + 8, p, 1, 128, 128, p, None), (p, p + 8, 1, 128, 128, p, None),
                  (p, p, 1, 128, 128, p + 8, None), (p, p, 65535 * 128 + 1, 128, 128, p, None)]:
         assert lib.attn_w4bf16_gemm(*args, None) == _lib.ATTN_EINVAL, args
+
+
+# Edges of the plans: 32- and 256-token tiles, an odd number of 128-feature halves, K split over
+# 2, 3 and 4 pairs of a cluster with uneven slices, groups fewer than splits, several rounds.
+PLANS = [("t33_k512", 33, 256, 512), ("t32_k1664_13_groups", 32, 1024, 1664), ("t250_n640", 250, 640, 1024),
+         ("t257_n2048", 257, 2048, 384), ("t64_n6144", 64, 6144, 1024), ("t2_n22016_two_rounds", 2, 22016, 256),
+         ("t1030_n4992", 1030, 4992, 256)]
+
+
+@pytest.mark.parametrize("tag,T,N,K", PLANS, ids=[c[0] for c in PLANS])
+def test_w4_gemm_plans_match_oracle(torch, tag, T, N, K):
+    codes, scales, zeros = mat(tag, N, K)
+    x = gen.normal_bf16("w4gemm", f"{tag}_x", (T, K), 1.0)
+    check(codes, scales, zeros, x, run(torch, codes, scales, zeros, x))
