@@ -40,8 +40,10 @@ __global__ void __launch_bounds__(128) rope_append_kernel(const uint16_t* __rest
     constexpr int HALF = D / 2;
     constexpr int ROPE_UNITS = D / 16;  // 8 pairs per unit
     constexpr int COPY_UNITS = D / 8;   // 8 elements per unit
-    // K1 is launched in stream order (its inputs are complete when it starts); the K2
-    // launch that follows it may begin its q-side prologue as soon as every K1 CTA runs.
+    // K1 is a dependent launch: its CTAs may be resident while the previous kernel ends, and
+    // start only once that is complete.  The K2 launch that follows may then begin its q-side
+    // prologue as soon as every K1 CTA runs (it reads q, so never before this wait).
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int i = blockIdx.x;
     const int b = blockIdx.y;
@@ -116,14 +118,18 @@ cudaError_t launch_rope_append(const Shape& s, const uint16_t* k, const uint16_t
                                const int32_t* d_hist, int chunk, int seq_stride, const float* cos_tab,
                                const float* sin_tab, const float* cos_t, const float* sin_t, uint16_t* k_cache,
                                uint16_t* v_cache, int* err, cudaStream_t st) {
-    const dim3 grid(static_cast<unsigned>(chunk), static_cast<unsigned>(s.batch));
-    if (s.head_dim == 128)
-        rope_append_kernel<128><<<grid, 128, 0, st>>>(k, v, hist, d_hist, chunk, seq_stride, s.n_kv_heads, s.max_len, cos_tab,
-                                                      sin_tab, cos_t, sin_t, k_cache, v_cache, err);
-    else
-        rope_append_kernel<64><<<grid, 128, 0, st>>>(k, v, hist, d_hist, chunk, seq_stride, s.n_kv_heads, s.max_len, cos_tab,
-                                                     sin_tab, cos_t, sin_t, k_cache, v_cache, err);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(chunk), static_cast<unsigned>(s.batch));
+    cfg.blockDim = dim3(128);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, s.head_dim == 128 ? rope_append_kernel<128> : rope_append_kernel<64>, k, v, hist,
+                              d_hist, chunk, seq_stride, s.n_kv_heads, s.max_len, cos_tab, sin_tab, cos_t, sin_t,
+                              k_cache, v_cache, err);
 }
 
 }  // namespace attn

@@ -560,6 +560,8 @@ __global__ void __launch_bounds__(256) rmsnorm_rows_kernel(const uint16_t* __res
                                                            const uint16_t* __restrict__ gamma, float eps, int T, int K,
                                                            uint16_t* __restrict__ xn) {
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    griddep_wait();  // a dependent launch, as is the GEMM that follows
+    griddep_launch_dependents();
     if (row >= T) return;
     const uint4* xr = reinterpret_cast<const uint4*>(x + static_cast<size_t>(row) * K);
     const int nchunk = K / 8;
@@ -676,8 +678,16 @@ cudaError_t configure(int dev) {
 
 cudaError_t launch_rmsnorm_rows(const uint16_t* x, const uint16_t* gamma, float eps, int T, int K, uint16_t* xn,
                                 cudaStream_t st) {
-    rmsnorm_rows_kernel<<<(T + 7) / 8, 256, 0, st>>>(x, gamma, eps, T, K, xn);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>((T + 7) / 8));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, rmsnorm_rows_kernel, x, gamma, eps, T, K, xn);
 }
 
 cudaError_t launch_w4_gemm(const uint8_t* tiles, const uint16_t* x, int T, int N, int K, uint16_t* y, int* err,
