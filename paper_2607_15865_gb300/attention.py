@@ -27,6 +27,15 @@ _BF16_LIKE = (torch.bfloat16, torch.int16, torch.uint16)
 
 
 def _ptr(t: torch.Tensor, name: str, shape=None) -> int:
+    # one pass of cheap tests for the arguments every call gets right (a third of the time of
+    # the checks below, six to eight times per call); whatever fails them is looked at in turn
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.dtype in _BF16_LIKE and t.is_contiguous() and (
+            shape is None or t.shape == shape):
+        return t.data_ptr()
+    return _ptr_checked(t, name, shape)
+
+
+def _ptr_checked(t, name: str, shape) -> int:
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype not in _BF16_LIKE:
@@ -39,8 +48,15 @@ def _ptr(t: torch.Tensor, name: str, shape=None) -> int:
 
 
 def _stream(stream) -> int:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    # the handle of torch.cuda.current_stream(), without building the Stream object
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+def _is_len(t, batch: int) -> bool:
+    return (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == torch.int32 and t.is_contiguous()
+            and t.shape == (batch,))
 
 
 class Attention:
@@ -57,6 +73,7 @@ class Attention:
         if rc != _lib.ATTN_OK:
             raise _lib.AttnError(rc, "attn_create", self.lib)
         self._ctx = handle
+        self._cache = (batch, n_kv_heads, max_len, head_dim)
 
     @classmethod
     def for_shape(cls, shape) -> "Attention":
@@ -82,7 +99,7 @@ class Attention:
             raise _lib.AttnError(rc, what, self.lib)
 
     def _cache_shape(self):
-        return (self.batch, self.n_kv_heads, self.max_len, self.head_dim)
+        return self._cache
 
     def _new_out(self, q: torch.Tensor, out):
         return torch.empty_like(q) if out is None else out
@@ -109,8 +126,7 @@ class Attention:
     def decode(self, q, k, v, hist_len: torch.Tensor, k_cache, v_cache, out=None, stream=None) -> torch.Tensor:
         qs = (self.batch, 1, self.n_q_heads, self.head_dim)
         ks = (self.batch, 1, self.n_kv_heads, self.head_dim)
-        if not (isinstance(hist_len, torch.Tensor) and hist_len.is_cuda and hist_len.dtype == torch.int32
-                and hist_len.is_contiguous() and tuple(hist_len.shape) == (self.batch,)):
+        if not _is_len(hist_len, self.batch):
             raise TypeError("hist_len must be a contiguous int32 CUDA tensor of shape [batch]")
         out = self._new_out(q, out)
         rc = self.lib.attn_decode(self._ctx, _ptr(q, "q", qs), _ptr(k, "k", ks), _ptr(v, "v", ks),
@@ -126,8 +142,7 @@ class Attention:
         n = q.shape[1]
         qs = (self.batch, n, self.n_q_heads, self.head_dim)
         ks = (self.batch, n, self.n_kv_heads, self.head_dim)
-        if not (isinstance(hist_len, torch.Tensor) and hist_len.is_cuda and hist_len.dtype == torch.int32
-                and hist_len.is_contiguous() and tuple(hist_len.shape) == (self.batch,)):
+        if not _is_len(hist_len, self.batch):
             raise TypeError("hist_len must be a contiguous int32 CUDA tensor of shape [batch]")
         out = self._new_out(q, out)
         rc = self.lib.attn_decode_multi(self._ctx, _ptr(q, "q", qs), _ptr(k, "k", ks), _ptr(v, "v", ks),
@@ -142,8 +157,7 @@ class Attention:
         """One decode step of the attention half of a decoder block with W4BF16 weights
         (attn_decode_layer): x [B, hidden] -> x + o_proj(attention(qkv_proj(RMSNorm(x))))."""
         hidden = x.shape[-1]
-        if not (isinstance(hist_len, torch.Tensor) and hist_len.is_cuda and hist_len.dtype == torch.int32
-                and hist_len.is_contiguous() and tuple(hist_len.shape) == (self.batch,)):
+        if not _is_len(hist_len, self.batch):
             raise TypeError("hist_len must be a contiguous int32 CUDA tensor of shape [batch]")
         for t, name in ((wqkv_tiles, "wqkv_tiles"), (wo_tiles, "wo_tiles")):
             if not (isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous() and t.dtype == torch.uint8):
@@ -218,8 +232,7 @@ class Attention:
         n = q.shape[0]
         qs = (n, self.batch, 1, self.n_q_heads, self.head_dim)
         ks = (n, self.batch, 1, self.n_kv_heads, self.head_dim)
-        if not (isinstance(hist_len, torch.Tensor) and hist_len.is_cuda and hist_len.dtype == torch.int32
-                and hist_len.is_contiguous() and tuple(hist_len.shape) == (self.batch,)):
+        if not _is_len(hist_len, self.batch):
             raise TypeError("hist_len must be a contiguous int32 CUDA tensor of shape [batch]")
         out = self._new_out(q, out)
         rc = self.lib.attn_decode_steps(self._ctx, _ptr(q, "q", qs), _ptr(k, "k", ks), _ptr(v, "v", ks),
