@@ -318,7 +318,7 @@ int attn_decode_noalloc(const attn_cfg* cfg, const float* d_cos, const float* d_
  *           during the previous call's last CTAs: set it only when the kernel right
  *           before this call on the stream does not write w_tiles.
  * K a positive multiple of 128 with attn_w4bf16_rows_per_launch(K) >= 1; any M >= 1,
- * N >= 1.  One launch serves attn_w4bf16_rows_per_launch(K) rows of x (x is staged in
+ * N >= 1.  One launch serves at least attn_w4bf16_rows_per_launch(K) rows of x (x is staged in
  * shared memory); further rows take further passes over the weights.  Enqueued on
  * `stream`; nothing is allocated or synchronised; buffers stay the caller's.
  * Returns ATTN_OK, ATTN_EINVAL (null pointer, bad size, alignment or flag), ATTN_EARCH
@@ -407,7 +407,8 @@ int attn_prefill_layer(attn_ctx* ctx, const uint16_t* x, const uint16_t* rms_gam
 int attn_w4bf16_gemm(const void* w_tiles, const uint16_t* x, int T, int N, int K, uint16_t* y, int32_t* d_err,
                      attn_stream_t stream);
 
-/* Rows of x one attn_w4bf16_gemv launch serves for inner size K: 8, 4, 2 or 1, or 0
+/* Rows of x any attn_w4bf16_gemv launch serves for inner size K (one without RMSNorm may
+ * serve up to 8 at every K): 8, 4, 2 or 1, or 0
  * when K is not a positive multiple of 128 or too large to stage (host only). */
 int attn_w4bf16_rows_per_launch(int K);
 

@@ -523,8 +523,7 @@ int attn_w4bf16_gemv_fused(const void* w_tiles, const uint16_t* x, int M, int N,
     if (w_tiles == nullptr || x == nullptr || y == nullptr) return ATTN_EINVAL;
     if (flags & ~ATTN_W4_WEIGHTS_STATIC) return ATTN_EINVAL;
     if (M < 1 || N < 1 || K < 128 || K % 128 != 0) return ATTN_EINVAL;
-    const int rows = attn::w4_gemv_max_rows(K);
-    if (rows < 1) return ATTN_EINVAL;
+    if (attn::w4_gemv_max_rows(K) < 1) return ATTN_EINVAL;
     if ((reinterpret_cast<uintptr_t>(w_tiles) & 15u) || (reinterpret_cast<uintptr_t>(x) & 15u) ||
         (reinterpret_cast<uintptr_t>(y) & 1u) || (reinterpret_cast<uintptr_t>(d_err) & 3u) ||
         (reinterpret_cast<uintptr_t>(rms_gamma) & 7u) || (reinterpret_cast<uintptr_t>(residual) & 1u) ||
@@ -556,8 +555,7 @@ int attn_w4bf16_gemv_fused(const void* w_tiles, const uint16_t* x, int M, int N,
     if (arch != 1) return ATTN_EARCH;
     const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     // Rows of x past what one launch stages take further passes over the weights.
-    for (int m0 = 0; m0 < M; m0 += rows) {
-        const int mc = std::min(rows, M - m0);
+    for (int m0 = 0, mc = 0; m0 < M; m0 += mc) {
         attn::W4Fused f = fz;
         const size_t r0 = static_cast<size_t>(m0);
         if (f.residual != nullptr) f.residual += r0 * N;
@@ -565,8 +563,8 @@ int attn_w4bf16_gemv_fused(const void* w_tiles, const uint16_t* x, int M, int N,
             f.y1 += r0 * (f.n1 - f.n0);
             f.y2 += r0 * (N - f.n1);
         }
-        e = attn::launch_w4_gemv(static_cast<const uint8_t*>(w_tiles), x + r0 * K, mc, N, K, y + r0 * fz.n0, d_err,
-                                 (flags & ATTN_W4_WEIGHTS_STATIC) != 0, f, st);
+        e = attn::launch_w4_gemv(static_cast<const uint8_t*>(w_tiles), x + r0 * K, M - m0, N, K, y + r0 * fz.n0, d_err,
+                                 (flags & ATTN_W4_WEIGHTS_STATIC) != 0, f, st, &mc);
         if (e != cudaSuccess) return cuda_fail(e, "w4_gemv");
     }
     return ATTN_OK;

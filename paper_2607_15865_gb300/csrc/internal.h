@@ -143,12 +143,13 @@ cudaError_t launch_decode_combine(const Shape& s, const int32_t* d_hist, int his
                                   cudaStream_t st);
 
 // W4BF16 GEMV (w4_gemv.cu): y[m, n] = sum_k x[m, k] (q[n, k] - z[n, k/128]) s[n, k/128] for
-// the 1 <= M <= w4_gemv_max_rows(K) activation rows of one launch.  tiles: the tile
+// the activation rows of one launch.  tiles: the tile
 // stream of attn_w4bf16_gemv (16-byte aligned); x: bf16 [M][K] (16-byte aligned);
 // y: bf16 [M][N].  K a multiple of 128.  A launch stages x and its group sums in the
-// shared memory its rings leave free.  A bounded wait that runs out sets
+// shared memory its rings leave free, whole per CTA or, where x is long, a slice of K per CTA
+// of a cluster.  A bounded wait that runs out sets
 // kDevErrTimeout in *err (when err is not null).
-int w4_gemv_max_rows(int K);  // 8, 4, 2, 1 or 0 (K too large)
+int w4_gemv_max_rows(int K);  // rows of x a CTA stages whole: 8, 4, 2, 1 or 0 (K too large)
 // Fused parts of a GEMV (all optional): RMSNorm of x before the product (gamma: bf16 [K],
 // 8-byte aligned), a residual added before rounding (bf16 [M][N]), and the output columns
 // split three ways: [0, n0) -> y (row stride n0), [n0, n1) -> y1, [n1, N) -> y2 (no split:
@@ -163,8 +164,9 @@ struct W4Fused {
 };
 // The launch is a programmatic dependent of the stream's previous kernel; early_weights lets
 // it read the tiles before that kernel has finished (see attn_w4bf16_gemv).
+// Serves the first *rows <= M of x's rows (at least w4_gemv_max_rows(K) of them where M has as many).
 cudaError_t launch_w4_gemv(const uint8_t* tiles, const uint16_t* x, int M, int N, int K, uint16_t* y, int* err,
-                           bool early_weights, const W4Fused& fz, cudaStream_t st);
+                           bool early_weights, const W4Fused& fz, cudaStream_t st, int* rows);
 
 // W4BF16 GEMM (w4_gemm.cu): y[t, n] = sum_k x[t, k] bf16((q - z) s)[n, k] for T tokens;
 // N and K multiples of 128; x bf16 [T][K] and y bf16 [T][N] 16-byte aligned; tiles: the

@@ -20,7 +20,9 @@
 //     of word i, a shift and one masked OR of the bf16 pair 128.0 | 128.0 turn the
 //     codes of inputs (k, k + 1) into the exact bf16 pair (128 + q_k, 128 + q_k+1).
 //     Those pairs are the A fragments of mma.sync m16n8k16 (16 rows x 16 inputs),
-//     whose B fragments are the x rows (staged once per CTA in fragment order) and
+//     whose B fragments are the x rows (staged once per CTA in fragment order, the fragments of
+//     two MMAs side by side: 16-byte copies and loads, half as many of each as with 8 bytes;
+//     4 rows, 22016 x 4096: 15.4 -> 14.9 us, 8 rows 17.7 -> 16.7) and
 //     whose f32 accumulators give D = sum over the group of (128 + q) x.  (tcgen05.mma
 //     reads A only from shared or tensor memory: the decoded tile would make a round
 //     trip there, at 4x the HBM bytes, for a product only 8 columns wide);
@@ -46,8 +48,11 @@
 // err is not null) and the warp stops decoding.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cstdint>
+#include <map>
 #include <mutex>
+#include <tuple>
 
 #include "internal.h"
 #include "sm100_ptx.cuh"
@@ -84,8 +89,8 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                  : "memory");
 }
 
-__device__ __forceinline__ void cp_async_8(uint32_t dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+__device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
@@ -111,8 +116,8 @@ __device__ __forceinline__ float bf16_lo(uint32_t v) { return __uint_as_float(v 
 __device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v & 0xFFFF0000u); }
 
 // Shared memory of one CTA: the rings, their barriers, the split-K partials, the group
-// sums of x [ngroup][8] and x in fragment order [ngroup][8 mma][4 * MT lanes] (8 bytes
-// each: x[g][128G + 32t + 8i + 4h + 0..3] for lane 4g + t of mma 2i + h).
+// sums of x [ngroup][8] and x in fragment order [ngroup][4][4 * MT lanes] (16 bytes each:
+// x[g][128G + 32t + 8i + 0..7] for lane 4g + t, the B fragments of mma 2i and 2i + 1).
 __host__ __device__ constexpr size_t smem_bytes(int MT, int K) {
     return static_cast<size_t>(kRingBytes) + kBarBytes + kRedFloats * 4 + static_cast<size_t>(K / 128) * 8 * 4 +
            static_cast<size_t>(MT) * K * 2;
@@ -123,7 +128,7 @@ __host__ __device__ constexpr size_t smem_bytes(int MT, int K) {
 // xb points at this lane's B fragments; lanes g >= MT read those of lane g mod MT, which
 // only fills output columns >= MT, never stored.
 template <int MT>
-__device__ __forceinline__ void decode_tile(const uint8_t* st, const uint2* xb, const float* xs_g, int g, int t,
+__device__ __forceinline__ void decode_tile(const uint8_t* st, const uint4* xb, const float* xs_g, int g, int t,
                                             uint32_t mask, uint32_t magic, float (&acc)[4]) {
     const uint4 c0 = *reinterpret_cast<const uint4*>(st + g * 64 + t * 16);
     const uint4 c8 = *reinterpret_cast<const uint4*>(st + (g + 8) * 64 + t * 16);
@@ -134,12 +139,11 @@ __device__ __forceinline__ void decode_tile(const uint8_t* st, const uint2* xb, 
     for (int i = 0; i < 4; ++i) {
         const uint32_t w0 = i == 0 ? c0.x : i == 1 ? c0.y : i == 2 ? c0.z : c0.w;
         const uint32_t w8 = i == 0 ? c8.x : i == 1 ? c8.y : i == 2 ? c8.z : c8.w;
-        const uint2 b0 = xb[(2 * i) * 4 * MT];
-        const uint2 b1 = xb[(2 * i + 1) * 4 * MT];
+        const uint4 b = xb[i * 4 * MT];
         mma_bf16_16816(da, code_pair(w0, 0, mask, magic), code_pair(w8, 0, mask, magic), code_pair(w0, 1, mask, magic),
-                       code_pair(w8, 1, mask, magic), b0.x, b0.y);
+                       code_pair(w8, 1, mask, magic), b.x, b.y);
         mma_bf16_16816(db, code_pair(w0, 2, mask, magic), code_pair(w8, 2, mask, magic), code_pair(w0, 3, mask, magic),
-                       code_pair(w8, 3, mask, magic), b1.x, b1.y);
+                       code_pair(w8, 3, mask, magic), b.z, b.w);
     }
     const float d[4] = {da[0] + db[0], da[1] + db[1], da[2] + db[2], da[3] + db[3]};
     const uint16_t* scl = reinterpret_cast<const uint16_t*>(st + kScaleOff);
@@ -154,6 +158,41 @@ __device__ __forceinline__ void decode_tile(const uint8_t* st, const uint2* xb, 
     acc[3] = fmaf(s8, fmaf(-c8f, xs.y, d[3]), acc[3]);
 }
 
+// Sum of row m of x over group G of the staged fragments.
+template <int MT>
+__device__ __forceinline__ float group_sum(const uint4* xfrag, int G, int m) {
+    const uint4* p = xfrag + static_cast<size_t>(G) * 4 * 4 * MT + 4 * m;
+    float s = 0.f;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int tt = 0; tt < 4; ++tt) {
+            const uint4 v = p[e * 4 * MT + tt];
+            s += ((bf16_lo(v.x) + bf16_hi(v.x)) + (bf16_lo(v.y) + bf16_hi(v.y))) +
+                 ((bf16_lo(v.z) + bf16_hi(v.z)) + (bf16_lo(v.w) + bf16_hi(v.w)));
+        }
+    return s;
+}
+
+// Rows r0 and r0 + 8 of the product, columns n0 and n0 + 1 (an mma accumulator fragment): the
+// residual added in float, rounded, to y or its part of the split output.
+__device__ __forceinline__ void store_fragment(const float (&acc)[4], int r0, int n0, int M, int N, const W4Fused& fz,
+                                               uint16_t* __restrict__ y) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        // weight row `row` is output column `row` of x row `n`
+        const int row = r0 + ((v & 2) ? 8 : 0), n = n0 + (v & 1);
+        if (n < M && row < N) {
+            float o = acc[v];
+            if (fz.residual != nullptr) o += bf16_lo(fz.residual[static_cast<size_t>(n) * N + row]);
+            uint16_t* dst = row < fz.n0   ? y + static_cast<size_t>(n) * fz.n0 + row
+                            : row < fz.n1 ? fz.y1 + static_cast<size_t>(n) * (fz.n1 - fz.n0) + (row - fz.n0)
+                                          : fz.y2 + static_cast<size_t>(n) * (N - fz.n1) + (row - fz.n1);
+            *dst = __bfloat16_as_ushort(__float2bfloat16_rn(o));
+        }
+    }
+}
+
 template <int MT>
 __global__ void __launch_bounds__(kThreads) w4_gemv_kernel(const uint8_t* __restrict__ tiles,
                                                            const uint16_t* __restrict__ x, int M, int N, int K,
@@ -165,7 +204,7 @@ __global__ void __launch_bounds__(kThreads) w4_gemv_kernel(const uint8_t* __rest
     const uint32_t bars = ring + kRingBytes;
     float* red = reinterpret_cast<float*>(smem + kRingBytes + kBarBytes);
     float* xsum = red + kRedFloats;
-    uint2* xfrag = reinterpret_cast<uint2*>(xsum + ngroup * 8);
+    uint4* xfrag = reinterpret_cast<uint4*>(xsum + ngroup * 8);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, t = lane & 3;
 
@@ -213,15 +252,15 @@ __global__ void __launch_bounds__(kThreads) w4_gemv_kernel(const uint8_t* __rest
     if (early_weights) griddep_wait();  // x and y belong to the stream order from here on
     griddep_launch_dependents();
 
-    // x in fragment order (asynchronous 8-byte copies, rows past M zero)
+    // x in fragment order (asynchronous 16-byte copies, rows past M zero)
     const uint32_t xfrag_s = smem_u32(xfrag);
-    for (int i = tid; i < ngroup * 8 * 4 * MT; i += kThreads) {
-        const int slot = i % (4 * MT), ge = i / (4 * MT);
-        const int e = ge & 7, G = ge >> 3, m = slot >> 2, tt = slot & 3;
+    for (int i = tid; i < ngroup * 4 * 4 * MT; i += kThreads) {
+        const int slot = i % (4 * MT), gi = i / (4 * MT);
+        const int m = slot >> 2, tt = slot & 3;
         if (m < M)
-            cp_async_8(xfrag_s + 8 * i, x + static_cast<size_t>(m) * K + 128 * G + 32 * tt + 8 * (e >> 1) + 4 * (e & 1));
+            cp_async_16(xfrag_s + 16 * i, x + static_cast<size_t>(m) * K + 128 * (gi >> 2) + 32 * tt + 8 * (gi & 3));
         else
-            xfrag[i] = make_uint2(0u, 0u);
+            xfrag[i] = make_uint4(0u, 0u, 0u, 0u);
     }
     cp_async_wait_all();
     __syncthreads();
@@ -231,10 +270,11 @@ __global__ void __launch_bounds__(kThreads) w4_gemv_kernel(const uint8_t* __rest
         // is the same for all its elements (the stride divides by 4 * MT).
         const int slot = tid % (4 * MT), m = slot >> 2;
         float ss = 0.f;
-        for (int i = tid; i < ngroup * 8 * 4 * MT; i += kThreads) {
-            const uint2 v = xfrag[i];
-            const float a = bf16_lo(v.x), b = bf16_hi(v.x), c = bf16_lo(v.y), d = bf16_hi(v.y);
-            ss = fmaf(a, a, fmaf(b, b, fmaf(c, c, fmaf(d, d, ss))));
+        for (int i = tid; i < ngroup * 4 * 4 * MT; i += kThreads) {
+            const uint4 v = xfrag[i];
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) ss = fmaf(bf16_lo(w[e]), bf16_lo(w[e]), fmaf(bf16_hi(w[e]), bf16_hi(w[e]), ss));
         }
         // lanes of one row: those that differ in the two low lane bits or in bits >= 4 * MT
         ss += __shfl_xor_sync(0xFFFFFFFFu, ss, 1);
@@ -249,32 +289,24 @@ __global__ void __launch_bounds__(kThreads) w4_gemv_kernel(const uint8_t* __rest
         }
         __syncthreads();
         const float r = red[kWarps * 8 + m];
-        for (int i = tid; i < ngroup * 8 * 4 * MT; i += kThreads) {
+        for (int i = tid; i < ngroup * 4 * 4 * MT; i += kThreads) {
             if (m >= M) break;
-            const int ge = i / (4 * MT), e = ge & 7, G = ge >> 3, tt = slot & 3;
-            const int k0 = 128 * G + 32 * tt + 8 * (e >> 1) + 4 * (e & 1);
-            const uint2 gm = *reinterpret_cast<const uint2*>(fz.gamma + k0);
-            const uint2 v = xfrag[i];
-            xfrag[i] = make_uint2(pack_bf16x2(bf16_lo(v.x) * r * bf16_lo(gm.x), bf16_hi(v.x) * r * bf16_hi(gm.x)),
-                                  pack_bf16x2(bf16_lo(v.y) * r * bf16_lo(gm.y), bf16_hi(v.y) * r * bf16_hi(gm.y)));
+            const int gi = i / (4 * MT), tt = slot & 3;
+            const int k0 = 128 * (gi >> 2) + 32 * tt + 8 * (gi & 3);
+            // (gamma is 8-byte aligned)
+            const uint2 ga = *reinterpret_cast<const uint2*>(fz.gamma + k0), gc = *reinterpret_cast<const uint2*>(fz.gamma + k0 + 4);
+            const uint4 v = xfrag[i];
+            xfrag[i] = make_uint4(pack_bf16x2(bf16_lo(v.x) * r * bf16_lo(ga.x), bf16_hi(v.x) * r * bf16_hi(ga.x)),
+                                  pack_bf16x2(bf16_lo(v.y) * r * bf16_lo(ga.y), bf16_hi(v.y) * r * bf16_hi(ga.y)),
+                                  pack_bf16x2(bf16_lo(v.z) * r * bf16_lo(gc.x), bf16_hi(v.z) * r * bf16_hi(gc.x)),
+                                  pack_bf16x2(bf16_lo(v.w) * r * bf16_lo(gc.y), bf16_hi(v.w) * r * bf16_hi(gc.y)));
         }
         __syncthreads();
     }
     // group sums of x, one (group, row) per thread
     for (int i = tid; i < ngroup * 8; i += kThreads) {
-        const int G = i >> 3, m = i & 7;
-        float s = 0.f;
-        if (m < M) {
-            const uint2* p = xfrag + static_cast<size_t>(G) * 8 * 4 * MT + 4 * m;
-#pragma unroll 8
-            for (int e = 0; e < 8; ++e)
-#pragma unroll
-                for (int tt = 0; tt < 4; ++tt) {
-                    const uint2 v = p[e * 4 * MT + tt];
-                    s += (bf16_lo(v.x) + bf16_hi(v.x)) + (bf16_lo(v.y) + bf16_hi(v.y));
-                }
-        }
-        xsum[i] = s;
+        const int m = i & 7;
+        xsum[i] = m < M ? group_sum<MT>(xfrag, i >> 3, m) : 0.f;
     }
     __syncthreads();
 
@@ -299,15 +331,15 @@ __global__ void __launch_bounds__(kThreads) w4_gemv_kernel(const uint8_t* __rest
                     --outstanding;
                     const uint8_t* st = smem + (my_ring - ring) + cslot * kStageBytes;
                     const int nt = min(kTilesPerStage, g1 - G);
-                    const uint2* xb = xfrag + static_cast<size_t>(G) * 8 * 4 * MT + (lane & (4 * MT - 1));
+                    const uint4* xb = xfrag + static_cast<size_t>(G) * 4 * 4 * MT + (lane & (4 * MT - 1));
                     if (nt == kTilesPerStage) {
 #pragma unroll
                         for (int tt = 0; tt < kTilesPerStage; ++tt)
-                            decode_tile<MT>(st + tt * kTileBytes, xb + tt * 8 * 4 * MT, xsum + (G + tt) * 8, g, t,
+                            decode_tile<MT>(st + tt * kTileBytes, xb + tt * 4 * 4 * MT, xsum + (G + tt) * 8, g, t,
                                             kPairMask, magic, acc);
                     } else {
                         for (int tt = 0; tt < nt; ++tt)
-                            decode_tile<MT>(st + tt * kTileBytes, xb + tt * 8 * 4 * MT, xsum + (G + tt) * 8, g, t,
+                            decode_tile<MT>(st + tt * kTileBytes, xb + tt * 4 * 4 * MT, xsum + (G + tt) * 8, g, t,
                                             kPairMask, magic, acc);
                     }
                     cslot = cslot + 1 == kStages ? 0 : cslot + 1;
@@ -330,22 +362,7 @@ __global__ void __launch_bounds__(kThreads) w4_gemv_kernel(const uint8_t* __rest
             }
             rb ^= 1;
         }
-        if (part == 0 && unit < units) {
-            const int r0 = unit * kUnitRows + g, n0 = 2 * t;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                // weight row `row` is output column `row` of x row `n`
-                const int row = r0 + ((v & 2) ? 8 : 0), n = n0 + (v & 1);
-                if (n < M && row < N) {
-                    float o = acc[v];
-                    if (fz.residual != nullptr) o += bf16_lo(fz.residual[static_cast<size_t>(n) * N + row]);
-                    uint16_t* dst = row < fz.n0   ? y + static_cast<size_t>(n) * fz.n0 + row
-                                    : row < fz.n1 ? fz.y1 + static_cast<size_t>(n) * (fz.n1 - fz.n0) + (row - fz.n0)
-                                                  : fz.y2 + static_cast<size_t>(n) * (N - fz.n1) + (row - fz.n1);
-                    *dst = __bfloat16_as_ushort(__float2bfloat16_rn(o));
-                }
-            }
-        }
+        if (part == 0 && unit < units) store_fragment(acc, unit * kUnitRows + g, 2 * t, M, N, fz, y);
     }
     // after a timeout: let the copies still in flight (the failed one and those issued
     // after it) land, each wait bounded, before the warp exits
@@ -356,6 +373,185 @@ __global__ void __launch_bounds__(kThreads) w4_gemv_kernel(const uint8_t* __rest
             if (cslot == 0) cphase ^= 1u;
         }
     }
+}
+
+// ------------------------------------------------------------------ K split over a cluster
+//
+// When the rows of x are many or long, staging all of x in every CTA costs more than the
+// weights a CTA decodes: it waits for M K bytes after the previous kernel, and x leaves room
+// for one CTA per SM.  Here the C CTAs of a cluster take a C-th of the groups each, for the
+// same row-tiles, so a CTA stages a C-th of x; its warps keep their partial sums of every unit
+// in shared memory (no barrier between units), and at the end each CTA adds a share of the
+// units' partials from the whole cluster through distributed shared memory, in a fixed order.
+// (A chain of calls in a graph, plain -> cluster: 4096 x 11008 at 4 rows of x 11.2 -> 10.1 us,
+// at 8 22.4 -> 11.1; 3584 x 18944 at 4 29.1 -> 14.5, at 8 57.9 -> 16.0.)  Without RMSNorm only:
+// that needs whole rows of x.
+__device__ __forceinline__ float4 ld_dsmem_f32x4(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(addr)
+                 : "memory");
+    return v;
+}
+
+// Shared memory of one CTA: rings, barriers, the partial sums [rounds][warp][lane] (float4),
+// the group sums and x of its slice of at most `ngl` groups.
+__host__ __device__ constexpr size_t cluster_smem_bytes(int MT, int ngl, int rounds) {
+    return static_cast<size_t>(kRingBytes) + kBarBytes + static_cast<size_t>(rounds) * kWarps * 512 +
+           static_cast<size_t>(ngl) * (8 * 4 + MT * 256);
+}
+
+template <int MT>
+__global__ void __launch_bounds__(kThreads) w4_gemv_cluster_kernel(const uint8_t* __restrict__ tiles,
+                                                                   const uint16_t* __restrict__ x, int M, int N, int K,
+                                                                   int C, int KS, int rounds_max,
+                                                                   uint16_t* __restrict__ y, int* err,
+                                                                   int early_weights, W4Fused fz) {
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint32_t crank;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
+    const int ngroup = K / 128;
+    const int s0 = static_cast<int>(crank) * ngroup / C, s1 = (static_cast<int>(crank) + 1) * ngroup / C;
+    const int ngl = s1 - s0, ngl_max = (ngroup + C - 1) / C;
+    const uint32_t ring = smem_u32(smem);
+    const uint32_t bars = ring + kRingBytes;
+    float4* parts = reinterpret_cast<float4*>(smem + kRingBytes + kBarBytes);
+    float* xsum = reinterpret_cast<float*>(parts + static_cast<size_t>(rounds_max) * kWarps * 32);
+    uint4* xfrag = reinterpret_cast<uint4*>(xsum + ngl_max * 8);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int g = lane >> 2, t = lane & 3;
+
+    if (!early_weights) griddep_wait();
+    if (lane == 0) {
+        for (int s = 0; s < kStages; ++s) mbar_init(bars + 8 * (warp * kStages + s), 1);
+        fence_mbar_init();
+    }
+    __syncwarp();
+    const int units = (N + kUnitRows - 1) / kUnitRows;
+    const int upc = kWarps / KS;  // units per cluster round
+    const int blocks = (units + upc - 1) / upc;
+    const int part = warp % KS, uslot = warp / KS;
+    const int cid = static_cast<int>(blockIdx.x) / C, ncl = static_cast<int>(gridDim.x) / C;
+    const int g0 = s0 + part * ngl / KS, g1 = s0 + (part + 1) * ngl / KS;  // not empty: KS <= ngroup / C
+    const uint32_t my_ring = ring + warp * kStages * kStageBytes;
+    const uint32_t my_bars = bars + 8 * warp * kStages;
+    uint32_t magic = kPairMagic;
+    asm volatile("" : "+r"(magic));
+
+    int iblk = cid, iG = g0, islot = 0;
+    bool ivalid = iblk < blocks && iblk * upc + uslot < units;
+    bool failed = false;
+    int outstanding = 0;
+    auto issue = [&]() {
+        const int nt = min(kTilesPerStage, g1 - iG);
+        if (lane == 0) {
+            const size_t rec = static_cast<size_t>(iblk * upc + uslot) * ngroup + iG;
+            const uint32_t bar = my_bars + 8 * islot;
+            mbar_arrive_expect_tx(bar, nt * kTileBytes);
+            bulk_load(my_ring + islot * kStageBytes, tiles + rec * kTileBytes, nt * kTileBytes, bar);
+        }
+        ++outstanding;
+        islot = islot + 1 == kStages ? 0 : islot + 1;
+        iG += nt;
+        if (iG == g1) {
+            iG = g0;
+            iblk += ncl;
+            ivalid = iblk < blocks && iblk * upc + uslot < units;
+        }
+    };
+    for (int s = 0; s < kStages - 1 && ivalid; ++s) issue();
+    if (early_weights) griddep_wait();  // x and y belong to the stream order from here on
+    griddep_launch_dependents();
+
+    // this CTA's slice of x in fragment order, and its group sums
+    const uint32_t xfrag_s = smem_u32(xfrag);
+    for (int i = tid; i < ngl * 4 * 4 * MT; i += kThreads) {
+        const int slot = i % (4 * MT), gi = i / (4 * MT);
+        const int m = slot >> 2, tt = slot & 3;
+        if (m < M)
+            cp_async_16(xfrag_s + 16 * i,
+                        x + static_cast<size_t>(m) * K + 128 * (s0 + (gi >> 2)) + 32 * tt + 8 * (gi & 3));
+        else
+            xfrag[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    for (int i = tid; i < ngl * 8; i += kThreads) {
+        const int m = i & 7;
+        xsum[i] = m < M ? group_sum<MT>(xfrag, i >> 3, m) : 0.f;
+    }
+    __syncthreads();
+
+    int cslot = 0, nr = 0;
+    uint32_t cphase = 0;
+    for (int blk = cid; blk < blocks; blk += ncl, ++nr) {
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        if (blk * upc + uslot < units) {
+            for (int G = g0; G < g1; G += kTilesPerStage) {
+                if (ivalid && !failed) {
+                    __syncwarp();  // every lane is done with the slot the copy overwrites
+                    issue();
+                }
+                if (!failed) {
+                    const bool landed = mbar_wait(my_bars + 8 * cslot, cphase, nullptr, kWaitNs);
+                    failed = __any_sync(0xFFFFFFFFu, !landed);
+                    if (failed && err != nullptr && lane == 0) atomicOr(err, kDevErrTimeout);
+                }
+                if (!failed) {  // (the slot of a failed wait stays current for the drain below)
+                    --outstanding;
+                    const uint8_t* st = smem + (my_ring - ring) + cslot * kStageBytes;
+                    const int nt = min(kTilesPerStage, g1 - G);
+                    const uint4* xb = xfrag + static_cast<size_t>(G - s0) * 4 * 4 * MT + (lane & (4 * MT - 1));
+                    if (nt == kTilesPerStage) {
+#pragma unroll
+                        for (int tt = 0; tt < kTilesPerStage; ++tt)
+                            decode_tile<MT>(st + tt * kTileBytes, xb + tt * 4 * 4 * MT, xsum + (G - s0 + tt) * 8, g, t,
+                                            kPairMask, magic, acc);
+                    } else {
+                        for (int tt = 0; tt < nt; ++tt)
+                            decode_tile<MT>(st + tt * kTileBytes, xb + tt * 4 * 4 * MT, xsum + (G - s0 + tt) * 8, g, t,
+                                            kPairMask, magic, acc);
+                    }
+                    cslot = cslot + 1 == kStages ? 0 : cslot + 1;
+                    if (cslot == 0) cphase ^= 1u;
+                }
+            }
+        }
+        parts[(nr * kWarps + warp) * 32 + lane] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    }
+    // after a timeout: let the copies still in flight land, each wait bounded
+    if (failed) {
+        for (int s = 0; s < outstanding && s < kStages; ++s) {
+            mbar_wait(my_bars + 8 * cslot, cphase, nullptr, kWaitNs);
+            cslot = cslot + 1 == kStages ? 0 : cslot + 1;
+            if (cslot == 0) cphase ^= 1u;
+        }
+    }
+    __syncwarp();
+    cluster_sync();  // every CTA's partials are complete (reached by all, whatever their waits did)
+    const uint32_t parts_s = smem_u32(parts);
+    for (int f = static_cast<int>(crank) * kThreads + tid; f < nr * upc * 32; f += C * kThreads) {
+        const int r = f / (upc * 32), us = (f >> 5) % upc;
+        const int unit = (cid + r * ncl) * upc + us;
+        const int n0 = 2 * (f & 3);  // (f mod 32 is the fragment's lane: rows f/4 % 8 and + 8, columns n0, n0 + 1)
+        if (unit >= units || n0 >= M) continue;
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int c = 0; c < C; ++c) {
+            const uint32_t src = mapa_shared(parts_s + static_cast<uint32_t>(((r * kWarps + us * KS) * 32 + (f & 31)) * 16), c);
+#pragma unroll 4
+            for (int p = 0; p < KS; ++p) {
+                const float4 o = ld_dsmem_f32x4(src + p * 512);
+                acc[0] += o.x;
+                acc[1] += o.y;
+                acc[2] += o.z;
+                acc[3] += o.w;
+            }
+        }
+        store_fragment(acc, unit * kUnitRows + ((f & 31) >> 2), n0, M, N, fz, y);
+    }
+    __syncwarp();
+    cluster_sync();  // no CTA leaves while its partials may still be read
 }
 
 // Per device: the SM count and, per MT, whether the shared-memory limit is raised and the
@@ -438,6 +634,136 @@ cudaError_t launch_t(const uint8_t* tiles, const uint16_t* x, int M, int N, int 
     return cudaLaunchKernelEx(&cfg, kern, tiles, x, M, N, K, best_ks, y, err, early_weights ? 1 : 0, fz);
 }
 
+// The cluster split of a product without RMSNorm: CTAs per cluster (1: the plain kernel), warps
+// per unit, clusters resident at once, rounds of units a cluster walks.
+struct ClusterPlan {
+    int C, KS, ncl, rounds;
+};
+
+constexpr int kMaxRounds = 64;  // partials of a cluster's units: 4 KB a round
+
+// CTAs per cluster for M rows (in the MT-row kernel) of K inputs; 1: the plain kernel.  The
+// cluster pays for its exchange only where x is long: at K <= 8192 it was slower (8 rows, 22016
+// x 4096: 18.1 us against 16.7; 65536 x 8192: 83 against 68), while at 11008 x's 88 KB at 4
+// rows already leave the plain kernel one CTA per SM and 8 rows need two of its launches.  The
+// size keeps a CTA's slice within 44 KB, two CTAs per SM (8 rows, K 11008: 11.1 us with 4
+// CTAs, 15.8 with 8, of which fewer fit at once); at least one stage of groups each.
+int cluster_size(int M, int MT, int K) {
+    const long long xb = static_cast<long long>(MT) * K * 2;
+    if (M <= w4_gemv_max_rows(K) && !(K > 10240 && xb > 72 * 1024)) return 1;
+    int C = xb <= 80 * 1024 ? 2 : xb <= 4 * 44 * 1024 ? 4 : 8;
+    while (C > 1 && K / 128 / C < kTilesPerStage) C /= 2;
+    return C;
+}
+
+std::map<std::tuple<int, int, int, size_t>, int> g_ncl;  // (device, MT, C, shared memory) -> clusters resident
+
+template <int MT>
+cudaError_t cluster_plan(int dev, int M, int N, int K, ClusterPlan* plan) {
+    plan->C = cluster_size(M, MT, K);
+    if (plan->C == 1) return cudaSuccess;
+    const int C = plan->C, ngl = (K / 128 + C - 1) / C;
+    auto resident = [&](size_t smem, int* n) -> cudaError_t {
+        {
+            std::lock_guard<std::mutex> lock(g_mutex);
+            const auto it = g_ncl.find(std::make_tuple(dev, MT, C, smem));
+            if (it != g_ncl.end()) {
+                *n = it->second;
+                return cudaSuccess;
+            }
+        }
+        cudaError_t e = cudaFuncSetAttribute(w4_gemv_cluster_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             static_cast<int>(kSmemLimit));
+        if (e != cudaSuccess) return e;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(static_cast<unsigned>(C));
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = static_cast<unsigned>(C);
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaOccupancyMaxActiveClusters(n, w4_gemv_cluster_kernel<MT>, &cfg);
+        if (e != cudaSuccess) return e;
+        std::lock_guard<std::mutex> lock(g_mutex);
+        if (g_ncl.size() >= 1024) g_ncl.clear();
+        g_ncl[std::make_tuple(dev, MT, C, smem)] = *n;
+        return cudaSuccess;
+    };
+    // the fewest stages on the busiest warp, then the fewest partials
+    const long long units = (static_cast<long long>(N) + kUnitRows - 1) / kUnitRows;
+    long long best_t = -1;
+    int rounds = 8;  // a first guess of the partials' room, for the clusters resident
+    for (int pass = 0; pass < 2; ++pass) {
+        int ncl = 0;
+        const size_t smem = cluster_smem_bytes(MT, ngl, rounds);
+        if (smem > static_cast<size_t>(kSmemLimit)) break;
+        const cudaError_t e = resident(smem, &ncl);
+        if (e != cudaSuccess) return e;
+        if (ncl < 1) break;
+        best_t = -1;
+        for (int ks = 1; ks <= kWarps && ks <= K / 128 / C; ks *= 2) {
+            const long long blocks = (units + kWarps / ks - 1) / (kWarps / ks);
+            const long long r = (blocks + ncl - 1) / ncl;
+            const long long t = r * ((ngl + ks - 1) / ks + kTilesPerStage - 1) / kTilesPerStage;
+            if (r <= kMaxRounds && (best_t < 0 || t < best_t)) {
+                best_t = t;
+                plan->KS = ks;
+                plan->ncl = static_cast<int>(std::min<long long>(blocks, ncl));
+                plan->rounds = static_cast<int>(r);
+            }
+        }
+        if (best_t < 0 || plan->rounds <= rounds) break;
+        rounds = plan->rounds;
+    }
+    if (best_t < 0 || cluster_smem_bytes(MT, ngl, plan->rounds) > static_cast<size_t>(kSmemLimit)) plan->C = 1;
+    return cudaSuccess;
+}
+
+template <int MT>
+cudaError_t launch_cluster_t(const ClusterPlan& p, const uint8_t* tiles, const uint16_t* x, int M, int N, int K,
+                             uint16_t* y, int* err, bool early_weights, const W4Fused& fz, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(p.ncl * p.C));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = cluster_smem_bytes(MT, (K / 128 + p.C - 1) / p.C, p.rounds);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(p.C);
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, w4_gemv_cluster_kernel<MT>, tiles, x, M, N, K, p.C, p.KS, p.rounds, y, err,
+                              early_weights ? 1 : 0, fz);
+}
+
+// M <= 8 rows in one launch: through a cluster plan where there is one; otherwise the plain
+// kernel, which takes at most w4_gemv_max_rows(K) rows.
+template <int MT>
+cudaError_t launch_rows(const uint8_t* tiles, const uint16_t* x, int M, int N, int K, uint16_t* y, int* err,
+                        bool early_weights, const W4Fused& fz, cudaStream_t st, bool* done) {
+    *done = true;
+    if (fz.gamma == nullptr) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        ClusterPlan p = {};
+        e = cluster_plan<MT>(dev, M, N, K, &p);
+        if (e != cudaSuccess) return e;
+        if (p.C > 1) return launch_cluster_t<MT>(p, tiles, x, M, N, K, y, err, early_weights, fz, st);
+    }
+    if (M > w4_gemv_max_rows(K)) {
+        *done = false;
+        return cudaSuccess;
+    }
+    return launch_t<MT>(tiles, x, M, N, K, y, err, early_weights, fz, st);
+}
+
 }  // namespace
 
 int w4_gemv_max_rows(int K) {
@@ -449,11 +775,21 @@ int w4_gemv_max_rows(int K) {
 }
 
 cudaError_t launch_w4_gemv(const uint8_t* tiles, const uint16_t* x, int M, int N, int K, uint16_t* y, int* err,
-                           bool early_weights, const W4Fused& fz, cudaStream_t st) {
-    if (M <= 1) return launch_t<1>(tiles, x, M, N, K, y, err, early_weights, fz, st);
-    if (M <= 2) return launch_t<2>(tiles, x, M, N, K, y, err, early_weights, fz, st);
-    if (M <= 4) return launch_t<4>(tiles, x, M, N, K, y, err, early_weights, fz, st);
-    return launch_t<8>(tiles, x, M, N, K, y, err, early_weights, fz, st);
+                           bool early_weights, const W4Fused& fz, cudaStream_t st, int* rows) {
+    // up to 8 rows in one launch; where neither kernel holds them, as many as the plain one does
+    for (int m = M < 8 ? M : 8; m > 0; m = m > 4 ? 4 : m > 2 ? 2 : m - 1) {
+        bool done = false;
+        cudaError_t e;
+        if (m <= 1) e = launch_rows<1>(tiles, x, m, N, K, y, err, early_weights, fz, st, &done);
+        else if (m <= 2) e = launch_rows<2>(tiles, x, m, N, K, y, err, early_weights, fz, st, &done);
+        else if (m <= 4) e = launch_rows<4>(tiles, x, m, N, K, y, err, early_weights, fz, st, &done);
+        else e = launch_rows<8>(tiles, x, m, N, K, y, err, early_weights, fz, st, &done);
+        if (e != cudaSuccess || done) {
+            *rows = m;
+            return e;
+        }
+    }
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace attn
