@@ -22,7 +22,7 @@
 // decoding and four barrier operations per sixteen MMAs, took 183 us on 4096 x 6144 x 4096;
 // this takes 115 us, 22016 features 392 instead of 588.)  Few tokens leave most SMs idle, so K
 // is then split over the pairs of a cluster, which add their f32 partials through distributed
-// shared memory (32 tokens x 4096 x 4096: 10.3 us, 24.6 before).
+// shared memory (32 tokens x 4096 x 4096: 9 us, 24.6 before).
 //
 // Clusters of 2 S CTAs (S = split of K) walk output tiles, token tiles fastest.  Per CTA, 576
 // threads:
@@ -305,46 +305,51 @@ __global__ void __launch_bounds__(kThreads, 1) w4_gemm_kernel(const __grid_const
                 wait_full(bar(B_FULL0 + g % kStages), (g / kStages) & 1u, nullptr);
         }
     } else if (warp == kWarpMma) {
-        if (lane == 0 && half == 0) {
+        if (half == 0) {
+            // The whole warp runs the loop and one elected lane issues: the loop's values stay in
+            // uniform registers, which the MMA takes its operands from.  (Issued inside a branch
+            // of one lane, each of the eight MMAs of a group first moved its operands there: a
+            // group of 32 tokens took 0.40 us instead of 0.28, of 128 0.40 instead of 0.35.)
             const uint32_t idesc = idesc_bf16_f32(256, nt, false, false);
             constexpr uint32_t kHi = desc_hi_sw128(1024);
             const uint32_t x_lo0 = desc_lo_sw128(base + L::OFF_X, 16);
+            const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem, 0);
             const uint16_t mask = static_cast<uint16_t>(3u << (rank & ~1u));  // both CTAs of the pair
             uint32_t gs = 0;
             int tiles_done = 0;
             bool ok = true;
             for (int u = u0; u < n_units && ok; u += ustep, ++tiles_done) {
                 // the accumulator is free once the epilogue has read the previous tile's
-                if (tiles_done > 0 &&
-                    !wait_full(bar(B_ACCEMPTY), static_cast<uint32_t>(tiles_done - 1) & 1u, abort_flag)) {
-                    ok = false;
-                    break;
-                }
+                if (tiles_done > 0)
+                    ok = __all_sync(0xFFFFFFFFu,
+                                    wait_full(bar(B_ACCEMPTY), static_cast<uint32_t>(tiles_done - 1) & 1u, abort_flag));
+                if (!ok) break;
                 for (int G = g0; G < g1; ++G, ++gs) {
                     const int s = static_cast<int>(gs % kStages);
-                    if (!wait_full(bar(B_AFULL0 + s), (gs / kStages) & 1u, abort_flag)) {
-                        ok = false;
-                        break;
-                    }
+                    ok = __all_sync(0xFFFFFFFFu, wait_full(bar(B_AFULL0 + s), (gs / kStages) & 1u, abort_flag));
+                    if (!ok) break;
                     tc_fence_after();
                     const uint32_t xa = x_lo0 + ((s * kXStage) >> 4);
-                    const uint32_t a_col = tmem + kTmA + 64u * s, d_col = tmem + kTmAcc;
+                    const uint32_t a_col = tm + kTmA + 64u * s, d_col = tm + kTmAcc;
+                    if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) {
-                        const uint32_t c = ((kk >> 2) * kChunk + (kk & 3) * 32) >> 4;
-                        umma2_ts_w(d_col, a_col + 8u * kk, xa + c, kHi, idesc, (G > g0 || kk > 0) ? 1u : 0u);
+                        for (int kk = 0; kk < 8; ++kk) {
+                            const uint32_t c = ((kk >> 2) * kChunk + (kk & 3) * 32) >> 4;
+                            umma2_ts_w(d_col, a_col + 8u * kk, xa + c, kHi, idesc, (G > g0 || kk > 0) ? 1u : 0u);
+                        }
+                        umma2_commit_mc(bar(B_EMPTY0 + s), mask);
+                        if (G + 1 == g1) umma2_commit_mc(bar(B_ACCFULL), mask);  // the tile's products
                     }
-                    umma2_commit_mc(bar(B_EMPTY0 + s), mask);
+                    __syncwarp();
                 }
-                if (!ok) break;
-                umma2_commit_mc(bar(B_ACCFULL), mask);  // the tile's products are complete
             }
-            if (!ok) {
+            if (!ok && lane == 0) {
                 *abort_flag = 1;
                 atomicOr(err, kDevErrTimeout);
             }
             // also after an abort: the MMAs issued so far complete on it
-            umma2_commit_mc(bar(B_DRAIN), static_cast<uint16_t>(1u << rank));
+            if (elect_one()) umma2_commit_mc(bar(B_DRAIN), static_cast<uint16_t>(1u << rank));
+            __syncwarp();
             wait_full(bar(B_DRAIN), 0u, nullptr);
         }
     } else if (warp < kWarpEpi0) {
@@ -608,11 +613,12 @@ struct Plan {
 
 // The cheapest plan by a model of the busiest cluster, in microseconds as measured on a GB300
 // (calls one after another; K = 2048, 4096 and 11008, N = 3072 .. 22016, every nt and split):
-// a 128-input group costs its MMAs (0.526 at nt = 256) and at least the issuing thread's wait,
-// eight MMAs and commit (0.40: nt <= 192 all run K = 4096 in 17.4-18.3); a further tile of a
-// pair 1.4; a launch 4.6; a split its cluster barriers and the exchange of its partials.
-// What it weighs up, T x N at K = 4096: 8 x 6144 split 2 11.5, whole 17.4; 256 x 4096 128
-// tokens split 2 13.8, 256 whole 22.5; 1024 x 6144 in tiles of 192 33.3, of 256 41.2.
+// a 128-input group costs its MMAs (0.526 at nt = 256) and at least the chain of the issuing
+// warp (0.28 at nt = 32, 0.35 at 128); a further tile of a pair 1.4; a launch 4.7; a split its
+// cluster barriers and the exchange of its partials.
+// What it weighs up, T x N at K = 4096: 8 x 6144 split 2 9.7, whole 13.6; 256 x 4096 128
+// tokens split 2 12.8, 256 whole 22.6; 500 x 4096 in tiles of 128 17.1, of 256 22.8;
+// 1024 x 6144 in tiles of 192 32.9, of 256 41.2.
 Plan make_plan(int T, int N, int K, const int* clusters) {
     const int ngroup = K / 128, ft = (N + kBF - 1) / kBF;
     Plan best = {};
@@ -626,8 +632,8 @@ Plan make_plan(int T, int N, int K, const int* clusters) {
             const long long rounds = (units + clusters[split] - 1) / clusters[split];
             // (narrower tiles only while they fill idle SMs; a split only where SMs are idle)
             if ((n_tt > n_tt0 && rounds > 1 && nt < 64) || units > (split > 1 ? 4096 : 1LL << 29)) break;
-            const double group = std::max(0.526 * nt / kMaxNt, 0.40) * ((ngroup + split - 1) / split);
-            const double c = split == 1 ? 4.6 + rounds * group + (rounds - 1) * 1.4
+            const double group = std::max(0.526 * nt / kMaxNt, 0.265 + 0.00067 * nt) * ((ngroup + split - 1) / split);
+            const double c = split == 1 ? 4.7 + rounds * group + (rounds - 1) * 1.4
                                         : rounds * (group + 5.2 + 0.022 * (nt - 32));
             if (c < best_c * 0.999) {
                 best_c = c;
