@@ -536,7 +536,11 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
         }
         constexpr uint32_t kIdQK = idesc_bf16_f32(KT, NH, false, false);
         constexpr uint32_t kIdPV = idesc_bf16_f32(D, NH, true, false);
-        const uint32_t sQ = base + L::OFF_Q;
+        // The warp stays converged and one elected lane issues: the loop's values then live in
+        // uniform registers, where the MMA takes its operands from.
+        constexpr uint32_t kHi = desc_hi_sw128(1024);
+        const uint32_t q_lo = desc_lo_sw128(base + L::OFF_Q, 16);
+        const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem, 0);
         auto wait_all = [&](int barrier, uint32_t parity) -> bool {
             return __all_sync(0xFFFFFFFFu, mbar_wait(bar(barrier), parity, abort_flag, wait_ns));
         };
@@ -559,14 +563,15 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                 fence_proxy_async_smem();
             }
             __syncwarp();
-            if (lane == 0) {
-                tc_fence_after();
-                const uint32_t sP = base + L::OFF_P + (jj & 1) * (2 * NH * 128);
+            tc_fence_after();
+            const uint32_t v_lo = desc_lo_sw128(sV, L::BOX);
+            const uint32_t p_lo = desc_lo_sw128(base + L::OFF_P + (jj & 1) * (2 * NH * 128), 16);
+            if (elect_one()) {
 #pragma unroll
                 for (int kk = 0; kk < KT / 16; ++kk)
-                    umma_ss(tmem + TM_O, smem_desc_sw128(sV + kk * 16 * 128, L::BOX, 1024),
-                            smem_desc_sw128(sP + (kk >> 2) * NH * 128 + (kk & 3) * 32, 16, 1024), kIdPV,
-                            (jj > 0 || kk > 0) ? 1u : 0u);
+                    umma_ss_w(tm + TM_O, v_lo + ((kk * 16 * 128) >> 4), kHi,
+                              p_lo + (((kk >> 2) * NH * 128 + (kk & 3) * 32) >> 4), kHi, kIdPV,
+                              (jj > 0 || kk > 0) ? 1u : 0u);
                 umma_commit(bar(B_PVDONE));
                 umma_commit(bar(B_VEMPTY0 + jj % VST));
             }
@@ -602,15 +607,13 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                     fence_proxy_async_smem();
                 }
                 __syncwarp();
-                if (lane == 0) {
-                    tc_fence_after();
+                tc_fence_after();
+                const uint32_t k_lo = desc_lo_sw128(sK, 16);
+                if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk) {
-                        const uint32_t off = (kk >> 2) * L::BOX + (kk & 3) * 32;
-                        umma_ss(tmem + (j & 1) * NH, smem_desc_sw128(sK + off, 16, 1024),
-                                smem_desc_sw128(sQ + (kk >> 2) * NH * 128 + (kk & 3) * 32, 16, 1024), kIdQK,
-                                kk > 0 ? 1u : 0u);
-                    }
+                    for (int kk = 0; kk < D / 16; ++kk)
+                        umma_ss_w(tm + (j & 1) * NH, k_lo + (((kk >> 2) * L::BOX + (kk & 3) * 32) >> 4), kHi,
+                                  q_lo + (((kk >> 2) * NH * 128 + (kk & 3) * 32) >> 4), kHi, kIdQK, kk > 0 ? 1u : 0u);
                     umma_commit(bar(B_SFULL0 + (j & 1)));
                     umma_commit(bar(B_KEMPTY0 + ks));  // K is consumed once S^T(j) completes
                 }
@@ -625,18 +628,17 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                 // completes without an MMA (S(n-2) on that buffer was consumed: PFULL(n-2) seen)
                 if (lane == 0) mbar_arrive(bar(B_SFULL0 + (n & 1)));
                 if (n > 0) ok = issue_pv(n - 1);
-                if (ok && n > 0 && lane == 0) umma_commit(bar(B_OFULL));  // every PV is complete
+                if (ok && n > 0 && elect_one()) umma_commit(bar(B_OFULL));  // every PV is complete
             }
         }
         if (!ok && lane == 0) {
             *abort_flag = 1;
             atomicOr(err, kDevErrTimeout);
         }
-        if (lane == 0) {
-            umma_commit(bar(B_DRAIN));
-            mbar_wait(bar(B_DRAIN), 0, nullptr);
-        }
         __syncwarp();
+        if (elect_one()) umma_commit(bar(B_DRAIN));
+        __syncwarp();
+        mbar_wait(bar(B_DRAIN), 0, nullptr);
     } else {
         // ------------------------------------------------------------ softmax / epilogue (one thread per key)
         const int t = tid;  // key row of a tile; output dimension in the epilogue
