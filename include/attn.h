@@ -228,9 +228,9 @@ int attn_set_wait_limit(attn_ctx* ctx, long long limit_ns);
  *   ATTN_KERNEL_ROPE_APPEND     RoPE of the new keys + in-place cache append (every stage)
  *   ATTN_KERNEL_FLASH_FWD       causal flash attention (prefill, prefill_kv), with the
  *                               merge kernel of its split tail when it runs one
- *   ATTN_KERNEL_DECODE_SPLIT    split-KV decode (decode); with head_dim 128 it also
- *                               merges the splits and writes out itself
- *   ATTN_KERNEL_DECODE_COMBINE  log-sum-exp merge of the partials (decode, head_dim 64)
+ *   ATTN_KERNEL_DECODE_SPLIT    split-KV decode (decode); it also merges the splits and
+ *                               writes out itself
+ *   ATTN_KERNEL_DECODE_COMBINE  no kernel of this version (the merge is part of the decode)
  * (ATTN_KERNEL_FLASH_FWD also covers the small merge kernel that follows it when
  * the last round of its work is split across CTAs; both count as launches.)
  * attn_timing_enable(ctx, n) creates n pairs of CUDA events (blocking, the only
@@ -267,8 +267,8 @@ int attn_timing_read(attn_ctx* ctx, double* ms, long long* launches);
  *     back (it receives the ATTN_DEVERR_* bits, as attn_device_error reports);
  *   - the split-KV partials live in a static device array of
  *     ATTN_NOALLOC_SCRATCH_FLOATS floats (4 MiB) that every GPU which loads this
- *     library holds until the process exits, beside 40961 int counters
- *     (160 KiB).  Shapes whose partials do not fit even with one split
+ *     library holds until the process exits, beside 81921 int counters
+ *     (320 KiB).  Shapes whose partials do not fit even with one split
  *     (batch * n_q_heads * (head_dim + 2) > that size) are rejected with
  *     ATTN_EINVAL; larger ones use fewer splits.
  * All calls share those arrays.  Nothing in the partials has to start at zero

@@ -18,10 +18,9 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libattn_gb300.so")
 # (source, object name, extra nvcc flags)
-SOURCES = [("attn_api.cu", "attn_api", []), ("rope_append.cu", "rope_append", []), ("decode.cu", "decode", []),
+SOURCES = [("attn_api.cu", "attn_api", []), ("rope_append.cu", "rope_append", []),
            ("decode_tc.cu", "decode_tc", []), ("flash_fwd.cu", "flash_fwd", []),
-           ("decode_noalloc.cu", "decode_noalloc", []), ("w4_gemv.cu", "w4_gemv", []),
-           ("w4_gemm.cu", "w4_gemm", [])]
+           ("decode_noalloc.cu", "decode_noalloc", []), ("w4_gemv.cu", "w4_gemv", []), ("w4_gemm.cu", "w4_gemm", [])]
 HEADERS = ["internal.h", "sm100_ptx.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

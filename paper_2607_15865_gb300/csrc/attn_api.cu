@@ -5,9 +5,8 @@
 // the kernels of each stage on the caller's stream:
 //   prefill / prefill_kv : K1 rope_append (new k rotated + k, v appended in place)
 //                          -> K2 flash_fwd (q rotated in-kernel, causal attention)
-//   decode               : K3 (new k rotated + k, v appended at slot hist_len[b], read on
-//                          the device): decode_tc for head_dim 128, decode_split -> K4
-//                          decode_combine for head_dim 64
+//   decode               : K3 decode_tc (new k rotated + k, v appended at slot hist_len[b],
+//                          read on the device; the merge of the splits fused in)
 // No call allocates, frees or synchronises except attn_create/attn_destroy and
 // attn_device_error.
 #include <cuda.h>
@@ -222,7 +221,6 @@ int attn_create(const attn_cfg* cfg, attn_ctx** out) {
     }
     c->encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
     e = attn::configure_flash_fwd();
-    if (e == cudaSuccess) e = attn::configure_decode();
     if (e == cudaSuccess) e = attn::configure_decode_tc();
     if (e != cudaSuccess) {
         delete c;
@@ -327,7 +325,7 @@ namespace {
 // after_decode: the previous launch on `st` was this context's decode of the same caches
 // (a decode loop).
 // producer_early: the previous launch wrote q, k and v and nothing the decode streams (the
-// fused QKV GEMV of attn_decode_layer); the head_dim 128 decode then starts its K/V stream as
+// fused QKV GEMV of attn_decode_layer); the decode then starts its K/V stream as
 // a dependent launch before that kernel has finished.
 // seq_tok (head_dim 64): q, k, v and out point into arrays of seq_tok tokens per sequence (0: ntok).
 int run_decode(attn_ctx* c, const uint16_t* q, const uint16_t* k, const uint16_t* v, const int32_t* d_hist_len,
@@ -339,10 +337,8 @@ int run_decode(attn_ctx* c, const uint16_t* q, const uint16_t* k, const uint16_t
     if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(k_cache) || !aligned16(v_cache) ||
         !aligned16(out) || (reinterpret_cast<uintptr_t>(d_hist_len) & 3u))
         return ATTN_EINVAL;
-    const bool tc = c->cfg.head_dim == 128;  // tensor-core decode; head_dim 64 on the CUDA cores
     if (k_cache != c->dec_k || v_cache != c->dec_v) {
-        const cudaError_t me = tc ? attn::make_decode_tc_maps(c->encode, c->shape, k_cache, v_cache, &c->dec_maps)
-                                  : attn::make_decode_maps(c->encode, c->shape, k_cache, v_cache, &c->dec_maps);
+        const cudaError_t me = attn::make_decode_tc_maps(c->encode, c->shape, k_cache, v_cache, &c->dec_maps);
         if (me != cudaSuccess) {
             c->dec_k = c->dec_v = nullptr;
             std::snprintf(g_cuda_msg, sizeof g_cuda_msg, "cuTensorMapEncodeTiled failed for the decode caches");
@@ -354,31 +350,16 @@ int run_decode(attn_ctx* c, const uint16_t* q, const uint16_t* k, const uint16_t
     if (ntok < 1 || ntok > kMaxDraftTokens) return ATTN_EINVAL;
     // the partials hold batch * Hq * nsplit_max rows: ntok tokens share them
     const int ncg = attn::decode_tc_column_groups(c->cfg.n_q_heads / c->cfg.n_kv_heads, ntok);
-    // grid y and z (kv heads; sequences x column groups, or kv heads x head passes) stay
-    // within the 65535 limit of those grid dimensions
-    const int G = c->cfg.n_q_heads / c->cfg.n_kv_heads;
-    if (tc ? static_cast<long>(c->cfg.batch) * ncg > 65535
-           : static_cast<long>(c->cfg.n_kv_heads) * attn::decode_passes(c->shape, ntok) > 65535)
-        return ATTN_EINVAL;
-    if (seq_tok == 0) seq_tok = ntok;
-    const int nsplit = tc ? std::min(attn::decode_tc_num_splits(c->shape, c->num_sms, ncg, ntok), c->nsplit_max / ntok)
-                          : attn::decode_num_splits(c->shape, c->num_sms, c->nsplit_max / ntok, ntok);
-    cudaError_t e = timed(c, ATTN_KERNEL_DECODE_SPLIT, st, [&](int*) {
-        if (tc)
-            return attn::launch_decode_tc(c->shape, c->dec_maps, q, k, v, d_hist_len, hist_add, k_cache, v_cache, c->d_cos,
-                                          c->d_sin, c->d_part_o, c->d_part_ml, c->d_counters, nsplit, out,
-                                          c->d_err, after_decode, ntok, st, producer_early, c->wait_ns, c->num_sms);
-        return attn::launch_decode_split(c->shape, c->dec_maps, q, k, v, d_hist_len, hist_add, ntok, seq_tok, k_cache,
-                                         v_cache, c->d_cos, c->d_sin, c->d_part_o, c->d_part_ml, nsplit, c->d_err, st,
-                                         c->wait_ns);
+    // grid dimensions of sequences x column groups stay within 65535
+    if (static_cast<long>(c->cfg.batch) * ncg > 65535) return ATTN_EINVAL;
+    const int nsplit = std::min(attn::decode_tc_num_splits(c->shape, c->num_sms, ncg, ntok), c->nsplit_max / ntok);
+    const cudaError_t e = timed(c, ATTN_KERNEL_DECODE_SPLIT, st, [&](int*) {
+        return attn::launch_decode_tc(c->shape, c->dec_maps, q, k, v, d_hist_len, hist_add, k_cache, v_cache, c->d_cos,
+                                      c->d_sin, c->d_part_o, c->d_part_ml, c->d_counters, nsplit, out, c->d_err,
+                                      after_decode, ntok, seq_tok == 0 ? ntok : seq_tok, st, producer_early, c->wait_ns,
+                                      c->num_sms);
     });
-    if (e != cudaSuccess) return cuda_fail(e, "decode_split launch");
-    if (tc) return ATTN_OK;  // the tensor-core decode merges its splits itself
-    e = timed(c, ATTN_KERNEL_DECODE_COMBINE, st, [&](int*) {
-        return attn::launch_decode_combine(c->shape, d_hist_len, hist_add, ntok, seq_tok, c->d_part_o, c->d_part_ml,
-                                           nsplit, out, st);
-    });
-    if (e != cudaSuccess) return cuda_fail(e, "decode_combine launch");
+    if (e != cudaSuccess) return cuda_fail(e, "decode launch");
     return ATTN_OK;
 }
 
@@ -399,11 +380,12 @@ int attn_decode_multi(attn_ctx* c, const uint16_t* q, const uint16_t* k, const u
         return run_decode(c, q, k, v, d_hist_len, 0, false, k_cache, v_cache, out, st, n_new);
     // head_dim 64: up to 16 tokens per launch, read and written where they lie (n_new may be as
     // large as max_len); launch t0 continues at positions hist_len[b] + t0.  Fewer per launch
-    // only where the column passes of more would leave the grid's limits.
+    // only where the column groups of more would leave the grid's limits.
     if (q == nullptr || k == nullptr || v == nullptr || out == nullptr || n_new < 1 || n_new > c->cfg.max_len)
         return ATTN_EINVAL;
     int per = std::min(n_new, kMaxDraftTokens);
-    while (per > 1 && static_cast<long>(c->cfg.n_kv_heads) * attn::decode_passes(c->shape, per) > 65535) --per;
+    const int G = c->cfg.n_q_heads / c->cfg.n_kv_heads;
+    while (per > 1 && static_cast<long>(c->cfg.batch) * attn::decode_tc_column_groups(G, per) > 65535) --per;
     const size_t qtok = static_cast<size_t>(c->cfg.n_q_heads) * c->cfg.head_dim;  // elements of one token's rows
     const size_t ktok = static_cast<size_t>(c->cfg.n_kv_heads) * c->cfg.head_dim;
     for (int t0 = 0; t0 < n_new; t0 += per) {

@@ -7,9 +7,8 @@
 // front, or in a callback that must not touch the allocator.  Such a caller cannot
 // create an attn_ctx (attn_create allocates the tables and the split-KV partials).
 //
-// This entry point runs the same kernels as attn_decode (K3 with the new token's
-// append; for head_dim 64 also K4, which merges the splits) but needs no context: the
-// caller passes every input and output, including the RoPE tables and the error word,
+// This entry point runs the same kernel as attn_decode (K3 with the new token's append
+// and the merge of the splits) but needs no context: the caller passes every input and output, including the RoPE tables and the error word,
 // and the split-KV partials and merge counters live in the file-scope arrays below,
 // which the library holds on every device that loads it until the process exits.
 // Nothing is allocated or freed.
@@ -34,8 +33,9 @@ namespace {
 static __device__ __align__(256) float g_noalloc_scratch[ATTN_NOALLOC_SCRATCH_FLOATS];
 // Counters of the tensor-core decode for up to kNoallocCounters (sequence, kv head) items
 // (decode_tc_counter_ints of them); zero at load and left zero by every launch.
-// B*Hkv <= B*Hq <= scratch / (D + 2) < 8192.
-constexpr int kNoallocCounters = 8192;
+// B*Hkv <= B*Hq <= scratch / (D + 2) < 16384.
+constexpr int kNoallocCounters = 16384;
+static_assert(ATTN_NOALLOC_SCRATCH_FLOATS / (64 + 2) < kNoallocCounters, "an item per query head fits");
 static __device__ __align__(16) int g_noalloc_counters[5 * kNoallocCounters + 1] = {0};
 
 constexpr int kMaxDevices = 64;
@@ -75,8 +75,7 @@ int setup_device(int dev, float** scratch, int** counters, int* num_sms) {
         void* pc = nullptr;
         e = cudaGetSymbolAddress(&pc, g_noalloc_counters);
         if (e != cudaSuccess) return attn::record_cuda_error(e, "attn_decode_noalloc: counter array address");
-        e = attn::configure_decode();
-        if (e == cudaSuccess) e = attn::configure_decode_tc();
+        e = attn::configure_decode_tc();
         if (e != cudaSuccess) return attn::record_cuda_error(e, "attn_decode_noalloc: kernel attributes");
         g_counter_ptr[dev] = static_cast<int*>(pc);
         g_num_sms[dev] = sms;
@@ -128,26 +127,20 @@ extern "C" int attn_decode_noalloc(const attn_cfg* cfg, const float* d_cos, cons
     const attn::Shape s{cfg->batch, cfg->n_q_heads, cfg->n_kv_heads, cfg->head_dim, cfg->max_len};
     const long long fit = ATTN_NOALLOC_SCRATCH_FLOATS / per_split;
     const int cap = static_cast<int>(fit < 256 ? fit : 256);
-    const bool tc = cfg->head_dim == 128;
-    int nsplit = tc ? attn::decode_tc_num_splits(s, num_sms) : attn::decode_num_splits(s, num_sms, cap);
+    int nsplit = attn::decode_tc_num_splits(s, num_sms);
     nsplit = nsplit < cap ? nsplit : cap;
     float* part_o = scratch;
     float* part_ml = scratch + static_cast<size_t>(cfg->batch) * cfg->n_q_heads * nsplit * cfg->head_dim;
 
     attn::DecodeMaps maps;
-    const cudaError_t me = tc ? attn::make_decode_tc_maps(g_encode, s, k_cache, v_cache, &maps)
-                              : attn::make_decode_maps(g_encode, s, k_cache, v_cache, &maps);
+    const cudaError_t me = attn::make_decode_tc_maps(g_encode, s, k_cache, v_cache, &maps);
     if (me != cudaSuccess) {
         attn::record_error_text("attn_decode_noalloc: cuTensorMapEncodeTiled failed for the caches");
         return ATTN_ECUDA;
     }
     const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if (tc && static_cast<long long>(cfg->batch) * cfg->n_kv_heads > kNoallocCounters) return ATTN_EINVAL;
-    cudaError_t e = tc ? attn::launch_decode_tc(s, maps, q, k, v, d_hist_len, 0, k_cache, v_cache, d_cos, d_sin, part_o,
-                                                part_ml, counters, nsplit, out, d_err, false, 1, st, false,
-                                                attn::kWaitLimitNs, num_sms)
-                       : attn::launch_decode_split(s, maps, q, k, v, d_hist_len, 0, 1, 1, k_cache, v_cache, d_cos, d_sin,
-                                                   part_o, part_ml, nsplit, d_err, st);
-    if (e == cudaSuccess && !tc) e = attn::launch_decode_combine(s, d_hist_len, 0, 1, 1, part_o, part_ml, nsplit, out, st);
+    const cudaError_t e = attn::launch_decode_tc(s, maps, q, k, v, d_hist_len, 0, k_cache, v_cache, d_cos, d_sin, part_o,
+                                                 part_ml, counters, nsplit, out, d_err, false, 1, 1, st, false,
+                                                 attn::kWaitLimitNs, num_sms);
     return e == cudaSuccess ? ATTN_OK : attn::record_cuda_error(e, "attn_decode_noalloc: launch");
 }

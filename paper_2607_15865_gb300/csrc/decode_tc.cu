@@ -1,5 +1,5 @@
-// decode_tc.cu -- K3 for head_dim 128: split-KV decode attention on the tensor cores,
-// with the merge of the splits fused in.
+// decode_tc.cu -- K3: split-KV decode attention on the tensor cores, head_dim 128 and 64, with
+// the merge of the splits fused in.
 //
 // Decode (Section 4.4): one new query per sequence b at position p = hist_len[b]
 // attends to cache slots [0, p] of its kv head; its own k/v go to slot p (the
@@ -13,6 +13,10 @@
 // a tile fill the MMA's M dimension:
 //   S^T [128 keys x 16] = K_tile [128 x D] . Q^T       (Q: C columns, zero-padded to 16)
 //   O^T [D x 16]      += V_tile^T [D x 128] . P^T [128 x 16]
+// At head_dim 64 P is held to float precision, as the sum of three bf16 parts (further columns
+// of P^T and O^T, in the same MMAs), and the PV MMA's upper 64 rows are unused.  (Before, head_dim 64 ran on the CUDA cores, 64-key tiles and
+// a merge kernel: calls in a graph, 32 / 8 heads, B16 over 8190 tokens 72.1 us, now 56.7;
+// 5 tokens of 3 sequences 80.5 us, now 26.)
 // Both accumulate in TMEM.  The T = ceil((p+ntok)/128) key tiles of a sequence are
 // claimed by the nsplit CTAs of its item (b, kv head, column group): in a one-wave grid
 // split s starts with tile s, in a larger one only split 0 has a fixed first tile; every
@@ -60,7 +64,6 @@
 namespace attn {
 namespace {
 
-constexpr int D = 128;
 constexpr int KT = 128;     // keys per tile (MMA M)
 constexpr int NH = 16;      // padded columns of Q^T (MMA N): query heads x new tokens
 constexpr int kMaxTok = 16;  // new tokens per sequence in one launch (heads x tokens <= NH)
@@ -72,21 +75,29 @@ constexpr int VST = 4;      // V ring stages (a V tile is held until its PV comp
 constexpr int kThreads = 192;
 constexpr int kWarpTma = 4;
 constexpr int kWarpMma = 5;
-constexpr uint32_t kTmemCols = 64;  // S^T x2 [0,32), O^T [32,48)
 constexpr uint32_t TM_O = 32;
 
 enum Bar { B_QREADY, B_KFULL0, B_KFULL1, B_KEMPTY0, B_KEMPTY1, B_VFULL0, B_VFULL1, B_VFULL2, B_VFULL3,
            B_VEMPTY0, B_VEMPTY1, B_VEMPTY2, B_VEMPTY3, B_SFULL0, B_SFULL1, B_PFULL0, B_PFULL1, B_PVDONE, B_OFULL,
            B_DRAIN, NBAR };
 
-struct L {
+// Shared memory at head_dim D.  NP: bf16 parts that P is split into for the PV MMAs (head_dim 64
+// keeps its weights to float precision: p = hi + mid + lo, each the bf16 rounding of the rest).
+// The parts are further columns of P^T (16 each), so one MMA per 16 keys takes them all; O^T has
+// as many column groups, added up at the end.
+template <int D>
+struct Layout {
+    static constexpr int NP = D == 64 ? 3 : 1;
+    static constexpr int PC = NP * NH;                       // columns of P^T and O^T
+    static constexpr uint32_t TMEM_COLS = D == 64 ? 128 : 64;  // S^T x2 [0,32), O^T [32,32 + PC)
     static constexpr int BOX = KT * 128;           // [128 keys x 64 dims] bf16, 16 KB
-    static constexpr int TILE = 2 * BOX;           // one K (or V) tile, 32 KB
+    static constexpr int TILE = D / 64 * BOX;      // one K (or V) tile, 16 or 32 KB
     static constexpr int OFF_K = 0;                // K ring (the merge's weights reuse it)
     static constexpr int OFF_V = KST * TILE;       // V ring
-    static constexpr int OFF_Q = OFF_V + VST * TILE;  // Q^T [16 heads x 128] bf16, 2 x 2 KB
-    static constexpr int OFF_P = OFF_Q + 2 * NH * 128;          // P^T [16 x 128 keys] x 2 buffers
-    static constexpr int OFF_RED = OFF_P + 2 * 2 * NH * 128;    // float tile maxima [16 heads][4 warps]
+    static constexpr int OFF_Q = OFF_V + VST * TILE;  // Q^T [16 heads x D] bf16, D / 64 x 2 KB
+    static constexpr int P_BUF = 2 * PC * 128;                  // P^T [PC x 128 keys] bf16
+    static constexpr int OFF_P = OFF_Q + D / 64 * NH * 128;     // 2 buffers
+    static constexpr int OFF_RED = OFF_P + 2 * P_BUF;           // float tile maxima [16 heads][4 warps]
     static constexpr int OFF_LS = OFF_RED + NH * 4 * 4;         // float l partials [16 heads][4 warps]
     static constexpr int OFF_META = OFF_LS + NH * 4 * 4;       // int tile index per local tile, ring of 8
     static constexpr int OFF_BAR = OFF_META + 8 * 4;
@@ -94,18 +105,29 @@ struct L {
     static constexpr int OFF_ABORT = OFF_TMEM + 4;
     static constexpr int OFF_LAST = OFF_ABORT + 4;
     // int [8] at OFF_LAST: merge flag, merged slots, this CTA's partial slot, tiles it
-    // claimed, a helper split's first ticket
+    // claimed, a helper split's first ticket, new tokens whose v holds infinities or NaN
     static constexpr int OFF_CROW = OFF_LAST + 32;  // size_t [16]: partial row (slot 0) of column c
     static constexpr int OFF_OROW = OFF_CROW + NH * 8;  // size_t [16]: q / out row of column c
     static constexpr int BYTES = OFF_OROW + NH * 8;
     static constexpr int ALLOC = BYTES + 1024;
 };
-static_assert(L::ALLOC <= 232448, "shared memory of one CTA");
-static_assert((kThreads / 32) * NH * 8 + (kThreads / 32) * NH * D * 4 <= KST * L::TILE,
+static_assert(Layout<128>::ALLOC <= 232448, "shared memory of one CTA");
+static_assert((kThreads / 32) * NH * 8 + (kThreads / 32) * NH * 128 * 4 <= KST * Layout<128>::TILE &&
+                  (kThreads / 32) * NH * 8 + (kThreads / 32) * NH * 64 * 4 <= KST * Layout<64>::TILE,
               "merge buffers fit in the K ring");
+// At head_dim 64 the PV MMA still runs M = 128: its upper 64 rows read the 16 KB after the V tile
+// (the next stage, or Q and P after the last) and are never used; that must be shared memory.
+static_assert(Layout<64>::OFF_Q + Layout<64>::BOX <= Layout<64>::BYTES, "the last V stage is followed by 16 KB");
 
 __device__ __forceinline__ float bf16_at(const uint16_t* p) { return __uint_as_float(static_cast<uint32_t>(*p) << 16); }
 __device__ __forceinline__ uint16_t to_bf16(float x) { return __bfloat16_as_ushort(__float2bfloat16_rn(x)); }
+
+// A bf16 pair with infinities and NaN replaced by zero.
+__device__ __forceinline__ uint32_t finite_or_zero(uint32_t w) {
+    if ((w & 0x7F80u) == 0x7F80u) w &= 0xFFFF0000u;
+    if ((w & 0x7F800000u) == 0x7F800000u) w &= 0x0000FFFFu;
+    return w;
+}
 
 // Byte offset of element (row, col) in a [rows x 128] bf16 tile stored as two
 // 128-byte-swizzled 64-column chunks of `rows` rows (chunk stride rows * 128 bytes).
@@ -204,6 +226,27 @@ __device__ __forceinline__ bool halving_leader(int lane) {
     return N == 16 ? (lane & 1) == 0 : (lane & 3) == 0;
 }
 
+// The new tokens of a sequence that run: tokens [lo, hi), token i at position hist + i.
+// head_dim 128: all of them, or none where one would leave the cache (the sequence is skipped).
+// head_dim 64: those whose position is in [0, max_len) (tokens are skipped one by one, as decode
+// steps in order would; the columns of skipped tokens are computed with the others and never
+// written).
+struct TokRange {
+    int hist, lo, hi;
+};
+template <int D>
+__device__ __forceinline__ TokRange decode_tokens(int hist_len, int hist_add, int ntok, int max_len) {
+    const long long h = static_cast<long long>(hist_len) + hist_add;
+    if constexpr (D == 128) {
+        if (h < 0 || h > max_len - ntok) return {0, 0, 0};
+        return {static_cast<int>(h), 0, ntok};
+    } else {
+        const long long lo = h < 0 ? -h : 0, hi = min(static_cast<long long>(ntok), max_len - h);
+        if (lo >= hi) return {0, 0, 0};
+        return {static_cast<int>(h), static_cast<int>(lo), static_cast<int>(hi)};
+    }
+}
+
 // NHP: columns the softmax processes (8 when G * ntok <= 8, else 16); the MMA always
 // runs N = 16 with the rows of Q^T past the CTA's C columns zero.  With more than 16
 // columns (G * ntok > 16) the grid's z dimension is (sequence, column group): every column
@@ -216,17 +259,19 @@ __device__ __forceinline__ bool halving_leader(int lane) {
 // helper splits and slot and visit counters.  Each is its own instantiation, so that a
 // launch runs only the code of its mode.
 constexpr int kModeGlobal = 0, kModeCluster = 1, kModeWaves = 2;
-template <int NHP, int MAXTOK, int MODE>
+template <int D, int NHP, int MAXTOK, int MODE>
 __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
     const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
     const uint16_t* __restrict__ q, const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
-    const int32_t* __restrict__ d_hist, int hist_add, int ntok, uint16_t* __restrict__ k_cache,
+    const int32_t* __restrict__ d_hist, int hist_add, int ntok, int seq_tok, uint16_t* __restrict__ k_cache,
     uint16_t* __restrict__ v_cache, const float* __restrict__ cos_tab, const float* __restrict__ sin_tab, int Hq, int Hkv,
     int max_len, int nsplit,
     float scale_log2, float* __restrict__ part_o, float* __restrict__ part_ml, int* __restrict__ counters,
     uint16_t* __restrict__ out, int* __restrict__ err, int producer_early, uint64_t wait_ns, int ncg, int spec,
     int s0) {
+    using L = Layout<D>;
     constexpr bool WAVES = MODE == kModeWaves;
+    constexpr bool kGuardV = D == 64 && MAXTOK > 1;
     constexpr int HALF = D / 2;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -259,7 +304,10 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
     // The lengths, q and the new k/v are the caller's inputs: complete when this grid
     // starts (it is a dependent launch only after another decode step, which lets its
     // dependents start only once its own predecessors are complete).
-    const int hist = decode_hist(d_hist, b, hist_add);  // in flight while the barriers and TMEM are set up
+    // In flight while the barriers and TMEM are set up (volatile: the compiler may otherwise sink
+    // the load to its first use, behind that set-up: B1 over 1024 tokens 7.3 us instead of 6.9).
+    int hist_len;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(hist_len) : "l"(d_hist + b));
     const int kv_row = b * Hkv + g;
     const bool multi = nsplit > 1;
     // Several waves (s0 < nsplit): helper splits may claim after their item is merged, so
@@ -292,8 +340,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
             int tmax = 0, tsum = 0;
             if (batch <= 1024) {
                 for (int bb = lane; bb < batch; bb += 32) {
-                    const int hb = decode_hist(d_hist, bb, hist_add);
-                    const int tb = hb >= 0 && hb <= max_len - ntok ? (hb + ntok + KT - 1) / KT : 0;
+                    const TokRange rb = decode_tokens<D>(d_hist[bb], hist_add, ntok, max_len);
+                    const int tb = rb.hi > rb.lo ? (rb.hist + rb.hi + KT - 1) / KT : 0;
                     tmax = max(tmax, tb);
                     tsum += tb;
                 }
@@ -306,9 +354,10 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
             const bool even = batch <= 1024 && 10LL * tmax * batch <= 11LL * tsum;
             if (lane == 0) {
                 int t = -1;
-                if (hist >= 0 && hist <= max_len - ntok) {
+                const TokRange own = decode_tokens<D>(hist_len, hist_add, ntok, max_len);
+                if (own.hi > own.lo) {
                     if (!even) t = s0 + atomicAdd(claim_ctr, 1);
-                    if (t >= (hist + ntok + KT - 1) / KT) t = -1;
+                    if (t >= (own.hist + own.hi + KT - 1) / KT) t = -1;
                     if (t < 0 && atomicAdd(visit_ctr, 1) == nsplit - 1) {
                         *claim_ctr = 0;
                         *slot_ctr = 0;
@@ -330,6 +379,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
     const bool spec_first = spec != 0 && s < s0 && s * KT < max_len;
     if (warp == kWarpTma && lane == 0) {
         *abort_flag = 0;
+        lastv[5] = 0;
         mbar_init(bar(B_QREADY), 128);
         for (int st = 0; st < KST; ++st) {
             mbar_init(bar(B_KFULL0 + st), 1);
@@ -352,23 +402,24 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
         if (spec_first) {
             mbar_expect_tx(bar(B_KFULL0), L::TILE);
 #pragma unroll
-            for (int c = 0; c < 2; ++c)
+            for (int c = 0; c < D / 64; ++c)
                 tma_load_3d(base + L::OFF_K + c * L::BOX, &map_k, c * 64, s * KT, kv_row, bar(B_KFULL0));
             mbar_arrive_expect_tx(bar(B_VFULL0), L::TILE);
 #pragma unroll
-            for (int c = 0; c < 2; ++c)
+            for (int c = 0; c < D / 64; ++c)
                 tma_load_3d(base + L::OFF_V + c * L::BOX, &map_v, c * 64, s * KT, kv_row, bar(B_VFULL0));
         }
     }
 
     if (tid < NH) {
-        const int c = c0 + min(tid, C - 1);
-        const size_t r = (static_cast<size_t>(b) * ntok + c / G) * Hq + h0 + c % G;
-        reinterpret_cast<size_t*>(gb + L::OFF_OROW)[tid] = r;
-        reinterpret_cast<size_t*>(gb + L::OFF_CROW)[tid] = r * nsplit;
+        const int c = min(c0 + tid, G * ntok - 1);
+        reinterpret_cast<size_t*>(gb + L::OFF_OROW)[tid] =
+            (static_cast<size_t>(b) * seq_tok + c / G) * Hq + h0 + c % G;
+        reinterpret_cast<size_t*>(gb + L::OFF_CROW)[tid] =
+            ((static_cast<size_t>(b) * ntok + c / G) * Hq + h0 + c % G) * nsplit;
     }
     if (warp == kWarpMma) {
-        tmem_alloc(base + L::OFF_TMEM, kTmemCols);
+        tmem_alloc(base + L::OFF_TMEM, L::TMEM_COLS);
         tmem_relinquish();
     }
     tc_fence_before();
@@ -389,20 +440,26 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
         griddep_launch_dependents();
     }
 
-    const bool hist_ok = hist >= 0 && hist <= max_len - ntok;
-    if (!hist_ok && s == 0 && g == 0 && cg == 0 && tid == 0) atomicOr(err, kDevErrHistRange);
-    const int nkeys = hist + ntok;        // slots [0, hist) and the new tokens' [hist, hist + ntok)
+    const TokRange tr = decode_tokens<D>(hist_len, hist_add, ntok, max_len);
+    const int hist = tr.hist;
+    const bool item_ok = tr.lo < tr.hi;
+    // (head_dim 128: a sequence runs all its tokens or none)
+    auto runs = [&](int tt) { return D == 128 ? tt < ntok : tt >= tr.lo && tt < tr.hi; };
+    auto col_runs = [&](int h) { return D == 128 || runs((c0 + h) / G); };
+    if (tr.hi - tr.lo < ntok && s == 0 && g == 0 && cg == 0 && tid == 0) atomicOr(err, kDevErrHistRange);
+    const int nkeys = hist + tr.hi;       // slots [0, hist) and the new tokens', up to hist + hi - 1
     const int T = (nkeys + KT - 1) / KT;  // key tiles of the sequence; tile T-1 holds the last new slot
     // Splits s < s0 start with tile s; every other tile is claimed from the item's counter
     // (tickets s0, s0 + 1, ...).  A split that gets no tile writes nothing.
     // Rows of column c (token c / G, head h0 + c % G), tabulated once in the prologue:
-    // q / out row (b * ntok + c / G) * Hq + h0 + c % G, and partial row of slot 0 that
-    // times nsplit (slot sp adds sp).  Columns past C repeat column C - 1.
+    // q / out row (b * seq_tok + c / G) * Hq + h0 + c % G, and partial row of slot 0
+    // ((b * ntok + c / G) * Hq + h0 + c % G) * nsplit (slot sp adds sp).  Columns past the
+    // launch's repeat its last.
     const size_t* crow = reinterpret_cast<const size_t*>(gb + L::OFF_CROW);
     const size_t* orow = reinterpret_cast<const size_t*>(gb + L::OFF_OROW);
     int* meta = reinterpret_cast<int*>(gb + L::OFF_META);  // tile index of local tile j at [j % 8]; -1 ends
 
-    if (!hist_ok) {
+    if (!item_ok) {
         // sequence skipped: nothing written (the speculative copies land before the CTA ends)
         if (spec_first && warp == kWarpTma && lane == 0) {
             mbar_arrive(bar(B_KFULL0));
@@ -460,7 +517,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                 }
                 mbar_arrive_expect_tx(bar(B_KFULL0 + ks), L::TILE);
 #pragma unroll
-                for (int c = 0; c < 2; ++c)
+                for (int c = 0; c < D / 64; ++c)
                     tma_load_3d(base + L::OFF_K + ks * L::TILE + c * L::BOX, &map_k, c * 64, tile * KT, kv_row,
                                 bar(B_KFULL0 + ks));
                 issued_k = j + 1;
@@ -470,7 +527,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                 }
                 mbar_arrive_expect_tx(bar(B_VFULL0 + vs), L::TILE);
 #pragma unroll
-                for (int c = 0; c < 2; ++c)
+                for (int c = 0; c < D / 64; ++c)
                     tma_load_3d(base + L::OFF_V + vs * L::TILE + c * L::BOX, &map_v, c * 64, tile * KT, kv_row,
                                 bar(B_VFULL0 + vs));
                 issued_v = j + 1;
@@ -504,20 +561,21 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
         if (early) griddep_wait();
     } else if (warp == kWarpMma) {
         // ------------------------------------------------------------ tcgen05 issuer (+ the new tokens)
-        // Lane l handles dimensions 4l .. 4l+3 of each new token tt (slot hist + tt, rotated
-        // at that position by every CTA; written by the CTA that gets the slot's tile).
-        const int last_row = (hist + ntok - 1) - (T - 1) * KT;  // row of the last new slot in tile T-1
+        // Lane l (below D / 4) handles dimensions 4l .. 4l+3 of each new token tt (slot hist + tt,
+        // rotated at that position by every CTA; written by the CTA that gets the slot's tile).
+        const bool has_dims = D == 128 || 4 * lane < D;
+        const int last_row = (nkeys - 1) - (T - 1) * KT;  // row of the last new slot in tile T-1
         uint2 k_rot[MAXTOK], v_val[MAXTOK];
 #pragma unroll
         for (int tt = 0; tt < MAXTOK; ++tt) {
             if (tt >= ntok) break;
-            const int d0 = 4 * lane;
+            const int d0 = has_dims ? 4 * lane : 0;
             const int dp = d0 < HALF ? d0 + HALF : d0 - HALF;  // RoPE partner dimensions
-            const size_t src = (static_cast<size_t>(b * ntok + tt) * Hkv + g) * D;
+            const size_t src = ((static_cast<size_t>(b) * seq_tok + tt) * Hkv + g) * D;
             const uint2 kx = *reinterpret_cast<const uint2*>(k_new + src + d0);
             const uint2 ky = *reinterpret_cast<const uint2*>(k_new + src + dp);
             v_val[tt] = *reinterpret_cast<const uint2*>(v_new + src + d0);
-            const size_t pos = static_cast<size_t>(hist + tt);
+            const size_t pos = static_cast<size_t>(D == 128 ? hist + tt : min(max(hist + tt, 0), max_len - 1));
             const float4 c4 = *reinterpret_cast<const float4*>(cos_tab + pos * HALF + d0 % HALF);
             const float4 s4 = *reinterpret_cast<const float4*>(sin_tab + pos * HALF + d0 % HALF);
             const float xs[4] = {__uint_as_float(kx.x << 16), __uint_as_float(kx.x & 0xFFFF0000u),
@@ -535,7 +593,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
             k_rot[tt] = make_uint2(kb[0] | (kb[1] << 16), kb[2] | (kb[3] << 16));
         }
         constexpr uint32_t kIdQK = idesc_bf16_f32(KT, NH, false, false);
-        constexpr uint32_t kIdPV = idesc_bf16_f32(D, NH, true, false);
+        constexpr uint32_t kIdPV = idesc_bf16_f32(128, L::PC, true, false);
         // The warp stays converged and one elected lane issues: the loop's values then live in
         // uniform registers, where the MMA takes its operands from.
         constexpr uint32_t kHi = desc_hi_sw128(1024);
@@ -555,22 +613,33 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                 uint8_t* vt = gb + L::OFF_V + (jj % VST) * L::TILE;
 #pragma unroll
                 for (int tt = 0; tt < MAXTOK; ++tt)
-                    if (tt < ntok && (hist + tt) / KT == vtile)
-                        *reinterpret_cast<uint2*>(vt + sw_elem(hist + tt - vtile * KT, 4 * lane, KT)) = v_val[tt];
+                    if (runs(tt) && (hist + tt) / KT == vtile) {
+                        uint2 vv = v_val[tt];
+                        if constexpr (kGuardV) {
+                            // infinities and NaN of a new token's v must not meet the zero weights
+                            // of earlier tokens: they go in as zeros and are added at the end to
+                            // the columns that see the token
+                            const uint2 fin = make_uint2(finite_or_zero(vv.x), finite_or_zero(vv.y));
+                            if (__any_sync(0xFFFFFFFFu, fin.x != vv.x || fin.y != vv.y) && lane == 0)
+                                lastv[5] |= 1 << tt;
+                            vv = fin;
+                        }
+                        if (has_dims) *reinterpret_cast<uint2*>(vt + sw_elem(hist + tt - vtile * KT, 4 * lane, KT)) = vv;
+                    }
                 if (vtile == T - 1)
-                    for (int i = (last_row + 1) * 16 + lane; i < KT * 16; i += 32)
-                        *reinterpret_cast<uint4*>(vt + sw_elem(i >> 4, 8 * (i & 15), KT)) = make_uint4(0, 0, 0, 0);
+                    for (int i = (last_row + 1) * (D / 8) + lane; i < KT * (D / 8); i += 32)
+                        *reinterpret_cast<uint4*>(vt + sw_elem(i / (D / 8), 8 * (i % (D / 8)), KT)) = make_uint4(0, 0, 0, 0);
                 fence_proxy_async_smem();
             }
             __syncwarp();
             tc_fence_after();
             const uint32_t v_lo = desc_lo_sw128(sV, L::BOX);
-            const uint32_t p_lo = desc_lo_sw128(base + L::OFF_P + (jj & 1) * (2 * NH * 128), 16);
+            const uint32_t p_lo = desc_lo_sw128(base + L::OFF_P + (jj & 1) * L::P_BUF, 16);
             if (elect_one()) {
 #pragma unroll
                 for (int kk = 0; kk < KT / 16; ++kk)
                     umma_ss_w(tm + TM_O, v_lo + ((kk * 16 * 128) >> 4), kHi,
-                              p_lo + (((kk >> 2) * NH * 128 + (kk & 3) * 32) >> 4), kHi, kIdPV,
+                              p_lo + (((kk >> 2) * L::PC * 128 + (kk & 3) * 32) >> 4), kHi, kIdPV,
                               (jj > 0 || kk > 0) ? 1u : 0u);
                 umma_commit(bar(B_PVDONE));
                 umma_commit(bar(B_VEMPTY0 + jj % VST));
@@ -596,7 +665,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                 if (tile * KT + KT > hist) {  // new tokens in this tile: to the cache, rotated k into their rows
 #pragma unroll
                     for (int tt = 0; tt < MAXTOK; ++tt) {
-                        if (tt < ntok && (hist + tt) / KT == tile) {
+                        if (runs(tt) && (hist + tt) / KT == tile && has_dims) {
                             const size_t dst = (static_cast<size_t>(kv_row) * max_len + hist + tt) * D + 4 * lane;
                             *reinterpret_cast<uint2*>(k_cache + dst) = k_rot[tt];
                             *reinterpret_cast<uint2*>(v_cache + dst) = v_val[tt];
@@ -628,6 +697,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                 // completes without an MMA (S(n-2) on that buffer was consumed: PFULL(n-2) seen)
                 if (lane == 0) mbar_arrive(bar(B_SFULL0 + (n & 1)));
                 if (n > 0) ok = issue_pv(n - 1);
+                if constexpr (kGuardV) __threadfence_block();  // (lastv[5], read after OFULL)
                 if (ok && n > 0 && elect_one()) umma_commit(bar(B_OFULL));  // every PV is complete
             }
         }
@@ -648,29 +718,31 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
             // hist + c / G; zero rows past C; P^T buffers zeroed.  Each thread owns dimension t
             // of every column: all loads first, then the math.
             uint8_t* qs = gb + L::OFF_Q;
-            const int tp = t < HALF ? t + HALF : t - HALF;  // RoPE partner dimension
+            const int td = D == 128 ? t : t % D;                              // (head_dim 64: two threads per dimension)
+            const int tp = td < HALF ? td + HALF : td - HALF;  // RoPE partner dimension
             float qx[NHP], qy[NHP], c_t[NHP], s_t[NHP];
 #pragma unroll
             for (int c = 0; c < NHP; ++c) {
                 const int cc = min(c, C - 1);
                 const uint16_t* qrow = q + orow[cc] * D;
-                qx[c] = bf16_at(qrow + t);
+                qx[c] = bf16_at(qrow + td);
                 qy[c] = bf16_at(qrow + tp);
-                const size_t pos = static_cast<size_t>(hist + (c0 + cc) / G);
-                c_t[c] = cos_tab[pos * HALF + t % HALF];
-                s_t[c] = sin_tab[pos * HALF + t % HALF];
+                const int pc = hist + (c0 + cc) / G;
+                const size_t pos = static_cast<size_t>(D == 128 ? pc : min(max(pc, 0), max_len - 1));
+                c_t[c] = cos_tab[pos * HALF + td % HALF];
+                s_t[c] = sin_tab[pos * HALF + td % HALF];
             }
 #pragma unroll
             for (int c = 0; c < NH; ++c) {
                 uint16_t qb = 0;
                 if (c < NHP && c < C) {
-                    const float r = t < HALF ? __fsub_rn(__fmul_rn(qx[c], c_t[c]), __fmul_rn(qy[c], s_t[c]))
+                    const float r = td < HALF ? __fsub_rn(__fmul_rn(qx[c], c_t[c]), __fmul_rn(qy[c], s_t[c]))
                                              : __fadd_rn(__fmul_rn(qx[c], c_t[c]), __fmul_rn(qy[c], s_t[c]));
                     qb = to_bf16(r);
                 }
-                *reinterpret_cast<uint16_t*>(qs + sw_elem(c, t, NH)) = qb;
+                if (D == 128 || t < D) *reinterpret_cast<uint16_t*>(qs + sw_elem(c, t, NH)) = qb;
             }
-            for (int i = t; i < 2 * NH * 128 / 16; i += 128)
+            for (int i = t; i < 2 * L::P_BUF / 16; i += 128)
                 reinterpret_cast<uint4*>(gb + L::OFF_P)[i] = make_uint4(0, 0, 0, 0);
             fence_proxy_async_smem();
             mbar_arrive(bar(B_QREADY));
@@ -737,24 +809,33 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                     ok = !named_or_128(!mbar_wait(bar(B_PVDONE), static_cast<uint32_t>(j - 1) & 1u, abort_flag, wait_ns));
                     if (!ok) break;
                     tc_fence_after();
-                    uint32_t o[NHP];
-                    tmem_ld_cols<NHP>(tmem + lane_base + TM_O, o);
-                    tmem_wait_ld();
 #pragma unroll
-                    for (int h = 0; h < NHP; ++h) o[h] = __float_as_uint(__uint_as_float(o[h]) * alpha[h]);
-                    tmem_st_cols<NHP>(tmem + lane_base + TM_O, o);
+                    for (int part = 0; part < L::NP; ++part) {
+                        uint32_t o[NHP];
+                        tmem_ld_cols<NHP>(tmem + lane_base + TM_O + part * NH, o);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int h = 0; h < NHP; ++h) o[h] = __float_as_uint(__uint_as_float(o[h]) * alpha[h]);
+                        tmem_st_cols<NHP>(tmem + lane_base + TM_O + part * NH, o);
+                    }
                     tmem_wait_st();
                 }
             }
             // P^T (bf16, row = head, column = key of the tile); padded heads stay zero
-            uint8_t* pbuf = gb + L::OFF_P + (j & 1) * (2 * NH * 128);
+            uint8_t* pbuf = gb + L::OFF_P + (j & 1) * L::P_BUF;
 #pragma unroll
             for (int h = 0; h < NHP; ++h) {
                 if (h < C) {
                     const float m_ref = m_run[h] == -INFINITY ? 0.f : m_run[h];
                     const float p = fast_exp2(sc[h] - m_ref);
                     l_run[h] += p;
-                    *reinterpret_cast<uint16_t*>(pbuf + sw_elem(h, t, NH)) = to_bf16(p);
+                    float rest = p;
+#pragma unroll
+                    for (int part = 0; part < L::NP; ++part) {
+                        const uint16_t pb = to_bf16(rest);
+                        *reinterpret_cast<uint16_t*>(pbuf + sw_elem(part * NH + h, t, L::PC)) = pb;
+                        rest -= __uint_as_float(static_cast<uint32_t>(pb) << 16);  // exact
+                    }
                 }
             }
             fence_proxy_async_smem();
@@ -774,6 +855,25 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
             uint32_t o[NHP];
             tmem_ld_cols<NHP>(tmem + lane_base + TM_O, o);  // thread t = output dimension d
             tmem_wait_ld();
+#pragma unroll
+            for (int part = 1; part < L::NP; ++part) {
+                uint32_t o2[NHP];
+                tmem_ld_cols<NHP>(tmem + lane_base + TM_O + part * NH, o2);
+                tmem_wait_ld();
+#pragma unroll
+                for (int h = 0; h < NHP; ++h) o[h] = __float_as_uint(__uint_as_float(o[h]) + __uint_as_float(o2[h]));
+            }
+            if constexpr (kGuardV) {
+                const int odd = *reinterpret_cast<volatile int*>(lastv + 5);
+                for (int tt = 0; odd >> tt; ++tt) {
+                    if (!((odd >> tt) & 1) || t >= D) continue;
+                    const uint32_t w = v_new[((static_cast<size_t>(b) * seq_tok + tt) * Hkv + g) * D + t];
+                    if ((w & 0x7F80u) != 0x7F80u) continue;
+#pragma unroll
+                    for (int h = 0; h < NHP; ++h)
+                        if (h < C && (c0 + h) / G >= tt) o[h] = __float_as_uint(__uint_as_float(o[h]) + __uint_as_float(w << 16));
+                }
+            }
             named_sync_128();
             // the output (one split with tiles), the partial (m, l, acc) at slot s (global
             // merge), or (m, l, acc) staged in the idle V ring: read by the cluster's merge, or
@@ -786,8 +886,9 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                 if (h < C) {
                     const float4 l4 = reinterpret_cast<const float4*>(ls)[h];
                     const float l_tot = (l4.x + l4.y) + (l4.z + l4.w);
+                    if (D < 128 && t >= D) continue;  // (the PV MMA's unused rows)
                     if (alone) {
-                        out[orow[h] * D + t] = to_bf16(__uint_as_float(o[h]) / l_tot);
+                        if (col_runs(h)) out[orow[h] * D + t] = to_bf16(__uint_as_float(o[h]) / l_tot);
                     } else if constexpr (MODE == kModeGlobal) {
                         const size_t row = crow[h] + s;
                         part_o[row * D + t] = __uint_as_float(o[h]);
@@ -812,7 +913,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
         // reading its peers' staging directly, then waits at a second barrier until its own
         // staging has been read.  (T is the same in every CTA of the cluster, so all or none
         // of them take part.)
-        if (hist_ok && multi && T > 1) {
+        if (item_ok && multi && T > 1) {
             tc_fence_before();
             cluster_sync();
             if (s == 0 && tid == 0) *claim_ctr = 0;  // every split has made its last claim
@@ -845,11 +946,11 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                         l_tot = fmaf(wgt, lr[r], l_tot);
                         acc = fmaf(wgt, orr[r], acc);
                     }
-                out[orow[h] * D + d] = to_bf16(acc / l_tot);
+                if (col_runs(h)) out[orow[h] * D + d] = to_bf16(acc / l_tot);
             }
             cluster_sync();
         }
-    } else if (hist_ok && multi) {
+    } else if (item_ok && multi) {
         bool contrib;  // (uniform over the CTA) this split wrote a partial and takes part
         if constexpr (WAVES) {
             tc_fence_before();
@@ -864,7 +965,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                     const int h = p / (D / 4), c = p % (D / 4);
                     const float4 v4 = st_o4[h * (D / 4) + c];
                     const float inv = 1.f / st_ml[h].y;
-                    *reinterpret_cast<uint2*>(out + orow[h] * D + 4 * c) =
+                    if (col_runs(h))
+                        *reinterpret_cast<uint2*>(out + orow[h] * D + 4 * c) =
                         make_uint2(to_bf16(v4.x * inv) | (static_cast<uint32_t>(to_bf16(v4.y * inv)) << 16),
                                    to_bf16(v4.z * inv) | (static_cast<uint32_t>(to_bf16(v4.w * inv)) << 16));
                 }
@@ -940,7 +1042,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                 for (int h = 0; h < NHP; ++h) {
                     const int hh = min(h, C - 1);
                     ml[h] = __ldcg(reinterpret_cast<const float2*>(part_ml) + crow[hh] + sp);
-                    o4[h] = __ldcg(reinterpret_cast<const float4*>(part_o + (crow[hh] + sp) * D) + lane);
+                    o4[h] = __ldcg(reinterpret_cast<const float4*>(part_o + (crow[hh] + sp) * D) + lane % (D / 4));
                 }
 #pragma unroll
                 for (int h = 0; h < NHP; ++h) {
@@ -959,7 +1061,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
 #pragma unroll
             for (int h = 0; h < NHP; ++h)
                 if (h < C) {
-                    reinterpret_cast<float4*>(racc + (warp * NH + h) * D)[lane] = acc[h];
+                    if (lane < D / 4) reinterpret_cast<float4*>(racc + (warp * NH + h) * D)[lane] = acc[h];
                     if (lane == 0) wml[warp * NH + h] = make_float2(mw[h], lw[h]);
                 }
             __syncthreads();
@@ -987,7 +1089,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                 const uint2 packed = make_uint2(
                     to_bf16(sum.x * inv) | (static_cast<uint32_t>(to_bf16(sum.y * inv)) << 16),
                     to_bf16(sum.z * inv) | (static_cast<uint32_t>(to_bf16(sum.w * inv)) << 16));
-                *reinterpret_cast<uint2*>(out + orow[h] * D + 4 * c) = packed;
+                if (col_runs(h)) *reinterpret_cast<uint2*>(out + orow[h] * D + 4 * c) = packed;
             }
         }
     }
@@ -995,7 +1097,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
     __syncthreads();
     if (warp == kWarpMma) {
         tc_fence_after();
-        tmem_dealloc(tmem, kTmemCols);
+        tmem_dealloc(tmem, L::TMEM_COLS);
     }
 }
 
@@ -1007,28 +1109,37 @@ constexpr int kMaxDevices = 64;
 constexpr int kMaxCluster = 16;
 int g_cluster_fit[kMaxDevices][kMaxCluster + 1] = {};
 
-#define DECODE_TC_MODES(NHP, MAXTOK)                                                          \
-    decode_tc_kernel<NHP, MAXTOK, kModeGlobal>, decode_tc_kernel<NHP, MAXTOK, kModeCluster>, \
-        decode_tc_kernel<NHP, MAXTOK, kModeWaves>
+#define DECODE_TC_MODES(D, NHP, MAXTOK)                                                             \
+    decode_tc_kernel<D, NHP, MAXTOK, kModeGlobal>, decode_tc_kernel<D, NHP, MAXTOK, kModeCluster>, \
+        decode_tc_kernel<D, NHP, MAXTOK, kModeWaves>
+
+template <int D>
+cudaError_t set_attributes() {
+    cudaError_t e = cudaSuccess;
+    for (auto fn : {DECODE_TC_MODES(D, 8, 1), DECODE_TC_MODES(D, 16, 1), DECODE_TC_MODES(D, 8, kMaxTok),
+                    DECODE_TC_MODES(D, 16, kMaxTok)})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Layout<D>::ALLOC);
+    for (auto fn : {decode_tc_kernel<D, 8, 1, kModeCluster>, decode_tc_kernel<D, 16, 1, kModeCluster>,
+                    decode_tc_kernel<D, 8, kMaxTok, kModeCluster>, decode_tc_kernel<D, 16, kMaxTok, kModeCluster>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+}
 
 cudaError_t configure_decode_tc() {
-    cudaError_t e = cudaSuccess;
-    for (auto fn : {DECODE_TC_MODES(8, 1), DECODE_TC_MODES(16, 1), DECODE_TC_MODES(8, kMaxTok),
-                    DECODE_TC_MODES(16, kMaxTok)})
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, L::ALLOC);
-    for (auto fn : {decode_tc_kernel<8, 1, kModeCluster>, decode_tc_kernel<16, 1, kModeCluster>,
-                    decode_tc_kernel<8, kMaxTok, kModeCluster>, decode_tc_kernel<16, kMaxTok, kModeCluster>})
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaError_t e = set_attributes<128>();
+    if (e == cudaSuccess) e = set_attributes<64>();
     int dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    // (the four cluster instantiations share the block size, shared memory and one block per SM)
+    // (the cluster instantiations share the block size and one block per SM; measured with the
+    // larger shared memory, of head_dim 128)
     for (int c = 2; c <= kMaxCluster; ++c) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(static_cast<unsigned>(c), 1, 1);
         cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = L::ALLOC;
+        cfg.dynamicSmemBytes = Layout<128>::ALLOC;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = static_cast<unsigned>(c);
@@ -1037,7 +1148,7 @@ cudaError_t configure_decode_tc() {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, decode_tc_kernel<8, 1, kModeCluster>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(&n, decode_tc_kernel<128, 8, 1, kModeCluster>, &cfg) != cudaSuccess) {
             n = 0;
             cudaGetLastError();  // a refused size is never used
         }
@@ -1066,15 +1177,17 @@ bool decode_tc_clusters_fit(int nsplit, long long items) {
 constexpr int kWaveSplits = 3;
 // One wave: at most 16 splits per item.  The long decode (8 items) measured 29.5 us with 16
 // splits, 30.4-30.8 us with 19 (one per SM), 32.5 with 12 and 42 with 8: past 16 the extra
-// partials and the later last CTA cost more than the SMs add.
-constexpr long kMaxWaveSplits1 = 16;
+// partials and the later last CTA cost more than the SMs add.  Up to 4 items take 32, which
+// leaves fewer SMs idle (4 items over 32767 tokens 20.9 -> 18.9 us; head_dim 64, 2 items over 32000: 23.9 -> 15.7).
+constexpr long kMaxWaveSplits1 = 16, kMaxWaveSplitsFew = 32, kFewItems = 4;
 
 int decode_tc_column_groups(int G, int ntok) { return (G * ntok + NH - 1) / NH; }
 
 int decode_tc_num_splits(const Shape& s, int num_sms, int ncg, int ntok) {
     const long items = static_cast<long>(s.batch) * s.n_kv_heads * ncg;
     const long max_tiles = std::max(1L, static_cast<long>((s.max_len + KT - 1) / KT));
-    long ns = 2 * items > num_sms ? kWaveSplits : std::min<long>(kMaxWaveSplits1, num_sms / items);
+    long ns = 2 * items > num_sms ? kWaveSplits
+                                  : std::min<long>(items <= kFewItems ? kMaxWaveSplitsFew : kMaxWaveSplits1, num_sms / items);
     ns = std::min(ns, std::min(max_tiles, 256L));
     // The last split of an item merges ns partials of up to 16 columns in the global merge,
     // while a cluster spreads the merge over its CTAs.  Fewer splits whose clusters fit on the
@@ -1092,7 +1205,8 @@ int decode_tc_num_splits(const Shape& s, int num_sms, int ncg, int ntok) {
 
 cudaError_t make_decode_tc_maps(PFN_encodeTiled encode, const Shape& s, const uint16_t* k_cache,
                                 const uint16_t* v_cache, DecodeMaps* maps) {
-    const cuuint64_t dims[3] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(s.max_len),
+    const cuuint64_t D = static_cast<cuuint64_t>(s.head_dim);
+    const cuuint64_t dims[3] = {D, static_cast<cuuint64_t>(s.max_len),
                                 static_cast<cuuint64_t>(s.batch) * s.n_kv_heads};
     const cuuint64_t strides[2] = {D * 2, D * 2 * static_cast<cuuint64_t>(s.max_len)};
     const cuuint32_t box[3] = {64, KT, 1};
@@ -1111,8 +1225,9 @@ cudaError_t launch_decode_tc(const Shape& s, const DecodeMaps& maps, const uint1
                              const uint16_t* v_new, const int32_t* d_hist, int hist_add, uint16_t* k_cache,
                              uint16_t* v_cache, const float* cos_tab, const float* sin_tab, float* part_o,
                              float* part_ml, int* counters, int nsplit, uint16_t* out, int* err, bool after_decode,
-                             int ntok, cudaStream_t st, bool producer_early, uint64_t wait_ns, int num_sms) {
-    const float scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(D)));
+                             int ntok, int seq_tok, cudaStream_t st, bool producer_early, uint64_t wait_ns,
+                             int num_sms) {
+    const float scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(s.head_dim)));
     const int G = s.n_q_heads / s.n_kv_heads;
     const int ncg = decode_tc_column_groups(G, ntok);
     // every split starts with its own tile when the grid is one wave, else only split 0
@@ -1125,7 +1240,7 @@ cudaError_t launch_decode_tc(const Shape& s, const DecodeMaps& maps, const uint1
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = L::ALLOC;
+    cfg.dynamicSmemBytes = s.head_dim == 64 ? Layout<64>::ALLOC : Layout<128>::ALLOC;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     unsigned n_attr = 0;
@@ -1152,14 +1267,21 @@ cudaError_t launch_decode_tc(const Shape& s, const DecodeMaps& maps, const uint1
     cfg.attrs = attr;
     cfg.numAttrs = n_attr;
     if (ntok < 1 || ntok > kMaxTok || G > NH) return cudaErrorInvalidValue;
-    using Kernel = decltype(&decode_tc_kernel<8, 1, kModeGlobal>);
-    static const Kernel kernels[4][3] = {{DECODE_TC_MODES(8, 1)},
-                                         {DECODE_TC_MODES(16, 1)},
-                                         {DECODE_TC_MODES(8, kMaxTok)},
-                                         {DECODE_TC_MODES(16, kMaxTok)}};
-    const Kernel kernel = kernels[ntok == 1 ? (G <= 8 ? 0 : 1) : (G * ntok <= 8 ? 2 : 3)][mode];
+    using Kernel = decltype(&decode_tc_kernel<128, 8, 1, kModeGlobal>);
+    static const Kernel kernels[2][4][3] = {
+        {{DECODE_TC_MODES(128, 8, 1)},
+         {DECODE_TC_MODES(128, 16, 1)},
+         {DECODE_TC_MODES(128, 8, kMaxTok)},
+         {DECODE_TC_MODES(128, 16, kMaxTok)}},
+        {{DECODE_TC_MODES(64, 8, 1)},
+         {DECODE_TC_MODES(64, 16, 1)},
+         {DECODE_TC_MODES(64, 8, kMaxTok)},
+         {DECODE_TC_MODES(64, 16, kMaxTok)}}};
+    const Kernel kernel =
+        kernels[s.head_dim == 64][ntok == 1 ? (G <= 8 ? 0 : 1) : (G * ntok <= 8 ? 2 : 3)][mode];
     return cudaLaunchKernelEx(&cfg, kernel, maps.k, maps.v, q,
-                              k_new, v_new, d_hist, hist_add, ntok, k_cache, v_cache, cos_tab, sin_tab, s.n_q_heads,
+                              k_new, v_new, d_hist, hist_add, ntok, seq_tok, k_cache, v_cache, cos_tab, sin_tab,
+                              s.n_q_heads,
                               s.n_kv_heads, s.max_len, nsplit, scale_log2, part_o, part_ml, counters, out, err,
                               producer_early ? 1 : 0, wait_ns, ncg, after_decode ? 0 : 1, s0);
 }

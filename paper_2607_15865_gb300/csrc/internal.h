@@ -18,8 +18,8 @@ constexpr int kDevErrTimeout = 2;
 int record_cuda_error(cudaError_t e, const char* where);
 void record_error_text(const char* text);
 
-// Default limit of every bounded wait of the kernels (1 s).  The launchers of flash_fwd,
-// decode_split and decode_tc take a limit for the waits of their main loops; the waits
+// Default limit of every bounded wait of the kernels (1 s).  The launchers of flash_fwd
+// and decode_tc take a limit for the waits of their main loops; the waits
 // that let copies and MMAs already issued finish (before a CTA that gave up exits) always
 // keep this default.
 constexpr uint64_t kWaitLimitNs = 1000000000ull;
@@ -81,39 +81,22 @@ cudaError_t launch_flash_fwd(const Shape& s, const FlashMaps& maps, int hist, in
                              const float* cos_t, const float* sin_t, uint16_t* out, float* ws_o, float* ws_ml, int* err,
                              int num_sms, cudaStream_t st, int* n_launched, uint64_t wait_ns = kWaitLimitNs);
 
-// K3 + K4: decode, head_dim 64.  The maps cover the whole caches as 3-D {D, max_len, B*Hkv}
-// with 64-key boxes (built once per cache pair).  K3 also rotates the new keys and
-// appends k and v from slot hist[b] on; K4 merges the splits (programmatic dependent launch).
 using PFN_encodeTiled = PFN_cuTensorMapEncodeTiled_v12000;
 struct DecodeMaps {
-    CUtensorMap k;
+    CUtensorMap k;  // the whole k cache as 3-D {D, max_len, B*Hkv}, box {64, 128, 1}
     CUtensorMap v;
 };
-cudaError_t configure_decode();  // dynamic shared-memory limits of K3 (once per device)
-// Passes of up to 8 (token, head) columns that a kv head's ntok new tokens take.
-int decode_passes(const Shape& s, int ntok);
-int decode_num_splits(const Shape& s, int num_sms, int max_splits, int ntok = 1);
-cudaError_t make_decode_maps(PFN_encodeTiled encode, const Shape& s, const uint16_t* k_cache,
-                             const uint16_t* v_cache, DecodeMaps* maps);
-// Decode lengths: sequence b's new token takes position d_hist[b] + hist_add (hist_add >= 0
-// lets a run of decode steps share one length array); see decode_hist().  1 <= ntok <= 16 new
-// tokens per sequence at positions d_hist[b] + hist_add + i; q, k_new, v_new and out point at
-// the first of them in arrays of seq_tok tokens per sequence.  A token whose position is
-// outside [0, max_len) is flagged and skipped.  The partials need B * ntok * Hq * nsplit rows.
-cudaError_t launch_decode_split(const Shape& s, const DecodeMaps& maps, const uint16_t* q, const uint16_t* k_new,
-                                const uint16_t* v_new, const int32_t* d_hist, int hist_add, int ntok, int seq_tok,
-                                uint16_t* k_cache, uint16_t* v_cache,
-                                const float* cos_tab, const float* sin_tab, float* part_o, float* part_ml,
-                                int nsplit, int* err, cudaStream_t st, uint64_t wait_ns = kWaitLimitNs);
-// K3 for head_dim 128 on the tensor cores (decode_tc.cu): maps with 128-key boxes; same
-// partial layout as launch_decode_split, but the merge is fused in (the split that
-// completes an item's tiles merges and writes `out`), so no K4 follows.  Splits claim key
-// tiles from a per-item counter (item: sequence, kv head, column group).  `counters`:
+// K3: decode on the tensor cores (decode_tc.cu), head_dim 128 or 64: rotates the new keys,
+// appends k and v from slot d_hist[b] + hist_add on and attends; the merge of the splits is
+// fused in (the split that completes an item's tiles merges and writes `out`).  Splits claim
+// key tiles from a per-item counter (item: sequence, kv head, column group).  `counters`:
 // decode_tc_counter_ints(items) ints, zero before the first launch; every launch leaves
-// them zero.  num_sms: whether the grid fits one wave.  1 <= ntok <= 16 new tokens per
-// sequence (q/k/v/out
-// [B, ntok, H, D]) at positions d_hist[b] + hist_add + i, token i attending causally to
-// slots [0, that position]; the partials need B * ntok * Hq * nsplit rows.
+// them zero.  num_sms: whether the grid fits one wave.  hist_add >= 0 lets a run of decode
+// steps share one length array.  1 <= ntok <= 16 new tokens per sequence (q/k/v/out point at
+// the first of them in [B, seq_tok, H, D]) at positions d_hist[b] + hist_add + i, token i
+// attending causally to slots [0, that position]; the partials (part_o [row][D], part_ml
+// [row][2]) need B * ntok * Hq * nsplit rows.  A sequence with a position outside
+// [0, max_len) is flagged and skipped, at head_dim 64 only its tokens out of range.
 // after_decode: the stream's previous kernel is a decode_tc launch (the
 // previous step of a decode loop); this one then starts as a dependent launch whose
 // setup overlaps that step's tail.  Never set it after any other kernel: the inputs
@@ -137,10 +120,7 @@ cudaError_t launch_decode_tc(const Shape& s, const DecodeMaps& maps, const uint1
                              uint16_t* v_cache,
                              const float* cos_tab, const float* sin_tab, float* part_o, float* part_ml,
                              int* counters, int nsplit, uint16_t* out, int* err, bool after_decode, int ntok,
-                             cudaStream_t st, bool producer_early, uint64_t wait_ns, int num_sms);
-cudaError_t launch_decode_combine(const Shape& s, const int32_t* d_hist, int hist_add, int ntok, int seq_tok,
-                                  const float* part_o, const float* part_ml, int nsplit, uint16_t* out,
-                                  cudaStream_t st);
+                             int seq_tok, cudaStream_t st, bool producer_early, uint64_t wait_ns, int num_sms);
 
 // W4BF16 GEMV (w4_gemv.cu): y[m, n] = sum_k x[m, k] (q[n, k] - z[n, k/128]) s[n, k/128] for
 // the activation rows of one launch.  tiles: the tile
@@ -188,14 +168,5 @@ cudaError_t launch_w4_gemm(const uint8_t* tiles, const uint16_t* x, int T, int N
 // sum of squares in a fixed order); gamma bf16 [K].
 cudaError_t launch_rmsnorm_rows(const uint16_t* x, const uint16_t* gamma, float eps, int T, int K, uint16_t* xn,
                                 cudaStream_t st);
-
-#ifdef __CUDACC__
-// Position of sequence b's decode token: d_hist[b] + hist_add, or -1 (out of range, so
-// the caller flags and skips the sequence) when the sum leaves int.
-__device__ __forceinline__ int decode_hist(const int32_t* d_hist, int b, int hist_add) {
-    const long long h = static_cast<long long>(d_hist[b]) + hist_add;
-    return h > 0x7FFFFFFFLL ? -1 : static_cast<int>(h);
-}
-#endif
 
 }  // namespace attn
