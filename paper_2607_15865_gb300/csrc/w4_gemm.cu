@@ -106,12 +106,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
 // Arrive on the mbarrier at the shared::cluster address `bar` (another CTA's, or this one's).
 // What it publishes is ordered by other means (tensor-memory stores by tcgen05.wait::st and
 // the tcgen05 fences, the X tile by the copy's own barrier), so it needs no cluster-scope
@@ -146,10 +140,6 @@ __device__ __forceinline__ bool wait_full(uint32_t bar, uint32_t parity, const v
     }
 }
 
-__device__ __forceinline__ void st_dsmem_f32(uint32_t addr, uint32_t v) {
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-
 // The CTA-pair forms of the tcgen05 operations (sm100_ptx.cuh has those of one CTA).
 __device__ __forceinline__ void tmem_alloc2(uint32_t holder_smem, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(holder_smem), "r"(ncols)
@@ -176,12 +166,6 @@ __device__ __forceinline__ void umma2_commit_mc(uint32_t bar, uint16_t mask) {
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
         "h"(mask)
         : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
 }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
@@ -558,21 +542,22 @@ __global__ void __launch_bounds__(kThreads, 1) w4_gemm_kernel(const __grid_const
     }
 }
 
-// RMSNorm rows: one warp per row of K values.  Pass 1: per-lane float sums of squares over
-// 16-byte chunks in order, then a shuffle tree (a fixed order); pass 2 re-reads the row
-// (L1/L2) and writes bf16((x * r) * gamma).
-__global__ void __launch_bounds__(256) rmsnorm_rows_kernel(const uint16_t* __restrict__ x,
-                                                           const uint16_t* __restrict__ gamma, float eps, int T, int K,
-                                                           uint16_t* __restrict__ xn) {
-    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+// RMSNorm rows: one CTA per row of K values, so that a chunk of a few hundred tokens fills the
+// device and a thread's 16-byte loads are all in flight (500 rows of 4096 with a warp per row:
+// @@L@@).  Per-thread float sums of squares over the chunks in order, a shuffle tree, then the
+// warps in order (a fixed order); a thread keeps its first kRmsKeep chunks in registers and
+// re-reads the rest (L1/L2) to write bf16((x * r) * gamma).
+constexpr int kRmsThreads = 128, kRmsKeep = 8;
+__global__ void __launch_bounds__(kRmsThreads) rmsnorm_rows_kernel(const uint16_t* __restrict__ x,
+                                                                   const uint16_t* __restrict__ gamma, float eps, int T,
+                                                                   int K, uint16_t* __restrict__ xn) {
+    __shared__ float part[kRmsThreads / 32];
+    const int tid = threadIdx.x, row = blockIdx.x;
     griddep_wait();  // a dependent launch, as is the GEMM that follows
     griddep_launch_dependents();
-    if (row >= T) return;
     const uint4* xr = reinterpret_cast<const uint4*>(x + static_cast<size_t>(row) * K);
     const int nchunk = K / 8;
-    float ss = 0.f;
-    for (int i = lane; i < nchunk; i += 32) {
-        const uint4 v = xr[i];
+    auto squares = [](float ss, const uint4& v) {
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -580,14 +565,28 @@ __global__ void __launch_bounds__(256) rmsnorm_rows_kernel(const uint16_t* __res
             ss = fmaf(a, a, ss);
             ss = fmaf(b, b, ss);
         }
-    }
+        return ss;
+    };
+    uint4 keep[kRmsKeep];
+#pragma unroll
+    for (int i = 0; i < kRmsKeep; ++i)
+        keep[i] = tid + i * kRmsThreads < nchunk ? xr[tid + i * kRmsThreads] : make_uint4(0u, 0u, 0u, 0u);
+    float ss = 0.f;
+#pragma unroll
+    for (int i = 0; i < kRmsKeep; ++i) ss = squares(ss, keep[i]);
+    for (int i = tid + kRmsKeep * kRmsThreads; i < nchunk; i += kRmsThreads) ss = squares(ss, xr[i]);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, off);
-    const float r = 1.0f / sqrtf(ss / static_cast<float>(K) + eps);
+    if ((tid & 31) == 0) part[tid >> 5] = ss;
+    __syncthreads();
+    float tot = 0.f;
+#pragma unroll
+    for (int w = 0; w < kRmsThreads / 32; ++w) tot += part[w];
+    const float r = 1.0f / sqrtf(tot / static_cast<float>(K) + eps);
     const uint4* gr = reinterpret_cast<const uint4*>(gamma);
     uint4* out = reinterpret_cast<uint4*>(xn + static_cast<size_t>(row) * K);
-    for (int i = lane; i < nchunk; i += 32) {
-        const uint4 v = xr[i], g = gr[i];
+    auto write = [&](int i, const uint4& v) {
+        const uint4 g = gr[i];
         const uint32_t w[4] = {v.x, v.y, v.z, v.w}, gw[4] = {g.x, g.y, g.z, g.w};
         uint32_t o[4];
 #pragma unroll
@@ -597,7 +596,11 @@ __global__ void __launch_bounds__(256) rmsnorm_rows_kernel(const uint16_t* __res
             o[e] = pack_bf16x2(lo, hi);
         }
         out[i] = make_uint4(o[0], o[1], o[2], o[3]);
-    }
+    };
+#pragma unroll
+    for (int i = 0; i < kRmsKeep; ++i)
+        if (tid + i * kRmsThreads < nchunk) write(tid + i * kRmsThreads, keep[i]);
+    for (int i = tid + kRmsKeep * kRmsThreads; i < nchunk; i += kRmsThreads) write(i, xr[i]);
 }
 
 std::mutex g_mutex;
@@ -685,8 +688,8 @@ cudaError_t configure(int dev) {
 cudaError_t launch_rmsnorm_rows(const uint16_t* x, const uint16_t* gamma, float eps, int T, int K, uint16_t* xn,
                                 cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>((T + 7) / 8));
-    cfg.blockDim = dim3(256);
+    cfg.gridDim = dim3(static_cast<unsigned>(T));
+    cfg.blockDim = dim3(kRmsThreads);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
