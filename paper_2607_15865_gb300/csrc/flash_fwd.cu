@@ -293,7 +293,15 @@ __device__ __forceinline__ bool rope_item(uint32_t qfull, uint32_t qready, uint3
     return w;
 }
 
-template <int D>
+// CL: every unit is one of two pieces of its item and each CTA has one; the two CTAs of an item
+// are a cluster and merge in the kernel.  Once every MMA of both is complete, each sends its
+// float O of half of the columns, and its (m, l), of every row to the other's idle group ring
+// and q tiles, and finishes the other half from what it received.  (prefill_kv 512 over 1536,
+// 32 heads, calls in a graph: 27.3 us with the merge kernel, which waits for the whole grid and
+// reads 17 MB of partials, 24.3 with this; 512 over 8000 63.7 -> 61.9.  With more pieces the
+// larger cluster and its longer exchange cost more than the merge kernel: four of 256 rows over
+// 1500 24.3 us against 22.2, of one row over 2000 15.6 against 14.0.)
+template <int D, bool CL>
 __global__ void __launch_bounds__(kThreads, 1)
     flash_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_v, const Sched sc, int s_stride, int Hkv,
@@ -555,6 +563,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             umma_commit(bar(B_DRAIN));
             mbar_wait(bar(B_DRAIN), 0, nullptr);
         }
+        if constexpr (CL) {  // the two cluster barriers of the merge, reached by every thread
+            __syncwarp();
+            cluster_sync();
+            cluster_sync();
+        }
     } else {
         // ------------------------------------------------------------ softmax / epilogue warpgroups
         warpgroup_reg_inc<kRegsHigh>();
@@ -568,6 +581,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         int items = 0;
         bool ok = true;
 
+        float cl_m = -INFINITY, cl_l = 0.f;  // CL: this row's (m, l), 0 keys unless set
         int lin = blockIdx.x;
         Unit un;
         if (lin < n_units) {
@@ -681,7 +695,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!ok) break;
                 ++o_cnt;
                 tc_fence_after();
-                if (un.piece < 0) {
+                if constexpr (CL) {
+                    cl_m = m_run;
+                    cl_l = l_run;
+                } else if (un.piece < 0) {
                     // O_T / l -> bf16 through this warp's staging area, 64 columns at a time: each
                     // thread writes its row there, then the warp stores 4 rows (512 contiguous-row
                     // bytes) per instruction instead of 32 rows 10 KB apart.
@@ -738,23 +755,82 @@ __global__ void __launch_bounds__(kThreads, 1)
                         __syncwarp();
                     }
                 }
-                if (un.piece >= 0 && row < it.rows(t)) {
+                if (!CL && un.piece >= 0 && row < it.rows(t)) {
                     ws_ml[prow * 2 + 0] = m_run;
                     ws_ml[prow * 2 + 1] = l_run;
                 }
                 tc_fence_before();
                 __syncwarp();
                 if ((threadIdx.x & 31) == 0) mbar_arrive(bar(B_OEMPTY0 + t));
-            } else if (un.piece >= 0 && row < it.rows(t)) {  // this piece holds no key of tile t
+            } else if (!CL && un.piece >= 0 && row < it.rows(t)) {  // this piece holds no key of tile t
                 ws_ml[prow * 2 + 0] = -INFINITY;
                 ws_ml[prow * 2 + 1] = 0.f;
             }
+            if constexpr (CL) break;  // (un stays this CTA's piece)
             lin = next;
             un = nun;
         }
         if (!ok) {
             *abort_flag = 1;
             atomicOr(err, kDevErrTimeout);
+        }
+        if constexpr (CL) {
+            constexpr int W = D / 2;  // columns that a CTA finishes
+            const int rank = static_cast<int>(cluster_rank()), rg = t * BM + row;
+            const bool rows_on = (row & ~31) < un.it.rows(t);  // (this warp has rows of the chunk)
+            const bool tile_on = ok && un.cnt(t) > 0;
+            // the peer's columns [W][256 rows] in the group ring, its (m, l) [256 rows] in the q tiles
+            const float* peer_o = reinterpret_cast<const float*>(gbase + L::OFF_G) + rg;
+            const float2* peer_ml = reinterpret_cast<const float2*>(gbase + L::OFF_Q) + rg;
+            __syncwarp();
+            cluster_sync();  // both CTAs' MMAs are complete: their group rings and q tiles are idle
+            tc_fence_after();
+            if (rows_on) {
+                const uint32_t ml = mapa_shared(base + L::OFF_Q, static_cast<uint32_t>(rank ^ 1)) + rg * 8;
+                st_dsmem_f32(ml, __float_as_uint(cl_m));
+                st_dsmem_f32(ml + 4, __float_as_uint(tile_on ? cl_l : 0.f));
+                if (tile_on) {  // (a tile without keys here has no O to send)
+                    const uint32_t dst = mapa_shared(base + L::OFF_G, static_cast<uint32_t>(rank ^ 1)) + rg * 4;
+#pragma unroll
+                    for (int c = 0; c < W; c += 32) {
+                        uint32_t o[32];
+                        tmem_ld32(o_col + (rank ^ 1) * W + c, o);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) st_dsmem_f32(dst + (c + e) * 2 * BM * 4, o[e]);
+                    }
+                }
+            }
+            __syncwarp();
+            cluster_sync();
+            if (ok && rows_on) {
+                // (a piece without keys of this row has l = 0; its O is undefined and left out)
+                const float2 pml = *peer_ml;
+                const bool mine = tile_on && cl_l > 0.f, theirs = pml.y > 0.f;
+                const float mm = fmaxf(mine ? cl_m : -INFINITY, theirs ? pml.x : -INFINITY);
+                const float wa = mine ? fast_exp2(cl_m - mm) : 0.f, wb = theirs ? fast_exp2(pml.x - mm) : 0.f;
+                const float inv = 1.f / ((mine ? cl_l * wa : 0.f) + (theirs ? pml.y * wb : 0.f));
+                uint16_t* orow =
+                    out + ((static_cast<size_t>(un.it.b) * s_stride + un.it.q0(t) + row) * Hq + un.it.h) * D + rank * W;
+#pragma unroll
+                for (int c = 0; c < W; c += 32) {
+                    uint32_t own[32];
+                    tmem_ld32(o_col + rank * W + c, own);
+                    tmem_wait_ld();
+                    float v[32];
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) {
+                        v[e] = mine ? wa * __uint_as_float(own[e]) : 0.f;
+                        if (theirs) v[e] = fmaf(wb, peer_o[(c + e) * 2 * BM], v[e]);
+                    }
+                    if (row < un.it.rows(t))
+#pragma unroll
+                        for (int e = 0; e < 32; e += 8)
+                            *reinterpret_cast<uint4*>(orow + c + e) =
+                                make_uint4(pack_bf16x2(v[e] * inv, v[e + 1] * inv), pack_bf16x2(v[e + 2] * inv, v[e + 3] * inv),
+                                           pack_bf16x2(v[e + 4] * inv, v[e + 5] * inv), pack_bf16x2(v[e + 6] * inv, v[e + 7] * inv));
+                }
+            }
         }
     }
 
@@ -823,7 +899,19 @@ __global__ void __launch_bounds__(256) flash_combine_kernel(const float* __restr
 // and the merge kernel.
 struct HostSchedule {
     int n_pairs, n_items, head, nsplit, n_units, grid, kvb;
+    bool cluster;  // two pieces per item, one cluster each, merged in the kernel
 };
+
+// Clusters of two CTAs that fit on the device at once, per device (configure_flash_fwd).
+constexpr int kMaxDevices = 64;
+int g_pairs_fit[kMaxDevices] = {};
+static_assert(128 / 2 * 2 * BM * 4 <= GS * Layout<128>::G_SLOT && 64 / 2 * 2 * BM * 4 <= GS * Layout<64>::G_SLOT &&
+                  2 * BM * 8 <= 2 * Layout<64>::Q_TILE,
+              "the peer's columns fit in the group ring, its (m, l) in the q tiles");
+bool pairs_fit(long long items) {
+    int dev = 0;
+    return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices && items <= g_pairs_fit[dev];
+}
 
 // Items are grouped in blocks of kv heads when the history is at least the chunk and the
 // launch's K/V exceeds kKvBlockFrom; a block's K/V stays within kKvBlockBytes (of 126 MB
@@ -892,6 +980,7 @@ HostSchedule make_schedule(const Shape& s, int hist, int chunk, int num_sms) {
     sc.head = best_ns > 1 ? full_rounds * num_sms : sc.n_items;
     sc.n_units = sc.head + (sc.n_items - sc.head) * sc.nsplit;
     sc.grid = std::min(sc.n_units, num_sms);
+    sc.cluster = sc.nsplit == 2 && sc.head == 0 && sc.n_units <= num_sms && pairs_fit(sc.n_items);
     return sc;
 }
 
@@ -928,16 +1017,19 @@ cudaError_t launch_d(const Shape& s, const FlashMaps& maps, int hist, int chunk,
     kcfg.blockDim = dim3(kThreads);
     kcfg.dynamicSmemBytes = Layout<D>::ALLOC;
     kcfg.stream = st;
-    cudaLaunchAttribute kattr[1];
+    cudaLaunchAttribute kattr[2];
     kattr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     kattr[0].val.programmaticStreamSerializationAllowed = 1;
+    kattr[1].id = cudaLaunchAttributeClusterDimension;
+    kattr[1].val.clusterDim.x = 2;
+    kattr[1].val.clusterDim.y = kattr[1].val.clusterDim.z = 1;
     kcfg.attrs = kattr;
-    kcfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&kcfg, flash_fwd_kernel<D>, maps.q, maps.k, maps.v, sc, s_stride,
+    kcfg.numAttrs = hs.cluster ? 2 : 1;
+    cudaError_t e = cudaLaunchKernelEx(&kcfg, hs.cluster ? flash_fwd_kernel<D, true> : flash_fwd_kernel<D, false>, maps.q, maps.k, maps.v, sc, s_stride,
                                        s.n_kv_heads, scale_log2, cos_t, sin_t, s.max_len, out, ws_o, ws_ml, err,
                                        wait_ns);
     *n_launched = 1;
-    if (e != cudaSuccess || hs.nsplit == 1) return e;
+    if (e != cudaSuccess || hs.nsplit == 1 || hs.cluster) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(2 * (hs.n_items - hs.head)), BM / 8);
     cfg.blockDim = dim3(256);
@@ -956,18 +1048,40 @@ cudaError_t launch_d(const Shape& s, const FlashMaps& maps, int hist, int chunk,
 // with exactly kLaunchRegs registers per thread: check before any launch.
 template <int D>
 cudaError_t configure_d() {
-    cudaFuncAttributes attr;
-    cudaError_t e = cudaFuncGetAttributes(&attr, flash_fwd_kernel<D>);
-    if (e != cudaSuccess) return e;
-    if (attr.numRegs != kLaunchRegs || attr.maxThreadsPerBlock < kThreads) return cudaErrorInvalidConfiguration;
-    return cudaFuncSetAttribute(flash_fwd_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Layout<D>::ALLOC);
+    for (auto fn : {flash_fwd_kernel<D, false>, flash_fwd_kernel<D, true>}) {
+        cudaFuncAttributes attr;
+        cudaError_t e = cudaFuncGetAttributes(&attr, fn);
+        if (e != cudaSuccess) return e;
+        if (attr.numRegs != kLaunchRegs || attr.maxThreadsPerBlock < kThreads) return cudaErrorInvalidConfiguration;
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Layout<D>::ALLOC);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace
 
 cudaError_t configure_flash_fwd() {
-    const cudaError_t e = configure_d<128>();
-    return e != cudaSuccess ? e : configure_d<64>();
+    cudaError_t e = configure_d<128>();
+    if (e == cudaSuccess) e = configure_d<64>();
+    int dev = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    // (one CTA per SM at either head_dim; measured with the larger shared memory)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = Layout<128>::ALLOC;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaOccupancyMaxActiveClusters(&g_pairs_fit[dev], flash_fwd_kernel<128, true>, &cfg);
+    if (e != cudaSuccess) return e;
+    return cudaSuccess;
 }
 
 cudaError_t launch_flash_fwd(const Shape& s, const FlashMaps& maps, int hist, int chunk, int s_stride,
