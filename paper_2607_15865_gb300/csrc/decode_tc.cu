@@ -347,7 +347,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
     unsigned long long* done_ctr = reinterpret_cast<unsigned long long*>(counters + ((3 * n_items + 1) & ~1)) + ctr_row;
     // A helper split (s >= s0: a grid of several waves) first asks its item's counter for a
     // tile.  If none is left -- the item is done, or its tiles are all taken -- the CTA
-    // records its visit and leaves before any set-up.  When the batch's lengths are within
+    // records its visit and leaves before any set-up.  When the items are more than half the SMs
+    // (spec & 2) and the batch's lengths are within
     // 10% of each other (read by one warp, batches of up to 1024) there is nothing to even
     // out, and helpers leave without asking: the splits 0 then finish their items alone and
     // write the outputs without a merge.  (After the previous decode step the counters are
@@ -371,7 +372,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                     tsum += __shfl_xor_sync(0xFFFFFFFFu, tsum, off);
                 }
             }
-            const bool even = batch <= 1024 && 10LL * tmax * batch <= 11LL * tsum;
+            const bool even = (spec & 2) != 0 && batch <= 1024 && 10LL * tmax * batch <= 11LL * tsum;
             if (lane == 0) {
                 int t = -1;
                 const TokRange own = decode_tokens<D>(hist_len, hist_add, ntok, max_len);
@@ -396,7 +397,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
     // tile, tile s, before the length is known: the K slot's arrival is held back until the
     // producer knows whether tile s holds keys of the sequence (the copies read in-range
     // slots or the map's zero fill either way; a tile past the sequence is not used).
-    const bool spec_first = spec != 0 && s < s0 && s * KT < max_len;
+    // (spec & 1)
+    const bool spec_first = (spec & 1) != 0 && s < s0 && s * KT < max_len;
     if (warp == kWarpTma && lane == 0) {
         *abort_flag = 0;
         lastv[5] = 0;
@@ -1187,10 +1189,10 @@ bool decode_tc_clusters_fit(int nsplit, long long items) {
 }
 }  // namespace
 
-// Split counts.  With at most half as many (sequence, kv head, column group) items as SMs,
+// Split counts.  With few (sequence, kv head, column group) items (up to 30% of the SMs),
 // one wave of CTAs, min(16, floor(SMs / items)) splits per item, each starting with its own
 // tile.
-// With more items, kWaveSplits splits per item over several waves: split 0 of every item
+// With more items, several waves (kWaveSplits splits per item above half the SMs): split 0 of every item
 // comes first and the later splits, dispatched as SMs free up, claim what their items
 // still have (nothing, for an item that is done), so long sequences in a batch of mixed
 // lengths get help once the short ones finish.
@@ -1201,12 +1203,21 @@ constexpr int kWaveSplits = 3;
 // leaves fewer SMs idle (4 items over 32767 tokens 20.9 -> 18.9 us; head_dim 64, 2 items over 32000: 23.9 -> 15.7).
 constexpr long kMaxWaveSplits1 = 16, kMaxWaveSplitsFew = 32, kFewItems = 4;
 
+// Between 30% and 50% of the SMs in items (46 .. 76), one wave gives every item the same 2 or 3
+// splits whatever its length; one split more makes it several waves, whose claims even out
+// mixed lengths.  Calls in a graph, 64 items (28 / 4 heads B16, 32 / 8 heads B8): lengths
+// 64 .. 8183 36.0 -> 30.0 and 32.9 -> 28.1 us, one long among short 34.4 -> 25.2, all 8190
+// 46.0 -> 45.4, but all 4096 27.6 -> 29.5 (32 / 8); 48 items 35.2 -> 25.6, all 8190
+// 38.0 -> 36.6.  At 40 items an even batch loses 12% (8190: 31.0 -> 34.8).
+bool mid_items(long items, int num_sms) { return 2 * items <= num_sms && 10 * items > 3 * num_sms; }
+
 int decode_tc_column_groups(int G, int ntok) { return (G * ntok + NH - 1) / NH; }
 
 int decode_tc_num_splits(const Shape& s, int num_sms, int ncg, int ntok) {
     const long items = static_cast<long>(s.batch) * s.n_kv_heads * ncg;
     const long max_tiles = std::max(1L, static_cast<long>((s.max_len + KT - 1) / KT));
     long ns = 2 * items > num_sms ? kWaveSplits
+              : mid_items(items, num_sms) ? num_sms / items + 1
                                   : std::min<long>(items <= kFewItems ? kMaxWaveSplitsFew : kMaxWaveSplits1, num_sms / items);
     ns = std::min(ns, std::min(max_tiles, 256L));
     // The last split of an item merges ns partials of up to 16 columns in the global merge,
@@ -1218,7 +1229,7 @@ int decode_tc_num_splits(const Shape& s, int num_sms, int ncg, int ntok) {
     // at most 64 tiles (B1 Hq32 over 1024 and 4096 tokens: 11.8 -> 10.3 us and 14.1 -> 12.9 us;
     // at 32767 tokens 12 splits took 32.5 us against 29.5 us with 16).
     const long cols = std::min<long>(NH, static_cast<long>(s.n_q_heads / s.n_kv_heads) * ntok);
-    if (2 * items <= num_sms && ((ntok > 1 && ns * cols >= 128) || (ntok == 1 && max_tiles <= 64)))
+    if (2 * items <= num_sms && !mid_items(items, num_sms) && ((ntok > 1 && ns * cols >= 128) || (ntok == 1 && max_tiles <= 64)))
         while (ns > 2 && !decode_tc_clusters_fit(static_cast<int>(ns), items)) --ns;
     return static_cast<int>(std::max(1L, ns));
 }
@@ -1303,7 +1314,8 @@ cudaError_t launch_decode_tc(const Shape& s, const DecodeMaps& maps, const uint1
                               k_new, v_new, d_hist, hist_add, ntok, seq_tok, k_cache, v_cache, cos_tab, sin_tab,
                               s.n_q_heads,
                               s.n_kv_heads, s.max_len, nsplit, scale_log2, part_o, part_ml, counters, out, err,
-                              producer_early ? 1 : 0, wait_ns, ncg, after_decode ? 0 : 1, s0);
+                              producer_early ? 1 : 0, wait_ns, ncg,
+                              (after_decode ? 0 : 1) | (2LL * s.batch * s.n_kv_heads * ncg > num_sms ? 2 : 0), s0);
 }
 
 }  // namespace attn
