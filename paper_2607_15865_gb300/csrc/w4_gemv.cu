@@ -66,6 +66,7 @@ constexpr int kWarps = kThreads / 32;
 // and 2..6 stages (deeper rings cost CTAs per SM and gained nothing)
 constexpr int kTilesPerStage = 4;  // tiles (groups) per bulk copy
 constexpr int kStages = 2;         // ring depth per warp
+constexpr int kGammaBatch = 4;     // fragments whose gammas a thread loads at once (RMSNorm)
 constexpr int kUnitRows = 16;      // rows per unit (the mma M)
 constexpr int kTileBytes = 1072;   // 16 x 64 code bytes, 16 scales, 16 zero points
 constexpr int kScaleOff = 1024, kZeroOff = 1056;
@@ -262,6 +263,21 @@ __global__ void __launch_bounds__(kThreads) w4_gemv_kernel(const uint8_t* __rest
         else
             xfrag[i] = make_uint4(0u, 0u, 0u, 0u);
     }
+    // gamma's values of this thread's next kGammaBatch fragments (gamma is 8-byte aligned); the
+    // first batch arrives with x
+    const int n_frag = ngroup * 4 * 4 * MT;
+    uint2 ga[kGammaBatch], gc[kGammaBatch];
+    auto load_gamma = [&](int i0) {
+#pragma unroll
+        for (int j = 0; j < kGammaBatch; ++j) {
+            const int i = i0 + j * kThreads;
+            if (i >= n_frag) break;
+            const int gi = i / (4 * MT), k0 = 128 * (gi >> 2) + 32 * (i & 3) + 8 * (gi & 3);
+            ga[j] = __ldg(reinterpret_cast<const uint2*>(fz.gamma + k0));
+            gc[j] = __ldg(reinterpret_cast<const uint2*>(fz.gamma + k0 + 4));
+        }
+    };
+    if (fz.gamma != nullptr) load_gamma(tid);
     cp_async_wait_all();
     __syncthreads();
     if (fz.gamma != nullptr) {
@@ -270,7 +286,7 @@ __global__ void __launch_bounds__(kThreads) w4_gemv_kernel(const uint8_t* __rest
         // is the same for all its elements (the stride divides by 4 * MT).
         const int slot = tid % (4 * MT), m = slot >> 2;
         float ss = 0.f;
-        for (int i = tid; i < ngroup * 4 * 4 * MT; i += kThreads) {
+        for (int i = tid; i < n_frag; i += kThreads) {
             const uint4 v = xfrag[i];
             const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -282,24 +298,23 @@ __global__ void __launch_bounds__(kThreads) w4_gemv_kernel(const uint8_t* __rest
         for (int off = 4 * MT; off < 32; off <<= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, off);
         if ((lane & 3) == 0 && lane < 4 * MT) red[warp * 8 + m] = ss;
         __syncthreads();
-        if (tid < MT) {
-            float tot = 0.f;
-            for (int w = 0; w < kWarps; ++w) tot += red[w * 8 + tid];
-            red[kWarps * 8 + tid] = 1.f / sqrtf(tot / static_cast<float>(K) + fz.eps);
-        }
-        __syncthreads();
-        const float r = red[kWarps * 8 + m];
-        for (int i = tid; i < ngroup * 4 * 4 * MT; i += kThreads) {
-            if (m >= M) break;
-            const int gi = i / (4 * MT), tt = slot & 3;
-            const int k0 = 128 * (gi >> 2) + 32 * tt + 8 * (gi & 3);
-            // (gamma is 8-byte aligned)
-            const uint2 ga = *reinterpret_cast<const uint2*>(fz.gamma + k0), gc = *reinterpret_cast<const uint2*>(fz.gamma + k0 + 4);
-            const uint4 v = xfrag[i];
-            xfrag[i] = make_uint4(pack_bf16x2(bf16_lo(v.x) * r * bf16_lo(ga.x), bf16_hi(v.x) * r * bf16_hi(ga.x)),
-                                  pack_bf16x2(bf16_lo(v.y) * r * bf16_lo(ga.y), bf16_hi(v.y) * r * bf16_hi(ga.y)),
-                                  pack_bf16x2(bf16_lo(v.z) * r * bf16_lo(gc.x), bf16_hi(v.z) * r * bf16_hi(gc.x)),
-                                  pack_bf16x2(bf16_lo(v.w) * r * bf16_lo(gc.y), bf16_hi(v.w) * r * bf16_hi(gc.y)));
+        float tot = 0.f;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) tot += red[w * 8 + m];
+        const float r = 1.f / sqrtf(tot / static_cast<float>(K) + fz.eps);
+        for (int i0 = tid; i0 < n_frag && m < M; i0 += kGammaBatch * kThreads) {
+            if (i0 != tid) load_gamma(i0);
+#pragma unroll
+            for (int j = 0; j < kGammaBatch; ++j) {
+                const int i = i0 + j * kThreads;
+                if (i >= n_frag) break;
+                const uint4 v = xfrag[i];
+                xfrag[i] =
+                    make_uint4(pack_bf16x2(bf16_lo(v.x) * r * bf16_lo(ga[j].x), bf16_hi(v.x) * r * bf16_hi(ga[j].x)),
+                               pack_bf16x2(bf16_lo(v.y) * r * bf16_lo(ga[j].y), bf16_hi(v.y) * r * bf16_hi(ga[j].y)),
+                               pack_bf16x2(bf16_lo(v.z) * r * bf16_lo(gc[j].x), bf16_hi(v.z) * r * bf16_hi(gc[j].x)),
+                               pack_bf16x2(bf16_lo(v.w) * r * bf16_lo(gc[j].y), bf16_hi(v.w) * r * bf16_hi(gc[j].y)));
+            }
         }
         __syncthreads();
     }
