@@ -39,6 +39,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
@@ -875,12 +876,28 @@ __global__ void __launch_bounds__(256) flash_combine_kernel(const float* __restr
         float acc[PER_LANE];
 #pragma unroll
         for (int e = 0; e < PER_LANE; ++e) acc[e] = 0.f;
-        for (int sp = 0; sp < nsplit; ++sp) {
-            const float ws = __shfl_sync(0xFFFFFFFFu, w, sp);
-            if (ws == 0.f) continue;  // a piece without keys of this tile: its O was never written
-            const float* src = ws_o + ((v0 + sp) * 2 * BM + t * BM + row) * D + lane * PER_LANE;
+        // A batch of pieces is loaded at once, a lane's columns in one load: the loop was a chain of
+        // one piece's loads after another (16 tokens over 2000, 24 heads: 16.4 -> 13.6 us; 100 over
+        // 3000, 28 heads: 19.3 -> 16.9).  At head_dim 64 a batch of 4: 8 made 256 over 1500 3% slower.
+        using Vec = std::conditional_t<D == 128, float4, float2>;
+        constexpr int kMergeBatch = D == 128 ? 8 : 4;
+        for (int s0 = 0; s0 < nsplit; s0 += kMergeBatch) {
+            Vec o[kMergeBatch];
+            float ws[kMergeBatch];
 #pragma unroll
-            for (int e = 0; e < PER_LANE; ++e) acc[e] = fmaf(ws, src[e], acc[e]);
+            for (int u = 0; u < kMergeBatch; ++u) {
+                ws[u] = s0 + u < nsplit ? __shfl_sync(0xFFFFFFFFu, w, s0 + u) : 0.f;
+                if (ws[u] != 0.f)  // (a piece without keys of this tile never wrote its O)
+                    o[u] = *reinterpret_cast<const Vec*>(ws_o + ((v0 + s0 + u) * 2 * BM + t * BM + row) * D +
+                                                         lane * PER_LANE);
+            }
+#pragma unroll
+            for (int u = 0; u < kMergeBatch; ++u) {
+                const float* src = reinterpret_cast<const float*>(&o[u]);
+#pragma unroll
+                for (int e = 0; e < PER_LANE; ++e)
+                    if (ws[u] != 0.f) acc[e] = fmaf(ws[u], src[e], acc[e]);
+            }
         }
         const float inv = 1.f / lw;
         uint16_t* dst = out + ((static_cast<size_t>(it.b) * s_stride + it.q0(t) + row) * Hq + it.h) * D + lane * PER_LANE;
