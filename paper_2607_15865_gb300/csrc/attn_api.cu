@@ -160,7 +160,8 @@ int run_prefill(attn_ctx* c, const uint16_t* q, const uint16_t* k, const uint16_
                                     static_cast<cuuint64_t>(s.batch)};
         const cuuint64_t strides[3] = {D * 2, D * 2 * s.n_q_heads,
                                        D * 2 * s.n_q_heads * static_cast<cuuint64_t>(seq_stride)};
-        const cuuint32_t box[4] = {64, 1, 128, 1};
+        const cuuint32_t heads = static_cast<cuuint32_t>(attn::flash_pack_heads(s, hist, chunk, c->num_sms));
+        const cuuint32_t box[4] = {64, heads, 128 / heads, 1};
         const int rc = encode_map(c, &maps.q, q, 4, dims, strides, box);
         if (rc != ATTN_OK) return rc;
     }

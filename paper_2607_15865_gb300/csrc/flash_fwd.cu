@@ -10,8 +10,9 @@
 // with_history template, Section 4.2).
 //
 // Design.  A persistent CTA per SM walks a static list of work items sorted
-// longest-first, dealt out in rounds of alternating direction.  An item is two 128-row query tiles (A, B) of one head, so each
-// K/V tile is brought in once for 256 queries.  384 threads, three warpgroups:
+// longest-first, dealt out in rounds of alternating direction.  An item is two 128-row query
+// tiles (A, B) of one head (of all heads of a kv head, where short chunks pack them into the
+// rows), so each K/V tile is brought in once for 256 rows.  384 threads, three warpgroups:
 //   WG0 (warps 0-3)   softmax + epilogue of tile A (one thread per row = TMEM lane)
 //   WG1 (warps 4-7)   softmax + epilogue of tile B
 //   WG2 (warps 8-11)  warp 8: TMA producer (lane 0: q tiles from a 4-D map of
@@ -110,7 +111,9 @@ __device__ __forceinline__ uint32_t sw128_offset(int row, int col) {
     return static_cast<uint32_t>(chunk * (128 * 128) + row * 128 + ((unit ^ (row & 7)) << 4));
 }
 
-// One work item: query tiles A (rows q0(0)..) and B (rows q0(1)..) of head h, sequence b.
+// One work item: query tiles A (tokens q0(0)..) and B (tokens q0(1)..) of head h, sequence b.  A
+// tile row is a token; with packed heads (PK) it is one of the query heads h .. of a kv head at a
+// token: row r is token r / heads, head h + r mod heads (see flash_pack_heads).
 // Scalar fields with select accessors keep every field in registers when the tile
 // index is only known at run time.
 struct Item {
@@ -124,7 +127,9 @@ struct Item {
     __device__ __forceinline__ int nkv(int t) const { return t ? nkvb : nkva; }
 };
 
-// The launch's work list: chunk S at history H, Hq query heads, batch sequences, n_pairs
+// The launch's work list: chunk S at history H, Hq groups of `heads` query heads that share
+// tiles of tok tokens (PK; 1 and BM else), n_heads heads in all, G groups per kv head, batch
+// sequences, n_pairs
 // query-tile pairs per (head, sequence); `head` items whole, the rest cut into nsplit
 // pieces; with the divisors the kernels use, as fast divisions (every division of the
 // schedule ran as a generic integer division before: about 1 us per decoded unit).
@@ -132,6 +137,8 @@ struct Sched {
     int S, H, Hq, G, batch, n_pairs, head, nsplit, n_units;
     int kvb;  // item order: 0 longest pairs first over all heads, else blocks of kvb kv heads
     FastDiv fd_grid, fd_hqb, fd_hq, fd_g, fd_ns, fd_pb, fd_per, fd_nb;
+    int n_heads, heads, tok;
+    FastDiv fd_heads;
 };
 
 // Item order.  By default the longest query-tile pairs come first across every (head,
@@ -142,6 +149,7 @@ struct Sched {
 // a pair together -- so the CTAs of a round walk the K/V of only those kv heads, which
 // stays in L2, and each kv head's cache is read from DRAM about once instead of once per
 // round.
+template <bool PK>
 __device__ __forceinline__ Item decode_item(int lin, const Sched& sc) {
     Item it;
     int qt;
@@ -160,15 +168,37 @@ __device__ __forceinline__ Item decode_item(int lin, const Sched& sc) {
         it.h = rem - it.b * sc.Hq;
         it.g = fdiv(it.h, sc.fd_g);
     }
+    if constexpr (PK) it.h *= sc.heads;
     const int pt = sc.n_pairs - 1 - qt;
-    it.q0a = pt * 2 * BM;
-    it.q0b = it.q0a + BM;
-    it.rowsa = max(0, min(BM, sc.S - it.q0a));
-    it.rowsb = max(0, min(BM, sc.S - it.q0b));
+    const int tok = PK ? sc.tok : BM;
+    it.q0a = pt * 2 * tok;
+    it.q0b = it.q0a + tok;
+    it.rowsa = max(0, min(tok, sc.S - it.q0a));  // (tokens)
+    it.rowsb = max(0, min(tok, sc.S - it.q0b));
     it.nkva = it.rowsa ? (sc.H + it.q0a + it.rowsa + BN - 1) / BN : 0;
     it.nkvb = it.rowsb ? (sc.H + it.q0b + it.rowsb + BN - 1) / BN : 0;
+    if constexpr (PK) {
+        it.rowsa *= sc.heads;
+        it.rowsb *= sc.heads;
+    }
     it.n_kv = max(it.nkva, it.nkvb);
     return it;
+}
+
+// Token of a tile's row `row` (relative to the tile's first), and the element offsets in `out` of
+// the row (relative to row 0) and of tile t's token `token`, head h.
+template <bool PK>
+__device__ __forceinline__ int row_token(int row, const Sched& sc) {
+    return PK ? fdiv(row, sc.fd_heads) : row;
+}
+template <bool PK>
+__device__ __forceinline__ size_t row_offset(int row, const Sched& sc, int D) {
+    const int tk = row_token<PK>(row, sc);
+    return (static_cast<size_t>(tk) * (PK ? sc.n_heads : sc.Hq) + (PK ? row - tk * sc.heads : 0)) * D;
+}
+template <bool PK>
+__device__ __forceinline__ size_t item_offset(const Item& it, int t, int token, const Sched& sc, int s_stride, int D) {
+    return ((static_cast<size_t>(it.b) * s_stride + it.q0(t) + token) * (PK ? sc.n_heads : sc.Hq) + it.h) * D;
 }
 
 // A work unit: a whole item, or one KV-range piece of an item from the tail of the
@@ -182,6 +212,7 @@ struct Unit {
     __device__ __forceinline__ int cnt(int t) const { return max(0, min(kv_hi, it.nkv(t)) - kv_lo); }
 };
 
+template <bool PK>
 __device__ __forceinline__ Unit decode_unit(int lin, const Sched& sc) {
     Unit u;
     u.piece = -1;
@@ -190,11 +221,11 @@ __device__ __forceinline__ Unit decode_unit(int lin, const Sched& sc) {
         const int tail = fdiv(v, sc.fd_ns);
         const int s = v - tail * sc.nsplit;
         u.piece = v;
-        u.it = decode_item(sc.head + tail, sc);
+        u.it = decode_item<PK>(sc.head + tail, sc);
         u.kv_lo = fdiv(u.it.n_kv * s, sc.fd_ns);
         u.kv_hi = fdiv(u.it.n_kv * (s + 1), sc.fd_ns);
     } else {
-        u.it = decode_item(lin, sc);
+        u.it = decode_item<PK>(lin, sc);
         u.kv_lo = 0;
         u.kv_hi = u.it.n_kv;
     }
@@ -278,16 +309,23 @@ __device__ __forceinline__ void rope_row_smem(uint8_t* qtile, int row, const Rop
     }
 }
 
-// Wait for an item's q tiles, rotate this thread's row, hand Q to the MMA warp.
-template <int D>
+// Wait for an item's q tiles, rotate this thread's row, hand Q to the MMA warp.  Packed heads
+// leave the tile's last 128 mod heads rows to no copy: they are zeroed.
+template <int D, bool PK>
 __device__ __forceinline__ bool rope_item(uint32_t qfull, uint32_t qready, uint32_t parity, const volatile int* abort,
-                                          uint8_t* qtile, int row, int rows, int pos0,
+                                          uint8_t* qtile, int row, int row_tok, int rows, int pos0, int copied_rows,
                                           const float* __restrict__ cos_t, const float* __restrict__ sin_t,
                                           int stride, uint64_t wait_ns) {
     RopeRow<D> tabs;
-    rope_load<D>(tabs, row < rows ? pos0 + row : pos0, cos_t, sin_t, stride);
+    rope_load<D>(tabs, row < rows ? pos0 + row_tok : pos0, cos_t, sin_t, stride);
     const bool w = __all_sync(0xFFFFFFFFu, mbar_wait(qfull, parity, abort, wait_ns));
     if (w && row < rows) rope_row_smem<D>(qtile, row, tabs);
+    if (PK && row >= copied_rows) {
+#pragma unroll
+        for (int u = 0; u < D / 8; ++u)
+            *reinterpret_cast<uint4*>(qtile + (u >> 3) * Layout<D>::CHUNK + row * 128 + (u & 7) * 16) =
+                make_uint4(0, 0, 0, 0);
+    }
     fence_proxy_async_smem();
     __syncwarp();
     if ((threadIdx.x & 31) == 0) mbar_arrive(qready);
@@ -302,7 +340,7 @@ __device__ __forceinline__ bool rope_item(uint32_t qfull, uint32_t qready, uint3
 // reads 17 MB of partials, 24.3 with this; 512 over 8000 63.7 -> 61.9.  With more pieces the
 // larger cluster and its longer exchange cost more than the merge kernel: four of 256 rows over
 // 1500 24.3 us against 22.2, of one row over 2000 15.6 against 14.0.)
-template <int D, bool CL>
+template <int D, bool CL, bool PK>
 __global__ void __launch_bounds__(kThreads, 1)
     flash_fwd_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_v, const Sched sc, int s_stride, int Hkv,
@@ -320,7 +358,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int S = sc.S, H = sc.H, Hq = sc.Hq, n_units = sc.n_units;
+    const int H = sc.H, n_units = sc.n_units;
 
     if (warp == kWarpTma && lane == 0) {
         // Barriers, then the first unit's q tiles right away: their copy overlaps the TMEM
@@ -346,8 +384,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         tma_prefetch_desc(&map_k);
         tma_prefetch_desc(&map_v);
         if (static_cast<int>(blockIdx.x) < n_units) {
-            const Item it = decode_unit(unit_of(blockIdx.x, sc), sc).it;
-            mbar_arrive_expect_tx(bar(B_QFULL), 2 * L::Q_TILE);
+            const Item it = decode_unit<PK>(unit_of(blockIdx.x, sc), sc).it;
+            mbar_arrive_expect_tx(bar(B_QFULL), PK ? 2 * L::DCH * 128 * sc.tok * sc.heads : 2 * L::Q_TILE);
 #pragma unroll
             for (int t = 0; t < 2; ++t)
 #pragma unroll
@@ -377,14 +415,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             bool ok = true;
             bool kv_visible = false;  // K1's cache writes complete (dependent launch)
             for (int lin = blockIdx.x; lin < n_units && ok; lin += gridDim.x) {
-                const Unit un = decode_unit(unit_of(lin, sc), sc);
+                const Unit un = decode_unit<PK>(unit_of(lin, sc), sc);
                 const Item& it = un.it;
                 if (items > 0) {  // (the first unit's q tiles were issued in the prologue)
                     if (!mbar_wait(bar(B_QEMPTY), static_cast<uint32_t>(items - 1) & 1u, abort_flag, wait_ns)) {
                         ok = false;
                         break;
                     }
-                    mbar_arrive_expect_tx(bar(B_QFULL), 2 * L::Q_TILE);
+                    mbar_arrive_expect_tx(bar(B_QFULL), PK ? 2 * L::DCH * 128 * sc.tok * sc.heads : 2 * L::Q_TILE);
 #pragma unroll
                     for (int t = 0; t < 2; ++t)
 #pragma unroll
@@ -397,7 +435,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // the next unit's q tiles into L2, so that their copy after this unit is short
                     const int nxt = lin + static_cast<int>(gridDim.x);
                     if (nxt < n_units) {
-                        const Item nt = decode_unit(unit_of(nxt, sc), sc).it;
+                        const Item nt = decode_unit<PK>(unit_of(nxt, sc), sc).it;
 #pragma unroll
                         for (int t = 0; t < 2; ++t)
                             if (nt.rows(t) > 0)
@@ -492,7 +530,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 gslot = gslot + 1 == GS ? 0 : gslot + 1;
             };
             for (int lin = blockIdx.x; lin < n_units && ok; lin += gridDim.x) {
-                const Unit un = decode_unit(unit_of(lin, sc), sc);
+                const Unit un = decode_unit<PK>(unit_of(lin, sc), sc);
                 const Item& it = un.it;
                 if (!mbar_wait(bar(B_QREADY), static_cast<uint32_t>(items) & 1u, abort_flag, wait_ns)) {
                     ok = false;
@@ -574,6 +612,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         warpgroup_reg_inc<kRegsHigh>();
         const int t = warp >> 2;            // query tile of this warpgroup
         const int row = threadIdx.x & 127;  // row in the tile == TMEM lane
+        const int q_rows = PK ? sc.tok * sc.heads : BM;  // rows that the q copies write
+        const int row_tok = row_token<PK>(row, sc);
         const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
         const uint32_t s_col = tmem + lane_base + t * BN;
         const uint32_t o_col = tmem + lane_base + L::TM_O + t * D;
@@ -586,16 +626,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         int lin = blockIdx.x;
         Unit un;
         if (lin < n_units) {
-            un = decode_unit(unit_of(lin, sc), sc);
-            ok = rope_item<D>(bar(B_QFULL), bar(B_QREADY), static_cast<uint32_t>(items) & 1u, abort_flag, qtile, row,
-                              un.it.rows(t), H + un.it.q0(t), cos_t, sin_t, tab_stride, wait_ns);
+            un = decode_unit<PK>(unit_of(lin, sc), sc);
+            ok = rope_item<D, PK>(bar(B_QFULL), bar(B_QREADY), static_cast<uint32_t>(items) & 1u, abort_flag, qtile,
+                                  row, row_tok, un.it.rows(t), H + un.it.q0(t), q_rows, cos_t, sin_t, tab_stride, wait_ns);
             ++items;
         }
         while (lin < n_units && ok) {
             const Item& it = un.it;
             float m_run = -INFINITY;  // reference max of P (log2 domain)
             float l_run = 0.f;
-            const int pos_row = H + it.q0(t) + row;  // last key this row may see
+            const int pos_row = H + it.q0(t) + row_tok;  // last key this row may see
             const int min_pos = H + it.q0(t);        // smallest row position of the tile
             const int n_tiles = un.cnt(t);
             for (int j = un.kv_lo; j < un.kv_lo + n_tiles; ++j) {
@@ -683,9 +723,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int next = lin + static_cast<int>(gridDim.x);
             Unit nun;
             if (next < n_units) {
-                nun = decode_unit(unit_of(next, sc), sc);
-                ok = rope_item<D>(bar(B_QFULL), bar(B_QREADY), static_cast<uint32_t>(items) & 1u, abort_flag, qtile,
-                                  row, nun.it.rows(t), H + nun.it.q0(t), cos_t, sin_t, tab_stride, wait_ns);
+                nun = decode_unit<PK>(unit_of(next, sc), sc);
+                ok = rope_item<D, PK>(bar(B_QFULL), bar(B_QREADY), static_cast<uint32_t>(items) & 1u, abort_flag, qtile,
+                                      row, row_tok, nun.it.rows(t), H + nun.it.q0(t), q_rows, cos_t, sin_t, tab_stride, wait_ns);
                 ++items;
                 if (!ok) break;
             }
@@ -706,7 +746,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const float inv_l = 1.f / l_run;
                     const int lane = threadIdx.x & 31, r0 = row & ~31;
                     uint8_t* stage = gbase + L::OFF_STAGE + warp * L::STAGE_WARP;
-                    uint16_t* obase = out + ((static_cast<size_t>(it.b) * s_stride + it.q0(t) + r0) * Hq + it.h) * D;
+                    uint16_t* obase = out + item_offset<PK>(it, t, PK ? 0 : r0, sc, s_stride, D);
 #pragma unroll
                     for (int c2 = 0; c2 < D / 64; ++c2) {
                         uint32_t o[2][32];
@@ -726,7 +766,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                             const int rr = 4 * i + (lane >> 3), ch = lane & 7;
                             const uint4 u = *reinterpret_cast<const uint4*>(stage + rr * 128 + ((ch ^ (rr & 7)) << 4));
                             if (r0 + rr < it.rows(t))
-                                *reinterpret_cast<uint4*>(obase + static_cast<size_t>(rr) * Hq * D + 64 * c2 + 8 * ch) = u;
+                                *reinterpret_cast<uint4*>(obase + row_offset<PK>(PK ? r0 + rr : rr, sc, D) + 64 * c2 +
+                                                          8 * ch) = u;
                         }
                         __syncwarp();
                     }
@@ -811,8 +852,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const float mm = fmaxf(mine ? cl_m : -INFINITY, theirs ? pml.x : -INFINITY);
                 const float wa = mine ? fast_exp2(cl_m - mm) : 0.f, wb = theirs ? fast_exp2(pml.x - mm) : 0.f;
                 const float inv = 1.f / ((mine ? cl_l * wa : 0.f) + (theirs ? pml.y * wb : 0.f));
-                uint16_t* orow =
-                    out + ((static_cast<size_t>(un.it.b) * s_stride + un.it.q0(t) + row) * Hq + un.it.h) * D + rank * W;
+                uint16_t* orow = out + item_offset<PK>(un.it, t, PK ? 0 : row, sc, s_stride, D) +
+                                 (PK ? row_offset<PK>(row, sc, D) : 0) + rank * W;
 #pragma unroll
                 for (int c = 0; c < W; c += 32) {
                     uint32_t own[32];
@@ -846,16 +887,16 @@ __global__ void __launch_bounds__(kThreads, 1)
 // Merges the pieces of each tail item: for every row, m* = max m_s over pieces with
 // l_s > 0, out = sum_s 2^(m_s - m*) O_s / sum_s 2^(m_s - m*) l_s -> bf16.
 // Block (tail item, query tile, group of 8 rows); one warp per row.
-template <int D>
+template <int D, bool PK>
 __global__ void __launch_bounds__(256) flash_combine_kernel(const float* __restrict__ ws_o,
                                                             const float* __restrict__ ws_ml, const Sched sc,
                                                             int s_stride, uint16_t* __restrict__ out) {
     constexpr int PER_LANE = D / 32;
     asm volatile("griddepcontrol.wait;" ::: "memory");  // the pieces are complete and visible
-    const int head = sc.head, nsplit = sc.nsplit, Hq = sc.Hq;
+    const int head = sc.head, nsplit = sc.nsplit;
     const int item = head + static_cast<int>(blockIdx.x) / 2;
     const int t = static_cast<int>(blockIdx.x) % 2;
-    const Item it = decode_item(item, sc);
+    const Item it = decode_item<PK>(item, sc);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row = static_cast<int>(blockIdx.y) * 8 + warp;
     if (row < it.rows(t)) {
@@ -900,7 +941,7 @@ __global__ void __launch_bounds__(256) flash_combine_kernel(const float* __restr
             }
         }
         const float inv = 1.f / lw;
-        uint16_t* dst = out + ((static_cast<size_t>(it.b) * s_stride + it.q0(t) + row) * Hq + it.h) * D + lane * PER_LANE;
+        uint16_t* dst = out + item_offset<PK>(it, t, 0, sc, s_stride, D) + row_offset<PK>(row, sc, D) + lane * PER_LANE;
 #pragma unroll
         for (int e = 0; e < PER_LANE; e += 2)
             *reinterpret_cast<uint32_t*>(dst + e) = pack_bf16x2(acc[e] * inv, acc[e + 1] * inv);
@@ -916,6 +957,7 @@ __global__ void __launch_bounds__(256) flash_combine_kernel(const float* __restr
 // and the merge kernel.
 struct HostSchedule {
     int n_pairs, n_items, head, nsplit, n_units, grid, kvb;
+    int heads;     // query heads that share a tile's rows
     bool cluster;  // two pieces per item, one cluster each, merged in the kernel
 };
 
@@ -946,10 +988,13 @@ int unit_of_host(int lin, int g, int n_units) {
 
 HostSchedule make_schedule(const Shape& s, int hist, int chunk, int num_sms) {
     HostSchedule sc;
-    const int n_qtiles = (chunk + BM - 1) / BM;
+    const int heads = sc.heads = flash_pack_heads(s, hist, chunk, num_sms);
+    const int tok = BM / heads;  // tokens of a tile
+    const int n_qtiles = (chunk + tok - 1) / tok;
     sc.n_pairs = (n_qtiles + 1) / 2;
-    sc.n_items = sc.n_pairs * s.n_q_heads * s.batch;
-    const int hq_b = s.n_q_heads * s.batch, G = s.n_q_heads / s.n_kv_heads;
+    const int hq = s.n_q_heads / heads;
+    sc.n_items = sc.n_pairs * hq * s.batch;
+    const int hq_b = hq * s.batch, G = hq / s.n_kv_heads;
     const double head_bytes = 4.0 * (static_cast<double>(hist) + chunk) * s.head_dim;  // K/V of one kv head
     sc.kvb = 0;
     if (hist >= chunk && head_bytes * s.batch * s.n_kv_heads > kKvBlockFrom) {
@@ -960,7 +1005,7 @@ HostSchedule make_schedule(const Shape& s, int hist, int chunk, int num_sms) {
     auto n_kv = [&](int item) {  // KV tiles of an item (longest pairs first, in either order)
         const int qt = sc.kvb ? item % (sc.n_pairs * sc.kvb * G) / (sc.kvb * G) : item / hq_b;
         const int pt = sc.n_pairs - 1 - qt;
-        return (hist + std::min(2 * BM * (pt + 1), chunk) + BN - 1) / BN;
+        return (hist + std::min(2 * tok * (pt + 1), chunk) + BN - 1) / BN;
     };
     // costs in KV steps of both query tiles (about 1.3 us each)
     const double c_unit = 1.6, c_split = 2.5, c_step = 1.0;
@@ -1009,8 +1054,12 @@ cudaError_t launch_d(const Shape& s, const FlashMaps& maps, int hist, int chunk,
     Sched sc;
     sc.S = chunk;
     sc.H = hist;
-    sc.Hq = s.n_q_heads;
-    sc.G = s.n_q_heads / s.n_kv_heads;
+    sc.heads = hs.heads;
+    sc.tok = BM / hs.heads;
+    sc.fd_heads = make_fastdiv(hs.heads);
+    sc.n_heads = s.n_q_heads;
+    sc.Hq = s.n_q_heads / hs.heads;
+    sc.G = sc.Hq / s.n_kv_heads;
     sc.batch = s.batch;
     sc.kvb = hs.kvb;
     sc.n_pairs = hs.n_pairs;
@@ -1018,14 +1067,14 @@ cudaError_t launch_d(const Shape& s, const FlashMaps& maps, int hist, int chunk,
     sc.nsplit = hs.nsplit;
     sc.n_units = hs.n_units;
     sc.fd_grid = make_fastdiv(hs.grid);
-    sc.fd_hqb = make_fastdiv(s.n_q_heads * s.batch);
-    sc.fd_hq = make_fastdiv(s.n_q_heads);
-    sc.fd_g = make_fastdiv(s.n_q_heads / s.n_kv_heads);
+    sc.fd_hqb = make_fastdiv(sc.Hq * s.batch);
+    sc.fd_hq = make_fastdiv(sc.Hq);
+    sc.fd_g = make_fastdiv(sc.G);
     sc.fd_ns = make_fastdiv(hs.nsplit);
     const int per = std::max(hs.kvb, 1) * sc.G;
     sc.fd_pb = make_fastdiv(hs.n_pairs * per);
     sc.fd_per = make_fastdiv(per);
-    sc.fd_nb = make_fastdiv(s.n_q_heads / per);
+    sc.fd_nb = make_fastdiv(sc.Hq / per);
     const float scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(D)));
     // Dependent launch after K1 (programmatic stream serialization): only the producer's
     // first K/V copy waits for K1 (griddep_wait).
@@ -1042,9 +1091,11 @@ cudaError_t launch_d(const Shape& s, const FlashMaps& maps, int hist, int chunk,
     kattr[1].val.clusterDim.y = kattr[1].val.clusterDim.z = 1;
     kcfg.attrs = kattr;
     kcfg.numAttrs = hs.cluster ? 2 : 1;
-    cudaError_t e = cudaLaunchKernelEx(&kcfg, hs.cluster ? flash_fwd_kernel<D, true> : flash_fwd_kernel<D, false>, maps.q, maps.k, maps.v, sc, s_stride,
-                                       s.n_kv_heads, scale_log2, cos_t, sin_t, s.max_len, out, ws_o, ws_ml, err,
-                                       wait_ns);
+    const bool pk = hs.heads > 1;
+    const auto fwd = hs.cluster ? (pk ? flash_fwd_kernel<D, true, true> : flash_fwd_kernel<D, true, false>)
+                                : (pk ? flash_fwd_kernel<D, false, true> : flash_fwd_kernel<D, false, false>);
+    cudaError_t e = cudaLaunchKernelEx(&kcfg, fwd, maps.q, maps.k, maps.v, sc, s_stride, s.n_kv_heads,
+                                       scale_log2, cos_t, sin_t, s.max_len, out, ws_o, ws_ml, err, wait_ns);
     *n_launched = 1;
     if (e != cudaSuccess || hs.nsplit == 1 || hs.cluster) return e;
     cudaLaunchConfig_t cfg = {};
@@ -1056,7 +1107,8 @@ cudaError_t launch_d(const Shape& s, const FlashMaps& maps, int hist, int chunk,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, flash_combine_kernel<D>, ws_o, ws_ml, sc, s_stride, out);
+    e = cudaLaunchKernelEx(&cfg, pk ? flash_combine_kernel<D, true> : flash_combine_kernel<D, false>, ws_o, ws_ml, sc,
+                           s_stride, out);
     *n_launched = 2;
     return e;
 }
@@ -1065,7 +1117,8 @@ cudaError_t launch_d(const Shape& s, const FlashMaps& maps, int hist, int chunk,
 // with exactly kLaunchRegs registers per thread: check before any launch.
 template <int D>
 cudaError_t configure_d() {
-    for (auto fn : {flash_fwd_kernel<D, false>, flash_fwd_kernel<D, true>}) {
+    for (auto fn : {flash_fwd_kernel<D, false, false>, flash_fwd_kernel<D, true, false>,
+                    flash_fwd_kernel<D, false, true>, flash_fwd_kernel<D, true, true>}) {
         cudaFuncAttributes attr;
         cudaError_t e = cudaFuncGetAttributes(&attr, fn);
         if (e != cudaSuccess) return e;
@@ -1077,6 +1130,27 @@ cudaError_t configure_d() {
 }
 
 }  // namespace
+
+// A chunk of up to a tile leaves tile rows empty, and every query head of a kv head walks the
+// same keys once per head: packed, the heads share the rows and the walk (the work of the tensor
+// cores and the exponentials of the empty rows go with it).  Where the heads of all the chunk's
+// tokens fill one tile that pays from four key steps on: it is the same walk for fewer items, cut
+// into more pieces (16 tokens over 8000, 40 heads: 35.0 -> 16.3 us; 1 over 2000: 16.2 -> 10.3; 16
+// over 380: 11.6 -> 9.4); with one to three steps there is nothing to cut and the row arithmetic
+// costs 0.1-0.4 us (16 over 250: 10.5 -> 10.7), unless the items are more than the SMs (16
+// sequences, 16 tokens without history: 22.8 -> 9.3).
+// With more rows an item becomes two tiles per key step and its pieces write more partial rows,
+// which only pays once the walk is long: 8 key steps per SM, or two whole rounds of items (32
+// heads, 128 over 8000: 31.8 -> 25.2 us, 128 over 20000: 61 -> 40, 16 sequences of 100 over 500:
+// 45.8 -> 32; below the line 100 over 3000 21.2 -> 21.9 and 4 sequences of 64 over 500 14.0 -> 17.0,
+// both before the merge loaded in batches).
+int flash_pack_heads(const Shape& s, int hist, int chunk, int num_sms) {
+    const int G = s.n_q_heads / s.n_kv_heads;
+    if (G == 1 || chunk > BM) return 1;
+    const long long items = static_cast<long long>(s.n_q_heads) * s.batch, steps = (hist + chunk + BN - 1) / BN;
+    if (chunk * G <= BM && (steps >= 4 || items > num_sms)) return G;
+    return items >= 2LL * num_sms || items * steps >= 8LL * num_sms ? G : 1;
+}
 
 cudaError_t configure_flash_fwd() {
     cudaError_t e = configure_d<128>();
@@ -1096,7 +1170,7 @@ cudaError_t configure_flash_fwd() {
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaOccupancyMaxActiveClusters(&g_pairs_fit[dev], flash_fwd_kernel<128, true>, &cfg);
+    e = cudaOccupancyMaxActiveClusters(&g_pairs_fit[dev], flash_fwd_kernel<128, true, false>, &cfg);
     if (e != cudaSuccess) return e;
     return cudaSuccess;
 }

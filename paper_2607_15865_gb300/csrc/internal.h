@@ -63,8 +63,10 @@ cudaError_t launch_rope_append(const Shape& s, const uint16_t* k, const uint16_t
 
 // K2: causal flash attention of `chunk` new queries at positions hist.. over cache
 // slots [0, hist+chunk) (prefill: hist=0).  RoPE of q is applied in the kernel.
+// Query heads that share a query tile's 128 rows: all of a kv head's, or 1.
+int flash_pack_heads(const Shape& s, int hist, int chunk, int num_sms);
 struct FlashMaps {
-    CUtensorMap q;  // q [B, S, Hq, D] as 4-D {D, Hq, S, B}; box {64, 1, 128, 1}
+    CUtensorMap q;  // q [B, S, Hq, D] as 4-D {D, Hq, S, B}; box {64, heads, 128 / heads, 1} (flash_pack_heads)
     CUtensorMap k;  // k_cache as 3-D {D, hist+chunk, B*Hkv}; box {64, 128, 1}
     CUtensorMap v;  // v_cache, same as k
 };
