@@ -14,9 +14,9 @@
 //   S^T [128 keys x 16] = K_tile [128 x D] . Q^T       (Q: C columns, zero-padded to 16)
 //   O^T [D x 16]      += V_tile^T [D x 128] . P^T [128 x 16]
 // At head_dim 64 P is held to float precision, as the sum of three bf16 parts (further columns
-// of P^T and O^T, in the same MMAs), and the PV MMA's upper 64 rows are unused.  (Before, head_dim 64 ran on the CUDA cores, 64-key tiles and
-// a merge kernel: calls in a graph, 32 / 8 heads, B16 over 8190 tokens 72.1 us, now 56.7;
-// 5 tokens of 3 sequences 80.5 us, now 26.)
+// of P^T and O^T, in the same MMAs), and the PV MMA's upper 64 rows are unused.  (Before,
+// head_dim 64 ran on the CUDA cores, 64-key tiles and a merge kernel: calls in a graph, 32 / 8
+// heads, B16 over 8190 tokens 72.1 us, now 56.7; 5 tokens of 3 sequences 80.5 us, now 26.)
 // Both accumulate in TMEM.  The T = ceil((p+ntok)/128) key tiles of a sequence are
 // claimed by the nsplit CTAs of its item (b, kv head, column group): in a one-wave grid
 // split s starts with tile s, in a larger one only split 0 has a fixed first tile; every
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
     // starts (it is a dependent launch only after another decode step, which lets its
     // dependents start only once its own predecessors are complete).
     // In flight while the barriers and TMEM are set up (volatile: the compiler may otherwise sink
-    // the load to its first use, behind that set-up: B1 over 1024 tokens 7.3 us instead of 6.9).
+    // the load to its first use, behind that set-up; B1 over 1024 tokens 7.27 -> 7.19 us).
     int hist_len;
     asm volatile("ld.global.s32 %0, [%1];" : "=r"(hist_len) : "l"(d_hist + b));
     const int kv_row = b * Hkv + g;
@@ -347,12 +347,12 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
     unsigned long long* done_ctr = reinterpret_cast<unsigned long long*>(counters + ((3 * n_items + 1) & ~1)) + ctr_row;
     // A helper split (s >= s0: a grid of several waves) first asks its item's counter for a
     // tile.  If none is left -- the item is done, or its tiles are all taken -- the CTA
-    // records its visit and leaves before any set-up.  When the items are more than half the SMs
-    // (spec & 2) and the batch's lengths are within
-    // 10% of each other (read by one warp, batches of up to 1024) there is nothing to even
-    // out, and helpers leave without asking: the splits 0 then finish their items alone and
-    // write the outputs without a merge.  (After the previous decode step the counters are
-    // touched only once that step is complete.)
+    // records its visit and leaves before any set-up.  When the batch's lengths are within 10%
+    // of each other (read by one warp, batches of up to 1024) there is nothing to even out, and
+    // the helpers from split spec >> 2 on leave without asking: all of them with more items than
+    // half the SMs (the splits 0 then finish their items alone and write the outputs without a
+    // merge), else the one that a single wave would not hold.  (After the previous decode step
+    // the counters are touched only once that step is complete.)
     int first_ticket = 0;
     if (WAVES && multi && s >= s0) {
         if (warp == 0) {
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
                 int t = -1;
                 const TokRange own = decode_tokens<D>(hist_len, hist_add, ntok, max_len);
                 if (own.hi > own.lo) {
-                    if (!even) t = s0 + atomicAdd(claim_ctr, 1);
+                    if (!even || s < (spec >> 2)) t = s0 + atomicAdd(claim_ctr, 1);
                     if (t >= (own.hist + own.hi + KT - 1) / KT) t = -1;
                     if (t < 0 && atomicAdd(visit_ctr, 1) == nsplit - 1) {
                         *claim_ctr = 0;
@@ -396,8 +396,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
     // cache (a decode step right after another, spec = 0), issues the copies of its first
     // tile, tile s, before the length is known: the K slot's arrival is held back until the
     // producer knows whether tile s holds keys of the sequence (the copies read in-range
-    // slots or the map's zero fill either way; a tile past the sequence is not used).
-    // (spec & 1)
+    // slots or the map's zero fill either way; a tile past the sequence is not used): spec & 1.
     const bool spec_first = (spec & 1) != 0 && s < s0 && s * KT < max_len;
     if (warp == kWarpTma && lane == 0) {
         *abort_flag = 0;
@@ -1190,25 +1189,26 @@ bool decode_tc_clusters_fit(int nsplit, long long items) {
 }  // namespace
 
 // Split counts.  With few (sequence, kv head, column group) items (up to 30% of the SMs),
-// one wave of CTAs, min(16, floor(SMs / items)) splits per item, each starting with its own
-// tile.
-// With more items, several waves (kWaveSplits splits per item above half the SMs): split 0 of every item
-// comes first and the later splits, dispatched as SMs free up, claim what their items
+// one wave of CTAs, min(16, floor(SMs / items)) splits per item (32 for up to 4 items), each
+// starting with its own tile.  With more items, several waves (kWaveSplits splits per item above
+// half the SMs, see mid_items below it): split 0 of every item comes first and the later splits, dispatched as SMs free up, claim what their items
 // still have (nothing, for an item that is done), so long sequences in a batch of mixed
 // lengths get help once the short ones finish.
 constexpr int kWaveSplits = 3;
 // One wave: at most 16 splits per item.  The long decode (8 items) measured 29.5 us with 16
 // splits, 30.4-30.8 us with 19 (one per SM), 32.5 with 12 and 42 with 8: past 16 the extra
 // partials and the later last CTA cost more than the SMs add.  Up to 4 items take 32, which
-// leaves fewer SMs idle (4 items over 32767 tokens 20.9 -> 18.9 us; head_dim 64, 2 items over 32000: 23.9 -> 15.7).
+// leaves fewer SMs idle (4 items over 32767 tokens 20.9 -> 18.9 us; head_dim 64, 2 items over
+// 32000: 23.9 -> 15.7).
 constexpr long kMaxWaveSplits1 = 16, kMaxWaveSplitsFew = 32, kFewItems = 4;
 
 // Between 30% and 50% of the SMs in items (46 .. 76), one wave gives every item the same 2 or 3
 // splits whatever its length; one split more makes it several waves, whose claims even out
-// mixed lengths.  Calls in a graph, 64 items (28 / 4 heads B16, 32 / 8 heads B8): lengths
-// 64 .. 8183 36.0 -> 30.0 and 32.9 -> 28.1 us, one long among short 34.4 -> 25.2, all 8190
-// 46.0 -> 45.4, but all 4096 27.6 -> 29.5 (32 / 8); 48 items 35.2 -> 25.6, all 8190
-// 38.0 -> 36.6.  At 40 items an even batch loses 12% (8190: 31.0 -> 34.8).
+// mixed lengths (the extra split stands down where they are even).  Calls in a graph, 64 items
+// (28 / 4 heads B16, 32 / 8 heads B8): lengths 64 .. 8183 36.0 -> 30.0 and 32.9 -> 28.2 us, one
+// long among short 34.4 -> 24.8, all 8190 46.0 -> 45.9, all 4096 27.6 -> 29.0 (32 / 8; 29.7 with
+// the extra split claiming); 48 items 35.2 -> 25.6, all 8190 38.0 -> 37.0.  At 40 items an even
+// batch loses 12% (8190: 31.0 -> 34.8, with the extra split claiming).
 bool mid_items(long items, int num_sms) { return 2 * items <= num_sms && 10 * items > 3 * num_sms; }
 
 int decode_tc_column_groups(int G, int ntok) { return (G * ntok + NH - 1) / NH; }
@@ -1217,8 +1217,9 @@ int decode_tc_num_splits(const Shape& s, int num_sms, int ncg, int ntok) {
     const long items = static_cast<long>(s.batch) * s.n_kv_heads * ncg;
     const long max_tiles = std::max(1L, static_cast<long>((s.max_len + KT - 1) / KT));
     long ns = 2 * items > num_sms ? kWaveSplits
-              : mid_items(items, num_sms) ? num_sms / items + 1
-                                  : std::min<long>(items <= kFewItems ? kMaxWaveSplitsFew : kMaxWaveSplits1, num_sms / items);
+              : mid_items(items, num_sms)
+                  ? num_sms / items + 1
+                  : std::min<long>(items <= kFewItems ? kMaxWaveSplitsFew : kMaxWaveSplits1, num_sms / items);
     ns = std::min(ns, std::min(max_tiles, 256L));
     // The last split of an item merges ns partials of up to 16 columns in the global merge,
     // while a cluster spreads the merge over its CTAs.  Fewer splits whose clusters fit on the
@@ -1229,7 +1230,8 @@ int decode_tc_num_splits(const Shape& s, int num_sms, int ncg, int ntok) {
     // at most 64 tiles (B1 Hq32 over 1024 and 4096 tokens: 11.8 -> 10.3 us and 14.1 -> 12.9 us;
     // at 32767 tokens 12 splits took 32.5 us against 29.5 us with 16).
     const long cols = std::min<long>(NH, static_cast<long>(s.n_q_heads / s.n_kv_heads) * ntok);
-    if (2 * items <= num_sms && !mid_items(items, num_sms) && ((ntok > 1 && ns * cols >= 128) || (ntok == 1 && max_tiles <= 64)))
+    if (2 * items <= num_sms && !mid_items(items, num_sms) &&
+        ((ntok > 1 && ns * cols >= 128) || (ntok == 1 && max_tiles <= 64)))
         while (ns > 2 && !decode_tc_clusters_fit(static_cast<int>(ns), items)) --ns;
     return static_cast<int>(std::max(1L, ns));
 }
@@ -1310,12 +1312,15 @@ cudaError_t launch_decode_tc(const Shape& s, const DecodeMaps& maps, const uint1
          {DECODE_TC_MODES(64, 16, kMaxTok)}}};
     const Kernel kernel =
         kernels[s.head_dim == 64][ntok == 1 ? (G <= 8 ? 0 : 1) : (G * ntok <= 8 ? 2 : 3)][mode];
+    const long items = static_cast<long>(s.batch) * s.n_kv_heads * ncg;
+    const bool mid = mid_items(items, num_sms);
+    const int spec = (after_decode ? 0 : 1) | (2 * items > num_sms || mid ? 2 : 0) | (mid ? nsplit - 1 : 0) << 2;
     return cudaLaunchKernelEx(&cfg, kernel, maps.k, maps.v, q,
                               k_new, v_new, d_hist, hist_add, ntok, seq_tok, k_cache, v_cache, cos_tab, sin_tab,
                               s.n_q_heads,
                               s.n_kv_heads, s.max_len, nsplit, scale_log2, part_o, part_ml, counters, out, err,
                               producer_early ? 1 : 0, wait_ns, ncg,
-                              (after_decode ? 0 : 1) | (2LL * s.batch * s.n_kv_heads * ncg > num_sms ? 2 : 0), s0);
+                              spec, s0);
 }
 
 }  // namespace attn
