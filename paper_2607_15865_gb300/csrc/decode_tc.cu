@@ -16,7 +16,7 @@
 // At head_dim 64 P is held to float precision, as the sum of three bf16 parts (further columns
 // of P^T and O^T, in the same MMAs), and the PV MMA's upper 64 rows are unused.  (Before,
 // head_dim 64 ran on the CUDA cores, 64-key tiles and a merge kernel: calls in a graph, 32 / 8
-// heads, B16 over 8190 tokens 72.1 us, now 56.7; 5 tokens of 3 sequences 80.5 us, now 26.)
+// heads, B16 over 8190 tokens 72.1 us, now 46.5; 5 tokens of 3 sequences 80.5 us, now 26.)
 // Both accumulate in TMEM.  The T = ceil((p+ntok)/128) key tiles of a sequence are
 // claimed by the nsplit CTAs of its item (b, kv head, column group): in a one-wave grid
 // split s starts with tile s, in a larger one only split 0 has a fixed first tile; every
@@ -32,7 +32,8 @@
 //              shuffles for 16 columns) and O^T is rescaled.  Epilogue: one thread
 //              per output dimension d;
 //   warp 4     TMA producer: K and V tiles of 128 keys (128-byte swizzle) into
-//              rings of 2 (K) and 4 (V) stages of 32 KB;
+//              rings of 2 (K) and 4 (V) stages of 32 KB (head_dim 64: 2 and 3 of 16 KB, so
+//              that two CTAs share an SM);
 //   warp 5     tcgen05 issuer; it also owns the new tokens: it rotates their k (RoPE
 //              from the table, the same float arithmetic and bf16 rounding as K1),
 //              writes k and v to their slots of the cache and into the shared-memory
@@ -71,7 +72,6 @@ constexpr int kMaxTok = 16;  // new tokens per sequence in one launch (heads x t
 // issuer keeps the new tokens' rotated k and v in registers, unrolled over MAXTOK, and
 // sixteen unrolled slots cost a single-token decode about 2 us.
 constexpr int KST = 2;      // K ring stages (a K tile is free once S^T of it completes)
-constexpr int VST = 4;      // V ring stages (a V tile is held until its PV completes)
 constexpr int kThreads = 192;
 constexpr int kWarpTma = 4;
 constexpr int kWarpMma = 5;
@@ -87,6 +87,7 @@ enum Bar { B_QREADY, B_KFULL0, B_KFULL1, B_KEMPTY0, B_KEMPTY1, B_VFULL0, B_VFULL
 // as many column groups, added up at the end.
 template <int D>
 struct Layout {
+    static constexpr int VST = D == 64 ? 3 : 4;  // V ring stages (a V tile is held until its PV completes)
     static constexpr int NP = D == 64 ? 3 : 1;
     static constexpr int PC = NP * NH;                       // columns of P^T and O^T
     static constexpr uint32_t TMEM_COLS = D == 64 ? 128 : 64;  // S^T x2 [0,32), O^T [32,32 + PC)
@@ -260,8 +261,14 @@ __device__ __forceinline__ TokRange decode_tokens(int hist_len, int hist_add, in
 // helper splits and slot and visit counters.  Each is its own instantiation, so that a
 // launch runs only the code of its mode.
 constexpr int kModeGlobal = 0, kModeCluster = 1, kModeWaves = 2;
+// CTAs of the kernel that an SM holds: two where the rings are half as large and the new tokens'
+// registers few (head_dim 64, one new token).  A tile is a chain of latencies there (half the
+// bytes of head_dim 128), so a second CTA fills the waits: calls in a graph, 32 / 8 heads, B24
+// of 8190 tokens 99.6 -> 67.1 us, B16 57.3 -> 46.5, B12 56.9 -> 37.1, B8 32.7 -> 28.5.
+constexpr int ctas_per_sm(int D, int ntok) { return D == 64 && ntok == 1 ? 2 : 1; }
+static_assert(2 * (Layout<64>::ALLOC + 1024) <= 233472, "shared memory of two CTAs");
 template <int D, int NHP, int MAXTOK, int MODE>
-__global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
+__global__ void __launch_bounds__(kThreads, ctas_per_sm(D, MAXTOK)) decode_tc_kernel(
     const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
     const uint16_t* __restrict__ q, const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
     const int32_t* __restrict__ d_hist, int hist_add, int ntok, int seq_tok, uint16_t* __restrict__ k_cache,
@@ -271,6 +278,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
     uint16_t* __restrict__ out, int* __restrict__ err, int producer_early, uint64_t wait_ns, int ncg, int spec,
     int s0) {
     using L = Layout<D>;
+    constexpr int VST = L::VST;
     constexpr bool WAVES = MODE == kModeWaves;
     constexpr bool kGuardV = D == 64 && MAXTOK > 1;
     constexpr int HALF = D / 2;
@@ -350,7 +358,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
     // records its visit and leaves before any set-up.  When the batch's lengths are within 10%
     // of each other (read by one warp, batches of up to 1024) there is nothing to even out, and
     // the helpers from split spec >> 2 on leave without asking: all of them with more items than
-    // half the SMs (the splits 0 then finish their items alone and write the outputs without a
+    // half the slots (the splits 0 then finish their items alone and write the outputs without a
     // merge), else the one that a single wave would not hold.  (After the previous decode step
     // the counters are touched only once that step is complete.)
     int first_ticket = 0;
@@ -1128,7 +1136,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tc_kernel(
 // once, per device, set by configure_decode_tc; 0 where the size is refused.
 constexpr int kMaxDevices = 64;
 constexpr int kMaxCluster = 16;
-int g_cluster_fit[kMaxDevices][kMaxCluster + 1] = {};
+int g_cluster_fit[kMaxDevices][2][kMaxCluster + 1] = {};  // [1]: two CTAs per SM
 
 #define DECODE_TC_MODES(D, NHP, MAXTOK)                                                             \
     decode_tc_kernel<D, NHP, MAXTOK, kModeGlobal>, decode_tc_kernel<D, NHP, MAXTOK, kModeCluster>, \
@@ -1154,13 +1162,14 @@ cudaError_t configure_decode_tc() {
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    // (the cluster instantiations share the block size and one block per SM; measured with the
+    // (the cluster instantiations share the block size; one block per SM is measured with the
     // larger shared memory, of head_dim 128)
-    for (int c = 2; c <= kMaxCluster; ++c) {
+    for (int i = 0; i < 2 * (kMaxCluster - 1); ++i) {
+        const int c = 2 + i / 2, two = i % 2;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(static_cast<unsigned>(c), 1, 1);
         cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = Layout<128>::ALLOC;
+        cfg.dynamicSmemBytes = two ? Layout<64>::ALLOC : Layout<128>::ALLOC;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = static_cast<unsigned>(c);
@@ -1169,31 +1178,34 @@ cudaError_t configure_decode_tc() {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, decode_tc_kernel<128, 8, 1, kModeCluster>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(
+                &n, two ? decode_tc_kernel<64, 8, 1, kModeCluster> : decode_tc_kernel<128, 8, 1, kModeCluster>, &cfg) != cudaSuccess) {
             n = 0;
             cudaGetLastError();  // a refused size is never used
         }
-        g_cluster_fit[dev][c] = n;
+        g_cluster_fit[dev][two][c] = n;
     }
     return cudaSuccess;
 }
 
 namespace {
 // Whether `items` clusters of nsplit CTAs all fit on the current device at once.
-bool decode_tc_clusters_fit(int nsplit, long long items) {
+bool decode_tc_clusters_fit(int nsplit, long long items, int per_sm) {
     int dev = 0;
     if (nsplit < 2 || nsplit > kMaxCluster || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
         return false;
-    return items <= g_cluster_fit[dev][nsplit];
+    return items <= g_cluster_fit[dev][per_sm - 1][nsplit];
 }
 }  // namespace
 
-// Split counts.  With few (sequence, kv head, column group) items (up to 30% of the SMs),
-// one wave of CTAs, min(16, floor(SMs / items)) splits per item (32 for up to 4 items), each
-// starting with its own tile.  With more items, several waves (kWaveSplits splits per item above
-// half the SMs, see mid_items below it): split 0 of every item comes first and the later splits, dispatched as SMs free up, claim what their items
-// still have (nothing, for an item that is done), so long sequences in a batch of mixed
-// lengths get help once the short ones finish.
+// Split counts; slots are the CTAs that the device holds at once (SMs, at head_dim 64 with one new
+// token twice as many).  With few (sequence, kv head, column group) items (up to 30% of the
+// slots), one wave of CTAs, min(16, floor(slots / items)) splits per item (32 for up to 4 items),
+// each starting with its own tile.  With more items, several waves (kWaveSplits splits per item
+// above half the slots, see mid_items below it): split 0 of every item comes first and the later
+// splits, dispatched as slots free up, claim what their items still have (nothing, for an item
+// that is done), so long sequences in a batch of mixed lengths get help once the short ones
+// finish.
 constexpr int kWaveSplits = 3;
 // One wave: at most 16 splits per item.  The long decode (8 items) measured 29.5 us with 16
 // splits, 30.4-30.8 us with 19 (one per SM), 32.5 with 12 and 42 with 8: past 16 the extra
@@ -1209,17 +1221,23 @@ constexpr long kMaxWaveSplits1 = 16, kMaxWaveSplitsFew = 32, kFewItems = 4;
 // long among short 34.4 -> 24.8, all 8190 46.0 -> 45.9, all 4096 27.6 -> 29.0 (32 / 8; 29.7 with
 // the extra split claiming); 48 items 35.2 -> 25.6, all 8190 38.0 -> 37.0.  At 40 items an even
 // batch loses 12% (8190: 31.0 -> 34.8, with the extra split claiming).
-bool mid_items(long items, int num_sms) { return 2 * items <= num_sms && 10 * items > 3 * num_sms; }
+// With two CTAs per SM from 39 items on, where clusters of that many splits no longer fit at once:
+// 40 items (32 / 8), mixed 22.4 -> 17.3 us, one long 22.7 -> 16.4, all 8190 24.2 -> 21.8, but all
+// 1000 8.9 -> 11.1; at 32 items all 1000 8.3 -> 11.0 for mixed 18.0 -> 15.7.
+bool mid_items(long items, int slots, int per_sm) {
+    return 2 * items <= slots && (per_sm == 2 ? 8 * items > slots : 10 * items > 3 * slots);
+}
 
 int decode_tc_column_groups(int G, int ntok) { return (G * ntok + NH - 1) / NH; }
 
 int decode_tc_num_splits(const Shape& s, int num_sms, int ncg, int ntok) {
+    const int per_sm = ctas_per_sm(s.head_dim, ntok), slots = num_sms * per_sm;
     const long items = static_cast<long>(s.batch) * s.n_kv_heads * ncg;
     const long max_tiles = std::max(1L, static_cast<long>((s.max_len + KT - 1) / KT));
-    long ns = 2 * items > num_sms ? kWaveSplits
-              : mid_items(items, num_sms)
-                  ? num_sms / items + 1
-                  : std::min<long>(items <= kFewItems ? kMaxWaveSplitsFew : kMaxWaveSplits1, num_sms / items);
+    long ns = 2 * items > slots ? kWaveSplits
+              : mid_items(items, slots, per_sm)
+                  ? slots / items + 1
+                  : std::min<long>(items <= kFewItems ? kMaxWaveSplitsFew : kMaxWaveSplits1, slots / items);
     ns = std::min(ns, std::min(max_tiles, 256L));
     // The last split of an item merges ns partials of up to 16 columns in the global merge,
     // while a cluster spreads the merge over its CTAs.  Fewer splits whose clusters fit on the
@@ -1230,9 +1248,9 @@ int decode_tc_num_splits(const Shape& s, int num_sms, int ncg, int ntok) {
     // at most 64 tiles (B1 Hq32 over 1024 and 4096 tokens: 11.8 -> 10.3 us and 14.1 -> 12.9 us;
     // at 32767 tokens 12 splits took 32.5 us against 29.5 us with 16).
     const long cols = std::min<long>(NH, static_cast<long>(s.n_q_heads / s.n_kv_heads) * ntok);
-    if (2 * items <= num_sms && !mid_items(items, num_sms) &&
+    if (2 * items <= slots && !mid_items(items, slots, per_sm) &&
         ((ntok > 1 && ns * cols >= 128) || (ntok == 1 && max_tiles <= 64)))
-        while (ns > 2 && !decode_tc_clusters_fit(static_cast<int>(ns), items)) --ns;
+        while (ns > 2 && !decode_tc_clusters_fit(static_cast<int>(ns), items, per_sm)) --ns;
     return static_cast<int>(std::max(1L, ns));
 }
 
@@ -1265,7 +1283,8 @@ cudaError_t launch_decode_tc(const Shape& s, const DecodeMaps& maps, const uint1
     const int ncg = decode_tc_column_groups(G, ntok);
     // every split starts with its own tile when the grid is one wave, else only split 0
     const long long ctas = static_cast<long long>(s.n_kv_heads) * s.batch * ncg * nsplit;
-    const int s0 = ctas <= num_sms ? nsplit : 1;
+    const int per_sm = ctas_per_sm(s.head_dim, ntok), slots = num_sms * per_sm;
+    const int s0 = ctas <= slots ? nsplit : 1;
     const dim3 grid = s0 == nsplit ? dim3(static_cast<unsigned>(nsplit), static_cast<unsigned>(s.n_kv_heads),
                                           static_cast<unsigned>(s.batch * ncg))
                                    : dim3(static_cast<unsigned>(s.n_kv_heads), static_cast<unsigned>(s.batch * ncg),
@@ -1287,7 +1306,7 @@ cudaError_t launch_decode_tc(const Shape& s, const DecodeMaps& maps, const uint1
     // one wave: the splits of an item are one cluster (their merge) when a cluster per item
     // fits on the device at once, else they merge through global memory
     const int mode = w ? kModeWaves
-                       : (decode_tc_clusters_fit(nsplit, static_cast<long long>(s.n_kv_heads) * s.batch * ncg)
+                       : (decode_tc_clusters_fit(nsplit, static_cast<long long>(s.n_kv_heads) * s.batch * ncg, per_sm)
                               ? kModeCluster
                               : kModeGlobal);
     if (mode == kModeCluster) {
@@ -1313,8 +1332,8 @@ cudaError_t launch_decode_tc(const Shape& s, const DecodeMaps& maps, const uint1
     const Kernel kernel =
         kernels[s.head_dim == 64][ntok == 1 ? (G <= 8 ? 0 : 1) : (G * ntok <= 8 ? 2 : 3)][mode];
     const long items = static_cast<long>(s.batch) * s.n_kv_heads * ncg;
-    const bool mid = mid_items(items, num_sms);
-    const int spec = (after_decode ? 0 : 1) | (2 * items > num_sms || mid ? 2 : 0) | (mid ? nsplit - 1 : 0) << 2;
+    const bool mid = mid_items(items, slots, per_sm);
+    const int spec = (after_decode ? 0 : 1) | (2 * items > slots || mid ? 2 : 0) | (mid ? nsplit - 1 : 0) << 2;
     return cudaLaunchKernelEx(&cfg, kernel, maps.k, maps.v, q,
                               k_new, v_new, d_hist, hist_add, ntok, seq_tok, k_cache, v_cache, cos_tab, sin_tab,
                               s.n_q_heads,
