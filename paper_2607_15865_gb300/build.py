@@ -21,7 +21,7 @@ LIB = os.path.join(PKG, "libattn_gb300.so")
 SOURCES = [("attn_api.cu", "attn_api", []), ("rope_append.cu", "rope_append", []),
            ("decode_tc.cu", "decode_tc", []), ("flash_fwd.cu", "flash_fwd", []),
            ("decode_noalloc.cu", "decode_noalloc", []), ("w4_gemv.cu", "w4_gemv", []), ("w4_gemm.cu", "w4_gemm", [])]
-HEADERS = ["internal.h", "sm100_ptx.cuh"]
+HEADERS = ["internal.h", "sm100_ptx.cuh", "flash_rows.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -43,6 +43,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "flash_rows.h"
 #include "internal.h"
 #include "sm100_ptx.cuh"
 
@@ -317,7 +318,7 @@ __device__ __forceinline__ bool rope_item(uint32_t qfull, uint32_t qready, uint3
                                           const float* __restrict__ cos_t, const float* __restrict__ sin_t,
                                           int stride, uint64_t wait_ns) {
     RopeRow<D> tabs;
-    rope_load<D>(tabs, row < rows ? pos0 + row_tok : pos0, cos_t, sin_t, stride);
+    rope_load<D>(tabs, rope_table_pos(row, rows, row_tok, pos0), cos_t, sin_t, stride);
     const bool w = __all_sync(0xFFFFFFFFu, mbar_wait(qfull, parity, abort, wait_ns));
     if (w && row < rows) rope_row_smem<D>(qtile, row, tabs);
     if (PK && row >= copied_rows) {
