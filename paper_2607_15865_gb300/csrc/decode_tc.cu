@@ -565,10 +565,6 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(D, MAXTOK)) decode_tc_ke
             if (!ok) {
                 *abort_flag = 1;
                 atomicOr(err, kDevErrTimeout);
-                for (int t = max(0, issued_k - KST); t < issued_k; ++t)
-                    mbar_wait(bar(B_KFULL0 + t % KST), static_cast<uint32_t>(t / KST) & 1u, nullptr);
-                for (int t = max(0, issued_v - VST); t < issued_v; ++t)
-                    mbar_wait(bar(B_VFULL0 + t % VST), static_cast<uint32_t>(t / VST) & 1u, nullptr);
                 if (claims) {
                     // take every ticket still unclaimed (and count it, unprocessed), so that the
                     // item's tiles are all accounted for and its merge and reset still happen
@@ -586,6 +582,13 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(D, MAXTOK)) decode_tc_ke
                 *slot_ctr = 0;
                 *visit_ctr = 0;
             }
+            // Every copy issued must land before the CTA may exit, also when this loop ended well
+            // and another warp's wait ran out.  (A loop that ended well has put its end mark in K
+            // slot issued_k mod KST, whose copy had landed before: its phase is past.)
+            for (int t = max(0, issued_k - KST + (ok ? 1 : 0)); t < issued_k; ++t)
+                mbar_wait(bar(B_KFULL0 + t % KST), static_cast<uint32_t>(t / KST) & 1u, nullptr);
+            for (int t = max(0, issued_v - VST); t < issued_v; ++t)
+                mbar_wait(bar(B_VFULL0 + t % VST), static_cast<uint32_t>(t / VST) & 1u, nullptr);
         }
         if (early) griddep_wait();
     } else if (warp == kWarpMma) {

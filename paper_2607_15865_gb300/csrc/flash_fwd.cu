@@ -477,11 +477,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (!ok) {
                 *abort_flag = 1;
                 atomicOr(err, kDevErrTimeout);
-                // every copy issued must land before the CTA may exit
-                if (items > 0) mbar_wait(bar(B_QFULL), static_cast<uint32_t>(items - 1) & 1u, nullptr);
-                for (uint32_t t = gc >= GS ? gc - GS : 0; t < gc; ++t)
-                    mbar_wait(bar(B_GFULL0 + static_cast<int>(t % GS)), (t / GS) & 1u, nullptr);
             }
+            // Every copy issued must land before the CTA may exit (or its cluster peer writes here),
+            // also when this loop ended well and another warp's wait ran out.
+            if (items > 0) mbar_wait(bar(B_QFULL), static_cast<uint32_t>(items - 1) & 1u, nullptr);
+            for (uint32_t t = gc >= GS ? gc - GS : 0; t < gc; ++t)
+                mbar_wait(bar(B_GFULL0 + static_cast<int>(t % GS)), (t / GS) & 1u, nullptr);
         } else if (warp == kWarpMma && lane == 0) {
             // ---------------------------------------------------- tcgen05 issuer
             constexpr uint32_t kIdS = idesc_bf16_f32(BM, BN, false, false);
