@@ -86,6 +86,11 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
+// Set `bit` of the caller's error word, where the caller gave one.
+__device__ __forceinline__ void record_dev_err(int* err, int bit) {
+    if (err != nullptr) atomicOr(err, bit);
+}
+
 // Limits below this are only used to exercise the failure path: such a wait gives up at
 // once unless its phase has already completed (a try_wait may itself block for a while).
 constexpr uint64_t kMinBlockingWaitNs = 1000;

@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kThreads, 1) w4_gemm_kernel(const __grid_const
             }
             if (!ok) {
                 *abort_flag = 1;
-                atomicOr(err, kDevErrTimeout);
+                record_dev_err(err, kDevErrTimeout);
             }
             // every copy issued must land before the CTA may exit
             for (uint32_t g = gs > kStages ? gs - kStages : 0; g < gs; ++g)
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kThreads, 1) w4_gemm_kernel(const __grid_const
             }
             if (!ok && lane == 0) {
                 *abort_flag = 1;
-                atomicOr(err, kDevErrTimeout);
+                record_dev_err(err, kDevErrTimeout);
             }
             // also after an abort: the MMAs issued so far complete on it
             if (elect_one()) umma2_commit_mc(bar(B_DRAIN), static_cast<uint16_t>(1u << rank));
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kThreads, 1) w4_gemm_kernel(const __grid_const
         }
         if (!ok && lane == 0) {
             *abort_flag = 1;
-            atomicOr(err, kDevErrTimeout);
+            record_dev_err(err, kDevErrTimeout);
         }
     }
 
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(kThreads, 1) w4_gemm_kernel(const __grid_const
             }
             if (!ok && lane == 0) {
                 *abort_flag = 1;
-                atomicOr(err, kDevErrTimeout);
+                record_dev_err(err, kDevErrTimeout);
             }
         }
     } else {
@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(kThreads, 1) w4_gemm_kernel(const __grid_const
             ok = __all_sync(0xFFFFFFFFu, wait_full(bar(B_ACCFULL), 0u, abort_flag));
             if (!ok && lane == 0) {
                 *abort_flag = 1;
-                atomicOr(err, kDevErrTimeout);
+                record_dev_err(err, kDevErrTimeout);
             }
             tc_fence_after();
         }

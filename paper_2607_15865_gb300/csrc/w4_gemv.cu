@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(kThreads) w4_gemv_kernel(const uint8_t* __rest
                 if (!failed) {
                     const bool landed = mbar_wait(my_bars + 8 * cslot, cphase, nullptr, kWaitNs);
                     failed = __any_sync(0xFFFFFFFFu, !landed);
-                    if (failed && err != nullptr && lane == 0) atomicOr(err, kDevErrTimeout);
+                    if (failed && lane == 0) record_dev_err(err, kDevErrTimeout);
                 }
                 if (!failed) {  // (the slot of a failed wait stays current for the drain below)
                     --outstanding;
@@ -511,7 +511,7 @@ __global__ void __launch_bounds__(kThreads) w4_gemv_cluster_kernel(const uint8_t
                 if (!failed) {
                     const bool landed = mbar_wait(my_bars + 8 * cslot, cphase, nullptr, kWaitNs);
                     failed = __any_sync(0xFFFFFFFFu, !landed);
-                    if (failed && err != nullptr && lane == 0) atomicOr(err, kDevErrTimeout);
+                    if (failed && lane == 0) record_dev_err(err, kDevErrTimeout);
                 }
                 if (!failed) {  // (the slot of a failed wait stays current for the drain below)
                     --outstanding;

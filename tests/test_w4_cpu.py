@@ -72,3 +72,15 @@ def test_tile_stream_round_trips_for_any_shape():
         assert (buf == W.write_tiles(codes, scales, zeros)).all()  # byte for byte, padding included
 
     prop()
+
+
+@pytest.mark.parametrize("source", ["w4_gemm.cu", "w4_gemv.cu"])
+def test_kernels_write_the_error_word_only_where_there_is_one(source):
+    """err may be NULL for these kernels.  Their waits have a fixed limit that no test can make run
+    out, so this reads the source: every write goes through record_dev_err, which tests for NULL."""
+    import os
+    csrc = os.path.join(os.path.dirname(_lib.__file__), "csrc")
+    text = open(os.path.join(csrc, source)).read()
+    assert "record_dev_err(err, kDevErrTimeout)" in text and "atomicOr" not in text
+    helper = open(os.path.join(csrc, "sm100_ptx.cuh")).read()
+    assert "if (err != nullptr) atomicOr(err, bit);" in helper
