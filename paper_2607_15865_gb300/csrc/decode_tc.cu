@@ -566,8 +566,10 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(D, MAXTOK)) decode_tc_ke
                 *abort_flag = 1;
                 atomicOr(err, kDevErrTimeout);
                 if (claims) {
-                    // take every ticket still unclaimed (and count it, unprocessed), so that the
-                    // item's tiles are all accounted for and its merge and reset still happen
+                    // take every ticket still unclaimed (and count it, unprocessed, as the one
+                    // claimed ahead), so that the item's tiles are all accounted for and its merge
+                    // and reset still happen
+                    if (nxt < T) ++claimed;
                     const int first = s0 + atomicAdd(claim_ctr, T);
                     if (first < T) claimed += T - first;
                 }

@@ -24,7 +24,8 @@ DEVERR_TIMEOUT = 2
 # head_dim 128 and 64: flash_fwd whose items are cut in pieces for the merge kernel, and the
 # decode's fused merge and counters; walks of one key tile, whose copies are all in flight when
 # the first wait gives up; two pieces per item, which meet at the cluster barriers of their merge
-# (as a tile of one head, and with the heads of a kv head packed into the rows).
+# (as a tile of one head, and with the heads of a kv head packed into the rows); decodes of
+# several waves, whose claimed and counted tiles must add up all the same (the packed case, waves_d64).
 CASES = [
     ("d128", Shape("wl128", 2, 8, 2, 128, 1024, 1.0e4), 300, 333),
     ("d64", Shape("wl64", 1, 4, 2, 64, 640, 1.0e4), 200, 150),
@@ -32,6 +33,7 @@ CASES = [
     ("one_key_tile_d64", Shape("wl1k64", 2, 4, 2, 64, 160, 1.0e4), 40, 50),
     ("cluster_d128", Shape("wlc", 1, 64, 8, 128, 900, 1.0e4), 600, 250),
     ("cluster_d64", Shape("wlc64", 1, 64, 8, 64, 900, 1.0e4), 600, 256),
+    ("waves_d64", Shape("wlw64", 20, 16, 8, 64, 1300, 1.0e4), 1100, 100),
     ("cluster_packed_d128", Shape("wlcp", 8, 32, 8, 128, 1100, 1.0e4), 1000, 16),
 ]
 
