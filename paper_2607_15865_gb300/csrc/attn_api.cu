@@ -322,6 +322,13 @@ int attn_prefill_kv(attn_ctx* c, const uint16_t* q, const uint16_t* k, const uin
 
 namespace {
 
+// Splits per item of a decode of ntok tokens: the partials hold batch * Hq * nsplit_max rows, which
+// the tokens share.
+int decode_splits(const attn_ctx* c, int ntok) {
+    const int ncg = attn::decode_tc_column_groups(c->cfg.n_q_heads / c->cfg.n_kv_heads, ntok);
+    return std::min(attn::decode_tc_num_splits(c->shape, c->num_sms, ncg, ntok), c->nsplit_max / ntok);
+}
+
 // One decode step of ntok new tokens per sequence at positions d_hist_len[b] + hist_add + i.
 // after_decode: the previous launch on `st` was this context's decode of the same caches
 // (a decode loop).
@@ -349,11 +356,10 @@ int run_decode(attn_ctx* c, const uint16_t* q, const uint16_t* k, const uint16_t
         c->dec_v = v_cache;
     }
     if (ntok < 1 || ntok > kMaxDraftTokens) return ATTN_EINVAL;
-    // the partials hold batch * Hq * nsplit_max rows: ntok tokens share them
     const int ncg = attn::decode_tc_column_groups(c->cfg.n_q_heads / c->cfg.n_kv_heads, ntok);
     // grid dimensions of sequences x column groups stay within 65535
     if (static_cast<long>(c->cfg.batch) * ncg > 65535) return ATTN_EINVAL;
-    const int nsplit = std::min(attn::decode_tc_num_splits(c->shape, c->num_sms, ncg, ntok), c->nsplit_max / ntok);
+    const int nsplit = decode_splits(c, ntok);
     const cudaError_t e = timed(c, ATTN_KERNEL_DECODE_SPLIT, st, [&](int*) {
         return attn::launch_decode_tc(c->shape, c->dec_maps, q, k, v, d_hist_len, hist_add, k_cache, v_cache, c->d_cos,
                                       c->d_sin, c->d_part_o, c->d_part_ml, c->d_counters, nsplit, out, c->d_err,
@@ -673,6 +679,29 @@ int attn_w4bf16_gemv(const void* w_tiles, const uint16_t* x, int M, int N, int K
                      int flags, attn_stream_t stream) {
     return attn_w4bf16_gemv_fused(w_tiles, x, M, N, K, nullptr, 0.f, nullptr, y, 0, nullptr, 0, nullptr, d_err, flags,
                                   stream);
+}
+
+// Exported for the tests, not part of attn.h: how the library cuts a call on this device (out[4] as
+// in internal.h; decode: splits per item and mode), so that a test can assert the path that it names.
+int attn_plan_prefill(const attn_ctx* c, int hist_len, int chunk_len, int* out) {
+    if (c == nullptr || out == nullptr || hist_len < 0 || chunk_len < 1 ||
+        static_cast<long>(hist_len) + chunk_len > c->cfg.max_len)
+        return ATTN_EINVAL;
+    attn::flash_plan(c->shape, hist_len, chunk_len, c->num_sms, out);
+    return ATTN_OK;
+}
+
+int attn_plan_decode(const attn_ctx* c, int n_new, int* out) {
+    if (c == nullptr || out == nullptr || n_new < 1 || n_new > kMaxDraftTokens) return ATTN_EINVAL;
+    out[0] = decode_splits(c, n_new);
+    out[1] = attn::decode_tc_mode(c->shape, c->num_sms, out[0], n_new);
+    return ATTN_OK;
+}
+
+int attn_plan_w4bf16(int gemm, int M, int N, int K, int rms, int* out) {
+    if (out == nullptr || M < 1 || N < 1 || K < 128 || K % 128 != 0) return ATTN_EINVAL;
+    const cudaError_t e = gemm ? attn::w4_gemm_plan(M, N, K, out) : attn::w4_gemv_plan(M, N, K, rms != 0, out);
+    return e == cudaSuccess ? ATTN_OK : cuda_fail(e, "w4bf16 plan");
 }
 
 const char* attn_strerror(int code) {

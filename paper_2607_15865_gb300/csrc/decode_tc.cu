@@ -1203,6 +1203,16 @@ bool decode_tc_clusters_fit(int nsplit, long long items, int per_sm) {
 }
 }  // namespace
 
+// How a launch of nsplit splits per item merges: more CTAs than the device holds at once run as
+// several waves; one wave's splits of an item are one cluster (their merge) when a cluster per item
+// fits at once, else they merge through global memory.
+int decode_tc_mode(const Shape& s, int num_sms, int nsplit, int ntok) {
+    const int per_sm = ctas_per_sm(s.head_dim, ntok), ncg = decode_tc_column_groups(s.n_q_heads / s.n_kv_heads, ntok);
+    const long long items = static_cast<long long>(s.n_kv_heads) * s.batch * ncg;
+    if (nsplit > 1 && items * nsplit > static_cast<long long>(num_sms) * per_sm) return kModeWaves;
+    return decode_tc_clusters_fit(nsplit, items, per_sm) ? kModeCluster : kModeGlobal;
+}
+
 // Split counts; slots are the CTAs that the device holds at once (SMs, at head_dim 64 with one new
 // token twice as many).  With few (sequence, kv head, column group) items (up to 30% of the
 // slots), one wave of CTAs, min(16, floor(slots / items)) splits per item (32 for up to 4 items),
@@ -1307,13 +1317,7 @@ cudaError_t launch_decode_tc(const Shape& s, const DecodeMaps& maps, const uint1
         attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
         ++n_attr;
     }
-    const bool w = s0 < nsplit;
-    // one wave: the splits of an item are one cluster (their merge) when a cluster per item
-    // fits on the device at once, else they merge through global memory
-    const int mode = w ? kModeWaves
-                       : (decode_tc_clusters_fit(nsplit, static_cast<long long>(s.n_kv_heads) * s.batch * ncg, per_sm)
-                              ? kModeCluster
-                              : kModeGlobal);
+    const int mode = decode_tc_mode(s, num_sms, nsplit, ntok);
     if (mode == kModeCluster) {
         attr[n_attr].id = cudaLaunchAttributeClusterDimension;
         attr[n_attr].val.clusterDim.x = static_cast<unsigned>(nsplit);

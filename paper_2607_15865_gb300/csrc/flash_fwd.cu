@@ -848,9 +848,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             __syncwarp();
             cluster_sync();
             if (ok && rows_on) {
-                // (a piece without keys of this row has l = 0; its O is undefined and left out)
+                // (a piece without keys of this row has l = 0; its O is undefined and left out.  A NaN l,
+                // of a NaN key or an infinite score, takes part and makes the row NaN; an O of weight 0
+                // may hold infinities and is left out, as the merge kernel does)
                 const float2 pml = *peer_ml;
-                const bool mine = tile_on && cl_l > 0.f, theirs = pml.y > 0.f;
+                const bool mine = tile_on && cl_l != 0.f, theirs = pml.y != 0.f;
                 const float mm = fmaxf(mine ? cl_m : -INFINITY, theirs ? pml.x : -INFINITY);
                 const float wa = mine ? fast_exp2(cl_m - mm) : 0.f, wb = theirs ? fast_exp2(pml.x - mm) : 0.f;
                 const float inv = 1.f / ((mine ? cl_l * wa : 0.f) + (theirs ? pml.y * wb : 0.f));
@@ -864,8 +866,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     float v[32];
 #pragma unroll
                     for (int e = 0; e < 32; ++e) {
-                        v[e] = mine ? wa * __uint_as_float(own[e]) : 0.f;
-                        if (theirs) v[e] = fmaf(wb, peer_o[(c + e) * 2 * BM], v[e]);
+                        v[e] = wa != 0.f ? wa * __uint_as_float(own[e]) : 0.f;
+                        if (wb != 0.f) v[e] = fmaf(wb, peer_o[(c + e) * 2 * BM], v[e]);
                     }
                     if (row < un.it.rows(t))
 #pragma unroll
@@ -1175,6 +1177,14 @@ cudaError_t configure_flash_fwd() {
     e = cudaOccupancyMaxActiveClusters(&g_pairs_fit[dev], flash_fwd_kernel<128, true, false>, &cfg);
     if (e != cudaSuccess) return e;
     return cudaSuccess;
+}
+
+void flash_plan(const Shape& s, int hist, int chunk, int num_sms, int out[4]) {
+    const HostSchedule hs = make_schedule(s, hist, chunk, num_sms);
+    out[0] = hs.heads;
+    out[1] = hs.nsplit;
+    out[2] = hs.cluster ? 1 : 0;
+    out[3] = hs.head;
 }
 
 cudaError_t launch_flash_fwd(const Shape& s, const FlashMaps& maps, int hist, int chunk, int s_stride,

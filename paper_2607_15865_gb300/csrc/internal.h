@@ -171,4 +171,15 @@ cudaError_t launch_w4_gemm(const uint8_t* tiles, const uint16_t* x, int T, int N
 cudaError_t launch_rmsnorm_rows(const uint16_t* x, const uint16_t* gamma, float eps, int T, int K, uint16_t* xn,
                                 cudaStream_t st);
 
+// How a call would be cut on the current device (host only; what the launchers decide from):
+//   flash_plan     query heads per tile row group, pieces per item of the tail, 1 where two pieces
+//                  are a cluster, whole items
+//   w4_gemv_plan   rows of the first launch, CTAs per cluster (1: the plain kernel), rounds of units
+//                  and warps per unit of a cluster
+//   w4_gemm_plan   tokens per tile, pairs that share a tile's K, tiles, clusters of the grid
+void flash_plan(const Shape& s, int hist, int chunk, int num_sms, int out[4]);
+int decode_tc_mode(const Shape& s, int num_sms, int nsplit, int ntok);  // 0 global merge, 1 cluster, 2 several waves
+cudaError_t w4_gemv_plan(int M, int N, int K, bool rms, int out[4]);
+cudaError_t w4_gemm_plan(int T, int N, int K, int out[4]);
+
 }  // namespace attn

@@ -683,6 +683,32 @@ cudaError_t configure(int dev) {
     return e;
 }
 
+// The current device, configured, and the plan of a product there.
+cudaError_t device_plan(int T, int N, int K, int* dev_out, Plan* plan) {
+    cudaError_t e = cudaGetDevice(dev_out);
+    const int dev = *dev_out;
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    {
+        std::lock_guard<std::mutex> lock(g_mutex);
+        if (g_encode == nullptr) {
+            cudaDriverEntryPointQueryResult qres;
+            void* fn = nullptr;
+            e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &qres);
+            if (e != cudaSuccess) return e;
+            if (qres != cudaDriverEntryPointSuccess || fn == nullptr) return cudaErrorNotSupported;
+            g_encode = reinterpret_cast<PFN_encodeTiled>(fn);
+        }
+        if (!g_configured[dev]) {
+            e = configure(dev);
+            if (e != cudaSuccess) return e;
+            g_configured[dev] = true;
+        }
+    }
+    *plan = find_plan(dev, T, N, K, g_clusters[dev]);
+    return plan->units < 1 ? cudaErrorInvalidValue : cudaSuccess;
+}
+
 }  // namespace
 
 cudaError_t launch_rmsnorm_rows(const uint16_t* x, const uint16_t* gamma, float eps, int T, int K, uint16_t* xn,
@@ -702,27 +728,9 @@ cudaError_t launch_rmsnorm_rows(const uint16_t* x, const uint16_t* gamma, float 
 cudaError_t launch_w4_gemm(const uint8_t* tiles, const uint16_t* x, int T, int N, int K, uint16_t* y, int* err,
                            cudaStream_t st, const W4GemmEpi* epi_in) {
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    Plan plan;
+    const cudaError_t e = device_plan(T, N, K, &dev, &plan);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    {
-        std::lock_guard<std::mutex> lock(g_mutex);
-        if (g_encode == nullptr) {
-            cudaDriverEntryPointQueryResult qres;
-            void* fn = nullptr;
-            e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &qres);
-            if (e != cudaSuccess) return e;
-            if (qres != cudaDriverEntryPointSuccess || fn == nullptr) return cudaErrorNotSupported;
-            g_encode = reinterpret_cast<PFN_encodeTiled>(fn);
-        }
-        if (!g_configured[dev]) {
-            e = configure(dev);
-            if (e != cudaSuccess) return e;
-            g_configured[dev] = true;
-        }
-    }
-    const Plan plan = find_plan(dev, T, N, K, g_clusters[dev]);
-    if (plan.units < 1) return cudaErrorInvalidValue;
     CUtensorMap map, map_wc, map_ws;
     {
         const cuuint64_t dims[2] = {static_cast<cuuint64_t>(K), static_cast<cuuint64_t>(T)};
@@ -778,6 +786,18 @@ cudaError_t launch_w4_gemm(const uint8_t* tiles, const uint16_t* x, int T, int N
     cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, plan.split > 1 ? w4_gemm_kernel<true> : w4_gemm_kernel<false>, map, map_wc, map_ws,
                               plan.nt, plan.split, plan.n_tt, plan.units, T, N, K, y, err, epi);
+}
+
+cudaError_t w4_gemm_plan(int T, int N, int K, int out[4]) {
+    int dev = 0;
+    Plan plan;
+    const cudaError_t e = device_plan(T, N, K, &dev, &plan);
+    if (e != cudaSuccess) return e;
+    out[0] = plan.nt;
+    out[1] = plan.split;
+    out[2] = plan.units;
+    out[3] = plan.split > 1 ? plan.units : std::min(plan.units, g_clusters[dev][1]);
+    return cudaSuccess;
 }
 
 }  // namespace attn

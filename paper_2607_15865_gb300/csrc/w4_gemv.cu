@@ -757,27 +757,34 @@ cudaError_t launch_cluster_t(const ClusterPlan& p, const uint8_t* tiles, const u
                               early_weights ? 1 : 0, fz);
 }
 
-// M <= 8 rows in one launch: through a cluster plan where there is one; otherwise the plain
-// kernel, which takes at most w4_gemv_max_rows(K) rows.
+// M <= 8 rows in one launch: through a cluster plan where there is one (C > 1); otherwise the plain
+// kernel (C = 1), which takes at most w4_gemv_max_rows(K) rows; *fits: one of them serves all M.
 template <int MT>
-cudaError_t launch_rows(const uint8_t* tiles, const uint16_t* x, int M, int N, int K, uint16_t* y, int* err,
-                        bool early_weights, const W4Fused& fz, cudaStream_t st, bool* done) {
-    *done = true;
-    if (fz.gamma == nullptr) {
+cudaError_t plan_rows(int M, int N, int K, bool rms, ClusterPlan* p, bool* fits) {
+    *p = {1, 0, 0, 0};
+    if (!rms) {
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
-        ClusterPlan p = {};
-        e = cluster_plan<MT>(dev, M, N, K, &p);
+        e = cluster_plan<MT>(dev, M, N, K, p);
         if (e != cudaSuccess) return e;
-        if (p.C > 1) return launch_cluster_t<MT>(p, tiles, x, M, N, K, y, err, early_weights, fz, st);
     }
-    if (M > w4_gemv_max_rows(K)) {
-        *done = false;
-        return cudaSuccess;
-    }
+    *fits = p->C > 1 || M <= w4_gemv_max_rows(K);
+    return cudaSuccess;
+}
+
+template <int MT>
+cudaError_t launch_rows(const uint8_t* tiles, const uint16_t* x, int M, int N, int K, uint16_t* y, int* err,
+                        bool early_weights, const W4Fused& fz, cudaStream_t st, bool* done) {
+    ClusterPlan p;
+    const cudaError_t e = plan_rows<MT>(M, N, K, fz.gamma != nullptr, &p, done);
+    if (e != cudaSuccess || !*done) return e;
+    if (p.C > 1) return launch_cluster_t<MT>(p, tiles, x, M, N, K, y, err, early_weights, fz, st);
     return launch_t<MT>(tiles, x, M, N, K, y, err, early_weights, fz, st);
 }
+
+// Rows to try after m of them did not fit one launch.
+int fewer_rows(int m) { return m > 4 ? 4 : m > 2 ? 2 : m - 1; }
 
 }  // namespace
 
@@ -792,7 +799,7 @@ int w4_gemv_max_rows(int K) {
 cudaError_t launch_w4_gemv(const uint8_t* tiles, const uint16_t* x, int M, int N, int K, uint16_t* y, int* err,
                            bool early_weights, const W4Fused& fz, cudaStream_t st, int* rows) {
     // up to 8 rows in one launch; where neither kernel holds them, as many as the plain one does
-    for (int m = M < 8 ? M : 8; m > 0; m = m > 4 ? 4 : m > 2 ? 2 : m - 1) {
+    for (int m = M < 8 ? M : 8; m > 0; m = fewer_rows(m)) {
         bool done = false;
         cudaError_t e;
         if (m <= 1) e = launch_rows<1>(tiles, x, m, N, K, y, err, early_weights, fz, st, &done);
@@ -803,6 +810,25 @@ cudaError_t launch_w4_gemv(const uint8_t* tiles, const uint16_t* x, int M, int N
             *rows = m;
             return e;
         }
+    }
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t w4_gemv_plan(int M, int N, int K, bool rms, int out[4]) {
+    for (int m = M < 8 ? M : 8; m > 0; m = fewer_rows(m)) {
+        ClusterPlan p;
+        bool fits = false;
+        const cudaError_t e = m <= 1   ? plan_rows<1>(m, N, K, rms, &p, &fits)
+                              : m <= 2 ? plan_rows<2>(m, N, K, rms, &p, &fits)
+                              : m <= 4 ? plan_rows<4>(m, N, K, rms, &p, &fits)
+                                       : plan_rows<8>(m, N, K, rms, &p, &fits);
+        if (e != cudaSuccess) return e;
+        if (!fits) continue;
+        out[0] = m;
+        out[1] = p.C;
+        out[2] = p.rounds;
+        out[3] = p.KS;
+        return cudaSuccess;
     }
     return cudaErrorInvalidValue;
 }
