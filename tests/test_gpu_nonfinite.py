@@ -8,8 +8,6 @@ Paths: prefill_kv in two-piece clusters (plain tiles, packed heads), through the
 whole; decode merged in a cluster, through global memory and in several waves, with one new token
 and several; both head dims.  Each case asserts its path.
 """
-import dataclasses
-
 import numpy as np
 import pytest
 
@@ -96,3 +94,74 @@ def test_prefill_infinite_value_in_a_piece_of_weight_zero(torch, name, shape, hi
     attn.close()
     want = np.repeat(vc[:, :, hist - 2], shape.group, axis=1)[:, None]  # [B, 1, Hq, D]
     assert (out == want).all()
+
+
+# name, shape, lengths, new tokens, merge mode
+DECODE = [
+    ("cluster_d128", Shape("nfd1", 1, 32, 8, 128, 2048, 1.0e4), [2000], 1, CLUSTER),
+    ("cluster_d64", Shape("nfd2", 1, 32, 8, 64, 2048, 1.0e4), [2000], 1, CLUSTER),
+    ("global_d128", Shape("nfd3", 8, 8, 1, 128, 8320, 1.0e4), [8200] + [500] * 7, 1, GLOBAL),
+    ("global_d64", Shape("nfd4", 1, 16, 2, 64, 9000, 1.0e4), [8500], 1, GLOBAL),
+    ("waves_d128", Shape("nfd5", 20, 16, 8, 128, 4096, 1.0e4), [4000] + [60 * b for b in range(19)], 1, WAVES),
+    ("waves_d64", Shape("nfd6", 24, 16, 8, 64, 4096, 1.0e4), [4000] + [60 * b for b in range(23)], 1, WAVES),
+    ("cluster_d128_three_tokens", Shape("nfd7", 1, 32, 8, 128, 2048, 1.0e4), [2000], 3, CLUSTER),
+    ("cluster_d64_three_tokens", Shape("nfd8", 1, 32, 8, 64, 2048, 1.0e4), [2000], 3, CLUSTER),
+    ("waves_d64_four_tokens", Shape("nfd9", 12, 32, 8, 64, 2100, 1.0e4), [2000] + [80 * b for b in range(11)], 4, WAVES),
+]
+
+
+def run_decode(torch, shape, hist, n, mode, edit=None):
+    """The decode of n tokens after edit(kc, vc, v); and the oracle's without the edit."""
+    from paper_2607_15865_gb300.attention import Attention
+    hist = np.asarray(hist, np.int32)
+    q, k, v = w.tokens(shape, "nfd", n)
+    kc, vc = w.cache(shape, "nfd", int(hist.max()), fill="zero")
+    ref = np.zeros(q.shape, np.uint16)
+    rk, rv = kc.copy(), vc.copy()
+    for i in range(n):
+        ref[:, i:i + 1] = O.decode(shape, q[:, i:i + 1].copy(), k[:, i:i + 1].copy(), v[:, i:i + 1].copy(), hist + i, rk, rv)
+    edit(kc, vc, v)
+    attn = Attention.for_shape(shape)
+    assert plan_util.decode(attn, n)[1] == mode
+    hl = torch.from_numpy(hist).cuda()
+    out = to_host(attn.decode_multi(to_dev(q), to_dev(k), to_dev(v), hl, to_dev(kc), to_dev(vc)))
+    assert attn.device_error() == 0
+    attn.close()
+    return out, ref
+
+
+@pytest.mark.parametrize("slot_from_end", [False, True], ids=["first_split", "last_split"])
+@pytest.mark.parametrize("name,shape,hist,n,mode", DECODE, ids=[c[0] for c in DECODE])
+def test_decode_nan_key_in_the_history(torch, name, shape, hist, n, mode, slot_from_end):
+    g = shape.n_kv_heads - 1
+
+    def edit(kc, vc, v):
+        kc[0, g, hist[0] - 2 if slot_from_end else 3, 5] = NAN
+    out, ref = run_decode(torch, shape, hist, n, mode, edit)
+    sees = np.zeros(out.shape[:3], bool)
+    sees[0, :, g * shape.group:] = True
+    assert is_nan(out[sees]).all(), f"{name}: {is_nan(out[sees]).mean():.3f} of the outputs that see the NaN are NaN"
+    assert_out_close(out[~sees], ref[~sees], f"{name} rest")
+
+
+ZERO = [("cluster_d128", 1, 128, 1, CLUSTER), ("cluster_d64", 1, 64, 1, CLUSTER), ("cluster_d64_two_tokens", 1, 64, 2, CLUSTER),
+        ("global_d128", 8, 128, 1, GLOBAL), ("global_d64_32_splits", 1, 64, 1, GLOBAL)]
+
+
+@pytest.mark.parametrize("name,batch,d,n,mode", ZERO, ids=[c[0] for c in ZERO])
+def test_decode_infinite_value_in_a_split_of_weight_zero(torch, name, batch, d, n, mode):
+    from paper_2607_15865_gb300.attention import Attention
+    long = mode == GLOBAL  # over 64 cache tiles the merge goes through global memory
+    shape = Shape("nfz", batch, 8, 1, d, 9000 if long else 1024, 1.0e4)
+    hist = 700  # six tiles, each of its own split
+    q, k, v = w.tokens(shape, "nfz", n)
+    kc, vc = w.cache(shape, "nfz", hist, fill="zero")
+    one_key_takes_all(shape, q, kc, hist - 2)
+    vc[:, :, 3, 1] = 0x7F80
+    attn = Attention.for_shape(shape)
+    splits, got = plan_util.decode(attn, n)
+    assert got == mode and splits >= 6
+    hl = torch.full((batch,), hist, dtype=torch.int32, device="cuda")
+    out = to_host(attn.decode_multi(to_dev(q), to_dev(k), to_dev(v), hl, to_dev(kc), to_dev(vc)))
+    attn.close()
+    assert (out == np.repeat(vc[:, :, hist - 2], shape.group, axis=1)[:, None]).all()
