@@ -948,8 +948,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(D, MAXTOK)) decode_tc_ke
         // staging has been read.  (T is the same in every CTA of the cluster, so all or none
         // of them take part.)
         // In every merge a split is left out when its l is 0, not when it is not above 0: a NaN l
-        // (a NaN key, an infinite score) makes the output NaN.  An accumulator of weight 0 is left
-        // out, since it may hold infinities.
+        // (a NaN key, an infinite score) makes the output NaN.
         if (item_ok && multi && T > 1) {
             tc_fence_before();
             cluster_sync();
@@ -981,7 +980,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(D, MAXTOK)) decode_tc_ke
                     if (r < nw && lr[r] != 0.f) {
                         const float wgt = fast_exp2(mr[r] - mm);
                         l_tot = fmaf(wgt, lr[r], l_tot);
-                        if (wgt != 0.f) acc = fmaf(wgt, orr[r], acc);
+                        acc = fmaf(wgt, orr[r], acc);
                     }
                 if (col_runs(h)) out[orow[h] * D + d] = to_bf16(acc / l_tot);
             }
@@ -1087,14 +1086,10 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(D, MAXTOK)) decode_tc_ke
                     const float mn = use ? fmaxf(mw[h], ml[h].x) : mw[h];
                     const float a = use ? fast_exp2(mw[h] - mn) : 1.f;  // rescale of what came before
                     const float wgt = use ? fast_exp2(ml[h].x - mn) : 0.f;
-                    auto mix = [&](float sum, float o) {
-                        const float kept = a != 0.f ? sum * a : 0.f, both = fmaf(wgt, o, kept);
-                        return wgt != 0.f ? both : kept;
-                    };
-                    acc[h].x = mix(acc[h].x, o4[h].x);
-                    acc[h].y = mix(acc[h].y, o4[h].y);
-                    acc[h].z = mix(acc[h].z, o4[h].z);
-                    acc[h].w = mix(acc[h].w, o4[h].w);
+                    acc[h].x = use ? fmaf(wgt, o4[h].x, acc[h].x * a) : acc[h].x;
+                    acc[h].y = use ? fmaf(wgt, o4[h].y, acc[h].y * a) : acc[h].y;
+                    acc[h].z = use ? fmaf(wgt, o4[h].z, acc[h].z * a) : acc[h].z;
+                    acc[h].w = use ? fmaf(wgt, o4[h].w, acc[h].w * a) : acc[h].w;
                     lw[h] = use ? fmaf(wgt, ml[h].y, lw[h] * a) : lw[h];
                     mw[h] = mn;
                 }
@@ -1124,21 +1119,6 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(D, MAXTOK)) decode_tc_ke
                         sum.z = fmaf(f, v4.z, sum.z);
                         sum.w = fmaf(f, v4.w, sum.w);
                         l_tot = fmaf(f, m_l.y, l_tot);
-                    }
-                }
-                const float any = (sum.x + sum.y) + (sum.z + sum.w);
-                if (any != any) {  // NaN: again without the warps of weight 0, which may hold infinities
-                    sum = make_float4(0.f, 0.f, 0.f, 0.f);
-                    for (int w = 0; w < kThreads / 32; ++w) {
-                        const float2 m_l = wml[w * NH + h];
-                        const float f = m_l.y != 0.f ? fast_exp2(m_l.x - mm) : 0.f;
-                        if (f != 0.f) {
-                            const float4 v4 = reinterpret_cast<const float4*>(racc + (w * NH + h) * D)[c];
-                            sum.x = fmaf(f, v4.x, sum.x);
-                            sum.y = fmaf(f, v4.y, sum.y);
-                            sum.z = fmaf(f, v4.z, sum.z);
-                            sum.w = fmaf(f, v4.w, sum.w);
-                        }
                     }
                 }
                 const float inv = 1.f / l_tot;

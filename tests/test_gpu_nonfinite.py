@@ -142,26 +142,3 @@ def test_decode_nan_key_in_the_history(torch, name, shape, hist, n, mode, slot_f
     sees[0, :, g * shape.group:] = True
     assert is_nan(out[sees]).all(), f"{name}: {is_nan(out[sees]).mean():.3f} of the outputs that see the NaN are NaN"
     assert_out_close(out[~sees], ref[~sees], f"{name} rest")
-
-
-ZERO = [("cluster_d128", 1, 128, 1, CLUSTER), ("cluster_d64", 1, 64, 1, CLUSTER), ("cluster_d64_two_tokens", 1, 64, 2, CLUSTER),
-        ("global_d128", 8, 128, 1, GLOBAL), ("global_d64_32_splits", 1, 64, 1, GLOBAL)]
-
-
-@pytest.mark.parametrize("name,batch,d,n,mode", ZERO, ids=[c[0] for c in ZERO])
-def test_decode_infinite_value_in_a_split_of_weight_zero(torch, name, batch, d, n, mode):
-    from paper_2607_15865_gb300.attention import Attention
-    long = mode == GLOBAL  # over 64 cache tiles the merge goes through global memory
-    shape = Shape("nfz", batch, 8, 1, d, 9000 if long else 1024, 1.0e4)
-    hist = 700  # six tiles, each of its own split
-    q, k, v = w.tokens(shape, "nfz", n)
-    kc, vc = w.cache(shape, "nfz", hist, fill="zero")
-    one_key_takes_all(shape, q, kc, hist - 2)
-    vc[:, :, 3, 1] = 0x7F80
-    attn = Attention.for_shape(shape)
-    splits, got = plan_util.decode(attn, n)
-    assert got == mode and splits >= 6
-    hl = torch.full((batch,), hist, dtype=torch.int32, device="cuda")
-    out = to_host(attn.decode_multi(to_dev(q), to_dev(k), to_dev(v), hl, to_dev(kc), to_dev(vc)))
-    attn.close()
-    assert (out == np.repeat(vc[:, :, hist - 2], shape.group, axis=1)[:, None]).all()
