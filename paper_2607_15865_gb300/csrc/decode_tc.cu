@@ -894,8 +894,13 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(D, MAXTOK)) decode_tc_ke
                 uint32_t o2[NHP];
                 tmem_ld_cols<NHP>(tmem + lane_base + TM_O + part * NH, o2);
                 tmem_wait_ld();
+                // (an infinite or NaN value made its sum with the first part so; the other parts, which
+                // may be zero or negative, would turn an infinity into NaN)
 #pragma unroll
-                for (int h = 0; h < NHP; ++h) o[h] = __float_as_uint(__uint_as_float(o[h]) + __uint_as_float(o2[h]));
+                for (int h = 0; h < NHP; ++h) {
+                    const float first = __uint_as_float(o[h]);
+                    o[h] = __float_as_uint(fabsf(first) < INFINITY ? first + __uint_as_float(o2[h]) : first);
+                }
             }
             if constexpr (kGuardV) {
                 const int odd = *reinterpret_cast<volatile int*>(lastv + 5);

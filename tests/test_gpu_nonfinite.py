@@ -142,3 +142,26 @@ def test_decode_nan_key_in_the_history(torch, name, shape, hist, n, mode, slot_f
     sees[0, :, g * shape.group:] = True
     assert is_nan(out[sees]).all(), f"{name}: {is_nan(out[sees]).mean():.3f} of the outputs that see the NaN are NaN"
     assert_out_close(out[~sees], ref[~sees], f"{name} rest")
+
+
+@pytest.mark.parametrize("name,shape,hist,n,mode", DECODE, ids=[c[0] for c in DECODE])
+def test_decode_infinite_values(torch, name, shape, hist, n, mode):
+    """Infinite values of a cached token, and at head_dim 64 of the first new token: that sign in their
+    dimensions, NaN where both signs meet, the other dimensions unchanged."""
+    g, h, d64 = shape.n_kv_heads - 1, hist[0], shape.head_dim == 64
+
+    def edit(kc, vc, v):
+        vc[0, g, h // 2, 1] = vc[0, g, h - 1, 3] = vc[0, g, 5, 7] = 0x7F80  # +inf
+        vc[0, g, h - 1, 7] = 0xFF80  # -inf
+        if d64:
+            v[0, 0, g, 9] = 0xFF80
+            v[0, 0, g, 3] = 0x7F80
+    out, ref = run_decode(torch, shape, hist, n, mode, edit)
+    hot = out[0, :, g * shape.group:]
+    assert (hot[..., [1, 3]] == 0x7F80).all(), hot[0, 0, :10]
+    assert is_nan(hot[..., 7]).all()
+    if d64:
+        assert (hot[..., 9] == 0xFF80).all()
+    plain = np.ones(out.shape, bool)
+    plain[0, :, g * shape.group:, [1, 3, 7, 9]] = False
+    assert_out_close(out[plain], ref[plain], f"{name} other dimensions")
