@@ -13,6 +13,7 @@ import pytest
 
 from oracle import w4_oracle as W
 from synthetic import gen
+from tests import plan_util
 
 pytestmark = pytest.mark.gpu
 
@@ -87,15 +88,21 @@ def test_w4_gemm_rejects_bad_arguments(torch):
         assert lib.attn_w4bf16_gemm(*args, None) == _lib.ATTN_EINVAL, args
 
 
-# Edges of the plans: 32- and 256-token tiles, an odd number of 128-feature halves, K split over
-# 2, 3 and 4 pairs of a cluster with uneven slices, groups fewer than splits, several rounds.
-PLANS = [("t33_k512", 33, 256, 512), ("t32_k1664_13_groups", 32, 1024, 1664), ("t250_n640", 250, 640, 1024),
-         ("t257_n2048", 257, 2048, 384), ("t64_n6144", 64, 6144, 1024), ("t2_n22016_two_rounds", 2, 22016, 256),
-         ("t1030_n4992", 1030, 4992, 256)]
+# Edges of the plans: 32- to 256-token tiles, an odd number of 128-feature halves, K split over
+# 2, 3 and 4 pairs of a cluster with uneven slices of K (13 groups) and of the tokens (a third pair
+# without any), groups fewer than splits, several rounds.  Each asserts tokens per tile and split.
+PLANS = [("t33_k512", 33, 256, 512, 32, 4), ("t32_k1664_13_groups", 32, 1024, 1664, 32, 4),
+         ("t20_k384_third_pair_without_tokens", 20, 128, 384, 32, 3), ("t100_n2560_k1664_13_groups", 100, 2560, 1664, 64, 3),
+         ("t33_n2048_k512", 33, 2048, 512, 32, 2), ("t250_n640", 250, 640, 1024, 32, 2),
+         ("t200_n1536_k1664_13_groups", 200, 1536, 1664, 64, 2), ("t128_one_group", 128, 128, 128, 32, 1),
+         ("t257_n2048", 257, 2048, 384, 32, 1), ("t64_n6144", 64, 6144, 1024, 32, 1),
+         ("t2_n22016_two_rounds", 2, 22016, 256, 32, 1), ("t1030_n4992", 1030, 4992, 256, 160, 1),
+         ("t256_n9984", 256, 9984, 128, 256, 1)]
 
 
-@pytest.mark.parametrize("tag,T,N,K", PLANS, ids=[c[0] for c in PLANS])
-def test_w4_gemm_plans_match_oracle(torch, tag, T, N, K):
+@pytest.mark.parametrize("tag,T,N,K,nt,split", PLANS, ids=[c[0] for c in PLANS])
+def test_w4_gemm_plans_match_oracle(torch, tag, T, N, K, nt, split):
+    assert plan_util.gemm(T, N, K)[:2] == (nt, split)
     codes, scales, zeros = mat(tag, N, K)
     x = gen.normal_bf16("w4gemm", f"{tag}_x", (T, K), 1.0)
     check(codes, scales, zeros, x, run(torch, codes, scales, zeros, x))
