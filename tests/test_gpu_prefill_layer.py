@@ -19,6 +19,7 @@ from oracle import w4_oracle as W
 from synthetic import gen
 from synthetic import workloads as wl
 from synthetic.workloads import Shape
+from tests import plan_util
 
 pytestmark = pytest.mark.gpu
 
@@ -59,6 +60,11 @@ CHUNKS = [
     ("b2_g4_d128_pkv", Shape("w4p_a", 2, 8, 2, 128, 1024, 1.0e6), 1024, 77, 150),
     ("b1_g2_d64_prefill", Shape("w4p_b", 1, 4, 2, 64, 512, 1.0e4), 256, 0, 200),
     ("b1_g4_d128_hidden4096", Shape("w4p_c", 1, 32, 8, 128, 2048, 5.0e5), 4096, 1536, 512),
+]
+# Few tokens: both GEMMs split K over a cluster's pairs, with the q / k / v output split and with the residual.
+SPLIT_K = [
+    ("b2_g4_d128_k_split4", Shape("w4p_d", 2, 8, 2, 128, 256, 1.0e6), 1024, 50, 17, 4),
+    ("b1_g2_d128_k_split2", Shape("w4p_e", 1, 32, 16, 128, 256, 1.0e6), 1024, 0, 20, 2),
 ]
 
 
@@ -105,6 +111,13 @@ def test_prefill_layer_matches_oracle(torch, tag, shape, hidden, hist, S):
     check_chunk(shape, hist, S, host_bits(h), host_bits(gk).reshape(kc.shape), host_bits(gv).reshape(vc.shape),
                 href, kr, vr, x)
     attn.close()
+
+
+@pytest.mark.parametrize("tag,shape,hidden,hist,S,split", SPLIT_K, ids=[c[0] for c in SPLIT_K])
+def test_prefill_layer_with_k_split(torch, tag, shape, hidden, hist, S, split):
+    T, qd, kd = shape.batch * S, shape.n_q_heads * shape.head_dim, shape.n_kv_heads * shape.head_dim
+    assert plan_util.gemm(T, qd + 2 * kd, hidden)[1] == split and plan_util.gemm(T, hidden, qd)[1] > 1
+    test_prefill_layer_matches_oracle(torch, tag, shape, hidden, hist, S)
 
 
 def test_prefill_layer_in_place_from_a_cuda_graph(torch):
