@@ -472,7 +472,7 @@ def run_ours(args):
             if name == "decode":
                 gbs = DECODE_BYTES / t_s / 1e9
                 stages[name] = {"ms": stage_ms[name], "GB/s": gbs, "frac_hbm": gbs / hbm,
-                                "kernel_ms": {k: kern[k][0] / K for k in ("decode_split", "decode_combine")}}
+                                "kernel_ms": {"decode_split": kern["decode_split"][0] / K}}
             else:
                 tf = FLOPS[name] / t_s / 1e12
                 # the flash kernel alone (called by itself): against the burst peak, as a
@@ -495,7 +495,7 @@ def run_ours(args):
                          "frac_of_burst_peak": flash_tflops / tc_peak, "burst_peak": tc_peak,
                          "launch_ms_avg": flash_ms / max(flash_n, 1)},
             "stages": stages,
-            "kernels_ms_per_step": {k: v[0] / K for k, v in kern.items()},
+            "kernels_ms_per_step": {k: v[0] / K for k, v in kern.items() if v[1]},
             "cpu_baseline": cpu,
             "e2e": {"value": job_tflops(world, e2e_ms), "unit": "TFLOP/s",
                     "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms,

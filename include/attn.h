@@ -49,8 +49,8 @@
  *
  * Errors.  Every int-returning call returns ATTN_OK (0) or a negative code and
  * writes nothing when it rejects its arguments; that includes shapes whose launch
- * would exceed a grid limit (a decode with batch x column groups, or head_dim 64
- * kv heads x head passes, above 65535; a prefill chunk whose pairs of 128-row
+ * would exceed a grid limit (a head_dim 128 decode of several tokens with batch x
+ * column groups above 65535; a prefill chunk whose pairs of 128-row
  * query tiles x n_q_heads x batch exceed 2^30).  Launch failures return
  * ATTN_ECUDA (attn_last_cuda_error_string() gives the runtime's text).  The
  * decode lengths live on the device, so a decode whose hist_len[b] is outside

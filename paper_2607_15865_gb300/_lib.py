@@ -24,6 +24,7 @@ EXPORTED = ("attn_create", "attn_destroy", "attn_prefill", "attn_prefill_kv", "a
             "attn_w4bf16_rows_per_launch", "attn_w4bf16_gemv_fused", "attn_decode_layer",
             "attn_w4bf16_gemm", "attn_prefill_layer", "attn_prefill_layer_workspace")
 NOALLOC_SCRATCH_FLOATS = 1 << 20
+# attn_timing_read's slots; no kernel runs as decode_combine (the decode merges itself): it reads 0
 KERNELS = ("rope_append", "flash_fwd", "decode_split", "decode_combine")
 
 

@@ -36,7 +36,7 @@ struct attn_ctx {
     float* d_sin_t;
     float* d_part_o;
     float* d_part_ml;
-    int* d_counters;    // decode counters, [2][B * Hkv] (merge count, tile claims), zero between launches
+    int* d_counters;    // decode counters (decode_tc_counter_ints), zero between launches
     uint16_t* d_lq;     // decode layer: q, k, v of the fused QKV projection and the attention
     uint16_t* d_lk;     // output, bf16 [B][Hq*D], [B][Hkv*D], [B][Hkv*D], [B][Hq*D]
     uint16_t* d_lv;

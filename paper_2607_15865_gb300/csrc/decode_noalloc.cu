@@ -8,8 +8,9 @@
 // create an attn_ctx (attn_create allocates the tables and the split-KV partials).
 //
 // This entry point runs the same kernel as attn_decode (K3 with the new token's append
-// and the merge of the splits) but needs no context: the caller passes every input and output, including the RoPE tables and the error word,
-// and the split-KV partials and merge counters live in the file-scope arrays below,
+// and the merge of the splits) but needs no context: the caller passes every input and
+// output, including the RoPE tables and the error word, and the split-KV partials and merge
+// counters live in the file-scope arrays below,
 // which the library holds on every device that loads it until the process exits.
 // Nothing is allocated or freed.
 //

@@ -63,6 +63,7 @@ cudaError_t launch_rope_append(const Shape& s, const uint16_t* k, const uint16_t
 
 // K2: causal flash attention of `chunk` new queries at positions hist.. over cache
 // slots [0, hist+chunk) (prefill: hist=0).  RoPE of q is applied in the kernel.
+
 // Query heads that share a query tile's 128 rows: all of a kv head's, or 1.
 int flash_pack_heads(const Shape& s, int hist, int chunk, int num_sms);
 struct FlashMaps {

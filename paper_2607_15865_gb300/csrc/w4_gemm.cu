@@ -20,7 +20,8 @@
 // cycles on both SMs, and the one issuing thread makes one wait, eight MMAs and one commit
 // per 128-input group.  (One CTA per 256 x 128 tile, its MMAs 128 x 128 x 16, twice the
 // decoding and four barrier operations per sixteen MMAs, took 183 us on 4096 x 6144 x 4096;
-// this takes 115 us, 22016 features 392 instead of 588.)  Few tokens leave most SMs idle, so K
+// this takes 115 us alone and 126 to 128 among
+// other calls, under the power cap; 22016 features 392 instead of 588 alone.)  Few tokens leave most SMs idle, so K
 // is then split over the pairs of a cluster, which add their f32 partials through distributed
 // shared memory (32 tokens x 4096 x 4096: 9 us, 24.6 before).
 //

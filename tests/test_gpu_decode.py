@@ -1,4 +1,4 @@
-"""GPU parity of decode (K1 + K3 + K4 through the C ABI) against the CPU oracle.
+"""GPU parity of decode (K3 through the C ABI) against the CPU oracle.
 
 Covers the decode sweep (batch 1/4/16 x valid lengths 1024/4096/8191 over a
 static maximum of 8192), mixed per-sequence lengths including 0 and max_len-1,

@@ -42,11 +42,10 @@ def rope_tables(shape):
     return np.cos(ang).astype(np.float32), np.sin(ang).astype(np.float32)
 
 
-# head_dim 128 runs the tensor-core decode (its merge fused in, counters in the static
-# array); head_dim 64 runs the CUDA-core split kernel and the merge kernel, both reading
-# and writing the static partials.  The scratch cap never binds below attn_decode's own
-# split count for these kernels' split rules (it would need more than 50 query heads per
-# kv head), so both calls run attn_decode's split count.
+# Both head dims run the tensor-core decode, its merge fused in, with partials and counters in
+# the static arrays.  The scratch cap never binds below attn_decode's own split count for these
+# shapes (at most 2^20 / (batch * Hq * (head_dim + 2)) splits: 63 and 1323), so both calls run
+# attn_decode's split count.
 CASES = [
     ("d128_b4", Shape("noalloc128", 4, 32, 8, 128, 8192, 5.0e5), 8191,
      ([1024, 4096, 8191, 17], [5, 0, 8000, 3000])),
