@@ -107,7 +107,7 @@ struct Layout {
     static constexpr int OFF_LAST = OFF_ABORT + 4;
     // int [8] at OFF_LAST: merge flag, merged slots, this CTA's partial slot, tiles it
     // claimed, a helper split's first ticket, new tokens whose v holds infinities or NaN, a
-    // helper split's sequence
+    // helper split's sequence, copies issued (several waves)
     static constexpr int OFF_CROW = OFF_LAST + 32;  // size_t [16]: partial row (slot 0) of column c
     static constexpr int OFF_OROW = OFF_CROW + NH * 8;  // size_t [16]: q / out row of column c
     static constexpr int BYTES = OFF_OROW + NH * 8;
@@ -487,6 +487,14 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(D, MAXTOK)) decode_tc_ke
     const size_t* crow = reinterpret_cast<const size_t*>(gb + L::OFF_CROW);
     const size_t* orow = reinterpret_cast<const size_t*>(gb + L::OFF_OROW);
     int* meta = reinterpret_cast<int*>(gb + L::OFF_META);  // tile index of local tile j at [j % 8]; -1 ends
+    // Wait for the last use of every ring slot by nk K and nv V copies.  (A loop that ended well has
+    // put its end mark in K slot nk mod KST, whose copy had landed before: its phase is past.)
+    auto drain = [&](int nk, int nv, bool ended_well) {
+        for (int t = max(0, nk - KST + (ended_well ? 1 : 0)); t < nk; ++t)
+            mbar_wait(bar(B_KFULL0 + t % KST), static_cast<uint32_t>(t / KST) & 1u, nullptr);
+        for (int t = max(0, nv - VST); t < nv; ++t)
+            mbar_wait(bar(B_VFULL0 + t % VST), static_cast<uint32_t>(t / VST) & 1u, nullptr);
+    };
 
     if (!item_ok) {
         // sequence skipped: nothing written (the speculative copies land before the CTA ends)
@@ -585,12 +593,14 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(D, MAXTOK)) decode_tc_ke
                 *visit_ctr = 0;
             }
             // Every copy issued must land before the CTA may exit, also when this loop ended well
-            // and another warp's wait ran out.  (A loop that ended well has put its end mark in K
-            // slot issued_k mod KST, whose copy had landed before: its phase is past.)
-            for (int t = max(0, issued_k - KST + (ok ? 1 : 0)); t < issued_k; ++t)
-                mbar_wait(bar(B_KFULL0 + t % KST), static_cast<uint32_t>(t / KST) & 1u, nullptr);
-            for (int t = max(0, issued_v - VST); t < issued_v; ++t)
-                mbar_wait(bar(B_VFULL0 + t % VST), static_cast<uint32_t>(t / VST) & 1u, nullptr);
+            // and another warp's wait ran out.  In several waves the CTA's last barrier comes first
+            // and only a CTA that gave up waits (5 tokens of 3 sequences at head_dim 64: 26.4 us a
+            // call, 26.7 with the wait here); a cluster or one wave waits here, where nothing is
+            // slower for it (4 tokens over 8188 14.45 us, 14.66 with the wait at the end).
+            if constexpr (WAVES)
+                lastv[7] = (issued_k << 1 | (ok ? 1 : 0)) | issued_v << 16;
+            else
+                drain(issued_k, issued_v, ok);
         }
         if (early) griddep_wait();
     } else if (warp == kWarpMma) {
@@ -1139,6 +1149,8 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm(D, MAXTOK)) decode_tc_ke
     if (warp == kWarpMma) {
         tc_fence_after();
         tmem_dealloc(tmem, L::TMEM_COLS);
+    } else if (WAVES && item_ok && tid == 32 * kWarpTma && *abort_flag) {
+        drain(lastv[7] >> 1 & 0x7FFF, lastv[7] >> 16, lastv[7] & 1);
     }
 }
 
